@@ -229,7 +229,7 @@ int vecchia_covariance(int kernel, const double* d_dev, int64_t count, const dou
 int vecchia_pivot_reciprocal(const double* d_dev, int64_t count, double* out_dev, void* stream);
 
 /*
- * vecchia_mul_by_positive — the product the full-warp likelihood kernels use to scale an
+ * vecchia_mul_by_positive — the product the 4-lane forward kernel uses to scale an
  * elimination column by its pivot reciprocal (Algorithm 1's factorisation step, written
  * as L D L^T), exposed so its exactness can be checked.  It uses no FP64 instruction:
  * the 106-bit mantissa product is formed from 32-bit integer limbs and rounded to
@@ -288,7 +288,7 @@ int vecchia_loglik_batched(const vecchia_plan_t* plans, const double* const* y_d
  * that owns every device byte, or a runtime that must never trigger an allocation
  * while serving).  It has no counterpart in the paper.  It calls no cudaMalloc,
  * cudaFree or other allocating routine; its scratch (partial sums for launches of at
- * most 4096 warps, an error slot and one covariance table, about 190 KB) is a
+ * most 4096 warps, an error slot and one covariance table, about 270 KB) is a
  * file-scope __device__ array that every GPU loading the library keeps until the
  * process exits.  The launch is capped at 4096 warps; the kernel strides over the
  * locations, so no n is too large for the scratch.
@@ -328,8 +328,8 @@ int vecchia_loglik_noalloc(const double* xy_dev, const double* y_dev, const int3
  * timed launches after one warm-up; the fastest wins) and recorded, process-wide, for
  * every later call with the same block size and kind (want_grad) on this device,
  * including the batched call's layouts created afterwards.  Without tuning, blocks of
- * up to 16 rows use 4 lanes, up to 32 rows 8, up to 48 rows 16 (forward) or 32
- * (gradient), larger ones a full warp; a call over fewer locations than would give
+ * up to 16 rows use 4 lanes, up to 29 rows 8 and up to 37 rows 16 (gradient: up to 26 and
+ * 35 rows), larger ones a full warp; a call over fewer locations than would give
  * one group of them per SM sub-partition widens those defaults (up to 16 lanes), and
  * a call with fewer groups than the shape's resident warps spreads them over every SM
  * with fewer warps per CTA.  Results are deterministic for a given plan, range and

@@ -68,7 +68,7 @@ struct BatchArgs {
 
 // One item with G lanes per location: the 32/G groups of the warp take the tile's
 // locations in turn.
-template <bool GRAD, int G>
+template <bool GRAD, int G, bool FIXED>
 __device__ __forceinline__ void run_item(const FieldDesc& fd, int64_t tile, const unsigned char* smem,
                                          const BatchArgs& a, double* base, const double* tab,
                                          const MaternConst& mc, const ThetaConst& tc, double* out, int lane) {
@@ -93,7 +93,7 @@ __device__ __forceinline__ void run_item(const FieldDesc& fd, int64_t tile, cons
   for (int64_t b = i0; b < i1; b += NL) {
     const int64_t i = b + grp;
     const bool active = i < i1;
-    process_location<GRAD, G, false>(active ? i : b, active, F, S, sched, pairs, area, tab, mc, tc, acc, false, nullptr,
+    process_location<GRAD, G, false, FIXED>(active ? i : b, active, F, S, sched, pairs, area, tab, mc, tc, acc, false, nullptr,
                               a.errloc, sub);
   }
   write_partial<G>(acc, out, lane);
@@ -145,13 +145,14 @@ __global__ void __launch_bounds__(384) vecchia_batched_kernel(const BatchArgs a)
       }
       continue;
     }
-    const MaternConst mc = load_matern_const(tab);
+    const MaternConst mc = matern_const_at(fix_const(tab));
     ThetaConst tc;
     tc.set(s2, beta, t2, kFamilyMatern, nu);
-    if (fd.lanes == 4) run_item<GRAD, 4>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
-    else if (fd.lanes == 8) run_item<GRAD, 8>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
-    else if (fd.lanes == 16) run_item<GRAD, 16>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
-    else run_item<GRAD, 32>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
+    if (fd.lanes == 4) run_item<GRAD, 4, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
+    else if (fd.lanes == 8) run_item<GRAD, 8, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
+    else if (fd.lanes == 16) run_item<GRAD, 16, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
+    else if (fixed_point_block(fd.m + 1, GRAD, 32)) run_item<GRAD, 32, true>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
+    else run_item<GRAD, 32, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
     __syncwarp();
   }
 }
@@ -395,7 +396,7 @@ extern "C" int vecchia_batched_prepare(const double* nus, int32_t nnu, void* str
         cudaMalloc(&p->d_tabs, sizeof(double*) * kMaxNu) != cudaSuccess)
       return VECCHIA_ENOMEM;
     for (int k = 0; k < kMaxNu; ++k)
-      if (cudaMalloc(&p->tabs[k], kTableBytes) != cudaSuccess) return VECCHIA_ENOMEM;
+      if (cudaMalloc(&p->tabs[k], kFixTableBytes) != cudaSuccess) return VECCHIA_ENOMEM;
   }
   VECCHIA_CUDA_TRY(cudaStreamSynchronize(s));
   for (int k = 0; k < nnu; ++k) {

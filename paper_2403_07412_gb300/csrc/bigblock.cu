@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
   float2* GVf = reinterpret_cast<float2*>(GV);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int NTH = blockDim.x;
-  const MaternConst mc = load_matern_const(a.tab);
+  const MaternConst mc = matern_const_at(fix_const(a.tab));
   ThetaConst tc;
   tc.set(a.sigma2, a.beta, a.tau2, a.family, a.nu);
   const double2* __restrict__ xy2 = reinterpret_cast<const double2*>(a.xy);
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       float u0h, u0l, u1h, u1l;
       pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
       pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-      const double val0 = rho_df(u0h, u0l, a.tab, mc), val1 = rho_df(u1h, u1l, a.tab, mc);
+      const double val0 = rho_fixed(u0h, u0l, a.tab, mc), val1 = rho_fixed(u1h, u1l, a.tab, mc);
       A[tri_off(K, c0) + r0 - c0] = ok0 ? val0 : 0.0;
       if (has1) A[tri_off(K, c1) + r1 - c1] = ok1 ? val1 : 0.0;
     }
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
         const int c0 = K - 2 - v0, r0 = c0 + 1 + (q0 - v0 * (v0 + 1) / 2);
         float u0h, u0l, h0h, h0l;
         pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
-        h_df(u0h, u0l, a.tab, mc, h0h, h0l);
+        h_fixed(u0h, u0l, a.tab, mc, h0h, h0l);
         beta_pair_add(WHf[r0], WHf[c0], GVf[r0], GVf[c0], h0h, h0l, pbh, pbl);
       }
     }

@@ -34,11 +34,11 @@
 #pragma once
 
 #include "common.cuh"
+#include "fixtable.cuh"
 #include "matern.cuh"
+#include "mmapanel.cuh"
 
 namespace vecchia {
-
-__host__ __device__ __forceinline__ int tri_off(int K, int c) { return (K - c) * (K - c + 1) / 2; }
 
 __host__ __device__ __forceinline__ int align_up(int x, int a) { return (x + a - 1) / a * a; }
 
@@ -63,6 +63,11 @@ struct SchedSize {
 // than the thirteenth warp gains (m = 60: 99.0 -> 102.3 ms; m = 45: 48.2 -> 50.0 ms), and
 // with 4 lanes the registers, not shared memory, limit the warps.
 __host__ __device__ constexpr bool regather_capable(bool grad, int G) { return grad && G == 8; }
+
+// Whether a full-warp block is eliminated in fixed point (mmapanel.cuh) instead of FP64.
+__host__ __device__ constexpr bool fixed_point_block(int K, bool grad, int G) {
+  return G == 32 && K >= (grad ? kFixedMinGrad : kFixedMinFwd);
+}
 
 // Per-warp shared-memory area for blocks up to size K: the packed triangle A and the
 // block rows' coordinates CX, CY (float pairs; on the sphere a third array CZ follows CY).
@@ -223,32 +228,11 @@ __device__ __forceinline__ double group_sum(double v) {
 // leaves early; inactive groups (active = false) compute a valid location and discard
 // it.  When terms_mode (the same for the whole warp), terms (if not null) receives l_i,
 // or {l_i, dl_i/dsigma2, dl_i/dbeta, dl_i/dtau2} when GRAD.  A block that is not positive definite gives a NaN term and records i in errloc.
-// x as a float pair hi + lo (hi: x's leading 24 bits, lo: the next 24, about 2^-48
-// relative), with integer operations; exponents far from 0 take the FP64 route.
-__device__ __forceinline__ float2 d2f_pair(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7FF) - 1023;
-  if (e < -90 || e > 90) {
-    const float hi = __double2float_rn(x);
-    return make_float2(hi, __double2float_rn(x - (double)hi));
-  }
-  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-  const float hi = __uint_as_float(sign | ((unsigned)(e + 127) << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
-  // remainder: mantissa bits 28..5, v 2^(e-47) = (v 2^-24) 2^(e-23)
-  const float lo = fscale(u24_float((unsigned)(b >> 5) & 0xFFFFFFu), e - 23);
-  return make_float2(hi, __uint_as_float(__float_as_uint(lo) | sign));
-}
-
-// x as a float pair (hi: x's leading 24 bits, lo: the next 24), by integer operations
-// only; |x| below 2^-100 gives (0, 0).  For values of moderate exponent (factor entries).
-__device__ __forceinline__ float2 d2f_trunc(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7FF) - 1023;
-  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-  const float hi = __uint_as_float(sign | ((unsigned)(e + 127) << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
-  const float lo = fscale(u24_float((unsigned)(b >> 5) & 0xFFFFFFu), e - 23);
-  const bool z = e < -100;
-  return make_float2(z ? 0.0f : hi, z ? 0.0f : __uint_as_float(__float_as_uint(lo) | sign));
+// Entry e of the unit factor as a float pair: from FP64, or as panels_to_pairs left it.
+template <bool PAIRS>
+__device__ __forceinline__ float2 factor_pair(const double* __restrict__ A, int e) {
+  if constexpr (PAIRS) return reinterpret_cast<const float2*>(A)[e];
+  else return d2f_trunc(A[e]);
 }
 
 // (h, l) -= (a.x + a.y)(b.x + b.y) in double-float arithmetic (about 2^-46 relative).
@@ -345,7 +329,10 @@ __device__ __forceinline__ void sphere_u_df(float ch, float cl, const FieldView&
   two_sum(wh, bh, s, e);
   e = __fadd_rn(e, __fadd_rn(wl, bl));
   const float vh = __fadd_rn(s, e), vl = __fsub_rn(e, __fsub_rn(vh, s));
-  df_mul(F.k2.x, F.k2.y, vh, vl, uh, ul);
+  float ph, pl;
+  df_mul(F.k2.x, F.k2.y, vh, vl, ph, pl);
+  uh = __fadd_rn(ph, pl);  // normalised: the table's argument wants |ul| <= ulp(uh) / 2
+  ul = __fsub_rn(pl, __fsub_rn(uh, ph));
 }
 
 // u of the pair (r, c) of the block, plane or sphere (a compile-time choice, so that the
@@ -399,7 +386,7 @@ __device__ __forceinline__ double beta_pass(const FieldView& F, int NP, const ui
     const int r0 = w0 & 0xFF, c0 = (w0 >> 8) & 0xFF;
     float u0h, u0l, h0h, h0l;
     pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
-    h_df(u0h, u0l, tab, mc, h0h, h0l);
+    h_fixed(u0h, u0l, tab, mc, h0h, h0l);
     beta_pair_add(WHf[r0], WHf[c0], GVf[r0], GVf[c0], h0h, h0l, pbh, pbl);
   }
   return f2d_scaled(pbh, 0) + f2d_scaled(pbl, 0);
@@ -423,7 +410,7 @@ __device__ __forceinline__ void coord_offsets(const FieldView& F, const ThetaCon
 
 // Returns whether the location's term is valid (positive definite block, finite data,
 // indices in range).
-template <bool GRAD, int G, bool SPHERE>
+template <bool GRAD, int G, bool SPHERE, bool FIXED>
 __device__ __forceinline__ bool process_location(int64_t i, bool active, const FieldView& F, const SchedSize& S,
                                                  const uint16_t* __restrict__ sched,
                                                  const uint32_t* __restrict__ pairs, const WarpArea& W,
@@ -455,6 +442,16 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   // the border by the assembly (that order measured 1% faster there)
   const bool regather = regather_capable(GRAD, G) && W.regather;  // warp-uniform
   const bool sep_buffers = GRAD && !regather;
+  // Full-warp blocks: the panels' elimination on the tensor cores (mmapanel.cuh) holds the
+  // data row in units of 2^ky; in the rare case that one of its entries outgrows them, the
+  // block is built and eliminated again with larger units.
+  static_assert(!FIXED || G == 32, "fixed point is for full-warp blocks");
+  constexpr bool kPanels = FIXED;
+  PanelScale ysc;
+  long long corner[2] = {0, 0};
+  bool ok = true;
+  for (int attempt = 0;; ++attempt) {
+  unsigned ytop = 0u;  // largest exponent field of the data
 #pragma unroll
   for (int s = 0; s < NSG; ++s) {
     const int p = sub + G * s;
@@ -469,6 +466,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
         coord_offsets<SPHERE>(F, tc, ps, js, j, xv, yv, zv);
         fv = F.yf[j];
       }
+      if constexpr (kPanels) ytop = max(ytop, exponent_field(fv));
       if (sep_buffers) {
         W.TV1[p] = fv;
       } else {
@@ -483,6 +481,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     CX[m] = make_float2(0.0f, 0.0f);
     CY[m] = make_float2(0.0f, 0.0f);
     if constexpr (SPHERE) CZ[m] = make_float2(0.0f, 0.0f);
+    if constexpr (kPanels) ytop = max(ytop, exponent_field(F.yf[js]));
     if (sep_buffers) {
       W.TV1[m] = F.yf[js];
     } else {
@@ -495,12 +494,20 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     bad_idx = (__ballot_sync(0xffffffffu, bad_idx) & gmask) != 0u;
   }
   __syncwarp();
+  if constexpr (kPanels) ysc.init(ytop, tc.sigma2, tc.gamma1, attempt);
   // ---- assemble: diagonal (and, with separate column buffers, the data border), then
   // the correlation pairs
   for (int c = sub; c < K; c += G) {
     const int o = tri_off(K, c);
-    A[o] = (c >= mi && c < m) ? 1.0 : tc.gamma1;
-    if (sep_buffers) A[o + K - c] = W.TV1[c];
+    const double dg = (c >= mi && c < m) ? 1.0 : tc.gamma1;
+    if constexpr (kPanels) {  // in fixed point (mmapanel.cuh)
+      const double yc = sep_buffers ? W.TV1[c] : A[o + K - c];
+      A[o] = __longlong_as_double(fixed_from_double(dg, 60 - 2 * ysc.f));
+      A[o + K - c] = __longlong_as_double(ysc.nonfinite ? 0LL : fixed_from_double(yc, 60 - ysc.ky));
+    } else {
+      A[o] = dg;
+      if (sep_buffers) A[o + K - c] = W.TV1[c];
+    }
   }
   if (sub == 0) A[0] = 0.0;
   // Two pairs per lane per iteration so one pair's loads overlap the other's FMAs.
@@ -516,25 +523,34 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     float u0h, u0l, u1h, u1l;
     pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
     pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-    const double val0 = rho_df(u0h, u0l, tab, mc), val1 = rho_df(u1h, u1l, tab, mc);
-    A[w0 >> 16] = v0 ? val0 : 0.0;
-    if (has1) A[w1 >> 16] = v1 ? val1 : 0.0;
+    if constexpr (kPanels) {  // units of 2^-60
+      const long long val0 = rho_fixed62(u0h, u0l, tab, mc) >> 2, val1 = rho_fixed62(u1h, u1l, tab, mc) >> 2;
+      A[w0 >> 16] = __longlong_as_double(v0 ? val0 : 0LL);
+      if (has1) A[w1 >> 16] = __longlong_as_double(v1 ? val1 : 0LL);
+    } else {
+      const double val0 = rho_fixed(u0h, u0l, tab, mc), val1 = rho_fixed(u1h, u1l, tab, mc);
+      A[w0 >> 16] = v0 ? val0 : 0.0;
+      if (has1) A[w1 >> 16] = v1 ? val1 : 0.0;
+    }
   }
   __syncwarp();
   // ---- L D L^T over the neighbour columns, two columns per step: column j, then column
   // j+1 updated by column j and scaled, then one pass over the remaining prefix applying
   // both (fma(-L1, T1, fma(-L0, T0, a)): the same roundings, in the same order, as two
   // single-column steps, with half the column transitions and shared-memory passes).
-  bool ok = true;
+  ok = true;
   double* __restrict__ TV1 = W.TV1;  // column j+1's unscaled entries
   // Column scaling by the pivot reciprocal: the integer round-to-nearest-even product
-  // (mul_by_positive, bit-identical to the DMUL) in the full-warp forward kernel, where
-  // it keeps an FP64 instruction off the column step's serial path (n = 1M, m = 60:
-  // 89.5 -> 86.4 ms), and in the 4-lane forward kernel (m = 10: 1.266 -> 1.245 ms); the
-  // DMUL in the gradient kernel, whose double-float adjoint leaves the FP64 queue shorter
-  // (103.4 -> 100.0 ms with the DMUL), and in 8- and 16-lane groups (2.5% faster at
-  // m = 30).
-  constexpr bool kIntScale = (G == 32 || G == 4) && !GRAD;
+  // (mul_by_positive, bit-identical to the DMUL) in the 4-lane forward kernel, where it
+  // keeps an FP64 instruction off the column step's serial path (m = 10, n = 1M: 1.266 ->
+  // 1.245 ms); the DMUL elsewhere (8- and 16-lane groups 2.5% faster with it at m = 30).
+  constexpr bool kIntScale = G == 4 && !GRAD;
+  if constexpr (kPanels) {
+    ok = panels_eliminate<GRAD>(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), ysc, corner, sub);
+    if (!ysc.grown || !ok || ysc.nonfinite || attempt == 7) break;
+    __syncwarp();
+    continue;
+  } else {
   int j = 0;
   for (; j + 2 < K; j += 2) {
     const int oj = tri_off(K, j), o1 = tri_off(K, j + 1);
@@ -655,8 +671,6 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     for (int r = j + 1 + sub; r <= K; r += G) {
       const double tv = A[oj + r - j];
       TV[r] = tv;
-      // integer product in the full-warp forward kernel (no wait behind other warps'
-      // FP64 work on the column step's serial path); DMUL elsewhere (kIntScale)
       if constexpr (kIntScale) {
         A[oj + r - j] = mul_by_positive(tv, inv);
       } else {
@@ -706,8 +720,16 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     }
     __syncwarp();
   }
-  const double st = A[1];  // s_i / sigma2
-  const double rr = A[2];  // y_i - mu_i
+  }
+  break;
+  }
+  double st = A[1];  // s_i / sigma2
+  double rr = A[2];  // y_i - mu_i
+  if constexpr (kPanels) {
+    st = mul_pow2((double)corner[0], 2 * ysc.f - 60);
+    rr = mul_pow2((double)corner[1], ysc.ky - 60);
+    if (ysc.grown || ysc.nonfinite) rr = __longlong_as_double(0x7FF8000000000000LL);  // data not finite (or far out of any scale)
+  }
   // The pivots and s_i depend on the covariance only, the residual on the data: a
   // non-finite residual (with a positive definite block) means a non-finite y in B_i.
   const bool pd = ok && positive_finite(st);
@@ -766,6 +788,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     }
   }
   constexpr int NS = (KCAP - 1 + G - 1) / G;  // slots of the K-1 <= KCAP-1 neighbour entries
+  if constexpr (kPanels) panels_to_pairs(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), ysc, sub);
   // The two unit backward solves run in double-float arithmetic on the FP32 pipe: each
   // step of their serial chain would otherwise wait behind the other warps' FP64 work.
   float2 wf[NS], bf[NS];
@@ -776,8 +799,8 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     bf[t] = make_float2(0.0f, 0.0f);
     if (c < K - 1) {
       const int o = tri_off(K, c);
-      wf[t] = d2f_trunc(A[o + m - c]);
-      bf[t] = d2f_trunc(A[o + K - c]);
+      wf[t] = factor_pair<kPanels>(A, o + m - c);
+      bf[t] = factor_pair<kPanels>(A, o + K - c);
     }
   }
   for (int c = K - 2; c >= 1; --c) {
@@ -795,7 +818,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     for (int t = 0; t < NS; ++t) {
       const int cc = sub + G * t;
       if (cc < c) {
-        const float2 l = d2f_trunc(A[tri_off(K, cc) + c - cc]);
+        const float2 l = factor_pair<kPanels>(A, tri_off(K, cc) + c - cc);
         df_fms(wf[t].x, wf[t].y, l, wc);
         df_fms(bf[t].x, bf[t].y, l, bc);
       }

@@ -25,6 +25,16 @@ constexpr int kIntWords = 5;
 constexpr int kNConst = 8;
 constexpr size_t kTableBytes = (size_t)16 * kIntWords * kNInt + sizeof(double) * kNConst;
 
+// The likelihood kernels' table (fixtable.cuh): 2^kFixSub intervals an octave, degree
+// kFixDeg, kFixWords 16-byte words an interval, then the same constants, then (Matérn) the
+// nodes of the quadrature that builds it.
+constexpr int kFixSub = 5;
+constexpr int kFixDeg = 7;
+constexpr int kFixWords = 5;
+constexpr int kFixInt = (kEHi - kELo) << kFixSub;
+constexpr int kFixNodes = 512;
+constexpr size_t kFixTableBytes = (size_t)16 * kFixWords * kFixInt + sizeof(double) * kNConst + 16 * (size_t)kFixNodes;
+
 // Largest conditioning sets: overall (CTA-per-location kernel) and for the warp kernels.
 constexpr int kMaxM = VECCHIA_MAX_M;
 constexpr int kMaxMWarp = VECCHIA_MAX_M_WARP;
@@ -35,6 +45,16 @@ constexpr int kMaxCtaWarps = 13;
 // keep at most four neighbour slots per lane, so their per-lane register arrays (and the
 // selects that index them) stay short.
 __host__ __device__ constexpr int max_k_for_lanes(int G) { return G == 4 ? 16 : (G == 8 ? 32 : kMaxMWarp + 1); }
+
+// Smallest full-warp blocks (rows) eliminated in fixed point (mmapanel.cuh) instead of FP64.
+// n = 100k, FP64 / fixed point, ms: forward m = 34 2.19 / 2.33, m = 38 2.79 / 2.55, m = 60 8.75 /
+// 5.39; with the gradient m = 42 4.16 / 4.69, m = 46 5.04 / 5.11, m = 50 6.20 / 6.03, m = 60 11.1 /
+// 8.32 (its adjoint reads the factor from digits).
+constexpr int kFixedMinFwd = 38;
+constexpr int kFixedMinGrad = 49;
+
+// First slot of column c of a packed block triangle (block.cuh).
+__host__ __device__ __forceinline__ int tri_off(int K, int c) { return (K - c) * (K - c + 1) / 2; }
 
 // Covariance families (VECCHIA_KERNEL_*): Matérn, Eq. (2); power exponential, Eq. (3).
 constexpr int kFamilyMatern = 0;

@@ -17,8 +17,7 @@
 
 namespace vecchia {
 
-int get_matern_table(double nu, cudaStream_t stream, const double** out);
-int get_cov_table(int family, double nu, cudaStream_t stream, const double** out);
+int get_cov_table(int family, double nu, cudaStream_t stream, const double** out, bool fixed);
 void cov_table_used(const double* tab, cudaStream_t stream);
 
 // A covariance table taken from the cache for one call: when the call's scope ends (after
@@ -31,7 +30,7 @@ struct TablePin {
   TablePin& operator=(const TablePin&) = delete;
   int get(int family, double nu, cudaStream_t s) {
     stream = s;
-    return get_cov_table(family, nu, s, &tab);
+    return get_cov_table(family, nu, s, &tab, true);
   }
   ~TablePin() {
     if (tab) cov_table_used(tab, stream);
@@ -101,9 +100,10 @@ struct SmemLayout {
 // Up to 13 warps per CTA for the forward pass (its two-vector blocks fit thirteen on an
 // SM at m = 60) and 12 for the gradient; the 8-lane gradient kernels are bounded for 16
 // warps per SM (two CTAs of 8, at most 128 registers a thread), which their second-gather
-// layout reaches at m = 25.
-template <bool GRAD, int G, bool SPHERE>
-__global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : 32 * kMaxCtaWarps) vecchia_lik_kernel(const LikArgs a) {
+// layout reaches at m = 25.  The fixed-point kernels (FIXED) take up to 168 registers a thread.
+template <bool GRAD, int G, bool SPHERE, bool FIXED>
+__global__ void __launch_bounds__(GRAD && G == 8 ? 512 : GRAD || FIXED ? 384 : 32 * kMaxCtaWarps)
+    vecchia_lik_kernel(const LikArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NL = 32 / G;
   const int K = a.m + 1;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : 32 * kMaxCtaWarp
   build_schedules(K, sched, pairs);
   __syncthreads();
 
-  const MaternConst mc = load_matern_const(a.tab);
+  const MaternConst mc = matern_const_at(fix_const(a.tab));
   ThetaConst tc;
   tc.set(a.sigma2, a.beta, a.tau2, a.family, a.nu);
   FieldView F;
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : 32 * kMaxCtaWarp
     const bool active = i < a.i1;
     const int64_t ii = active ? i : base;
     double* trow = terms_mode ? a.terms + ii * (GRAD ? 4 : 1) : nullptr;
-    process_location<GRAD, G, SPHERE>(ii, active, F, L.S, sched, pairs, area, a.tab, mc, tc, acc, terms_mode, trow,
+    process_location<GRAD, G, SPHERE, FIXED>(ii, active, F, L.S, sched, pairs, area, a.tab, mc, tc, acc, terms_mode, trow,
                               a.errloc, sub);
   }
   // The CTA's warps' sums are combined in warp order (compensated), one record per CTA.
@@ -204,27 +204,31 @@ struct LaunchCfg {
   int sms = 0;            // SMs of the device
 };
 
+using LikKernel = void (*)(const LikArgs);
+
 template <bool GRAD, bool SPHERE>
-void* kernel_ptr(int G) {
-  if (G == 4) return reinterpret_cast<void*>(vecchia_lik_kernel<GRAD, 4, SPHERE>);
-  if (G == 8) return reinterpret_cast<void*>(vecchia_lik_kernel<GRAD, 8, SPHERE>);
-  if (G == 16) return reinterpret_cast<void*>(vecchia_lik_kernel<GRAD, 16, SPHERE>);
-  return reinterpret_cast<void*>(vecchia_lik_kernel<GRAD, 32, SPHERE>);
+LikKernel kernel_ptr(int G, bool fixed) {
+  if (G == 4) return vecchia_lik_kernel<GRAD, 4, SPHERE, false>;
+  if (G == 8) return vecchia_lik_kernel<GRAD, 8, SPHERE, false>;
+  if (G == 16) return vecchia_lik_kernel<GRAD, 16, SPHERE, false>;
+  return fixed ? vecchia_lik_kernel<GRAD, 32, SPHERE, true> : vecchia_lik_kernel<GRAD, 32, SPHERE, false>;
 }
 
-void* lik_kernel(bool grad, int G, bool sphere) {
-  if (grad) return sphere ? kernel_ptr<true, true>(G) : kernel_ptr<true, false>(G);
-  return sphere ? kernel_ptr<false, true>(G) : kernel_ptr<false, false>(G);
+LikKernel lik_kernel(int K, bool grad, int G, bool sphere) {
+  const bool fixed = fixed_point_block(K, grad, G);
+  if (grad) return sphere ? kernel_ptr<true, true>(G, fixed) : kernel_ptr<true, false>(G, fixed);
+  return sphere ? kernel_ptr<false, true>(G, fixed) : kernel_ptr<false, false>(G, fixed);
 }
 
 // Lanes per location chosen when no tuning result exists: small blocks share a warp.  The
-// break points are the fastest measured shapes on GB300 at n = 1e6 (m = 15, 20, 25, 31,
-// 45, 60); the adjoint favours wider groups a little earlier than the forward pass.
+// break points are the fastest shapes measured at n = 100k (ms, 8 / 16 lanes: forward m = 28
+// 1.23 / 1.27, m = 30 1.53 / 1.48; with the gradient m = 23 1.07 / 1.16, m = 26 1.44 / 1.43, m = 30
+// 2.15 / 1.89; 16 / 32 lanes: forward m = 34 1.97 / 2.19, m = 38 2.70 / 2.55 (fixed point); with the
+// gradient m = 34 2.53 / 2.73, m = 38 3.61 / 3.40).
 int default_lanes(int K, bool grad) {
   if (K <= 16) return 4;
-  if (K <= 32) return 8;
-  if (K <= 48) return grad ? 32 : 16;
-  return 32;
+  if (grad) return K <= 26 ? 8 : (K <= 35 ? 16 : 32);
+  return K <= 29 ? 8 : (K <= 37 ? 16 : 32);
 }
 
 // Tuning results, per (device, K, grad): lanes per location and warps per CTA.
@@ -300,7 +304,7 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
   int dev = 0, sms = 0, smem_optin = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_shape_mu);
-  void* kern = lik_kernel(grad, G, sphere);
+  void* kern = reinterpret_cast<void*>(lik_kernel(K, grad, G, sphere));
   for (const ShapeEntry& e : g_shapes)
     if (e.dev == dev && e.K == K && e.grad == (int)grad && e.G == G && e.W == forced_W && e.sphere == (int)sphere) {
       const int rc = set_smem_limit(dev, kern, e.cfg.smem);
@@ -358,10 +362,15 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
 // Configuration for block size K: the tuned shape if vecchia_autotune recorded one, else
 // the default lanes per location.  VECCHIA_LANES_PER_LOCATION / VECCHIA_WARPS_PER_CTA
 // force either value (tuning experiments).  `count` (> 0: the call's locations) widens
-// the default groups, up to 16 lanes, while they would leave fewer location groups than
-// the GPU has sub-partitions: such a call is bound by each warp's serial latency, which
-// wider groups shorten (n = 2,000, m = 10, per call: 4 lanes 33.9 us, 8 lanes 30.7, 16
-// lanes 28.8, 32 lanes 41.1).
+// the default groups while they would leave fewer location groups than the GPU has
+// sub-partitions: such a call is bound by each warp's serial latency, which wider groups
+// shorten (n = 2,000, m = 10, per call: 4 lanes 33.9 us, 8 lanes 30.7, 16 lanes 28.8, 32
+// lanes 41.1; n = 1,000, m = 30 with the gradient: 8 lanes 131, 16 lanes 80.0, 32 lanes
+// 61.5; m = 10: 16 lanes 30.9, 32 lanes 32.0, so up to 16 lanes for the smallest blocks).
+// And where 16-lane groups would need a second turn of the resident warps while 8-lane
+// groups all fit at once, those are taken (m = 30, n = 6,000, 8 and 16 lanes: 121 and 137
+// us, with the gradient 176 and 190; n = 4,000, one turn either way: 148 and 131 with the
+// gradient).
 int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t count = -1) {
   int dev = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
@@ -379,30 +388,22 @@ int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t c
   if (!chosen && count > 0) {
     int sms = 0;
     VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    while (G < 16 && (count + 32 / G - 1) / (32 / G) < 4 * (int64_t)sms) G *= 2;
+    const int most = K <= 16 ? 16 : 32;
+    while (G < most && (count + 32 / G - 1) / (32 / G) < 4 * (int64_t)sms) G *= 2;
+    if (G == 16 && K <= max_k_for_lanes(8)) {
+      LaunchCfg wide, narrow;
+      int rc = shape_for(K, grad, 16, W, &wide, sphere);
+      if (!rc) rc = shape_for(K, grad, 8, W, &narrow, sphere);
+      if (rc) return rc;
+      if ((count + 1) / 2 > (int64_t)wide.blocks * wide.W && (count + 3) / 4 <= (int64_t)narrow.blocks * narrow.W) G = 8;
+    }
   }
   while (K > max_k_for_lanes(G)) G *= 2;
   return shape_for(K, grad, G, W, cfg, sphere);
 }
 
-template <bool SPHERE>
-void launch_lik_m(const LaunchCfg& cfg, bool grad, const LikArgs& a, cudaStream_t stream) {
-  if (grad) {
-    if (cfg.G == 4) vecchia_lik_kernel<true, 4, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-    else if (cfg.G == 8) vecchia_lik_kernel<true, 8, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-    else if (cfg.G == 16) vecchia_lik_kernel<true, 16, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-    else vecchia_lik_kernel<true, 32, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-  } else {
-    if (cfg.G == 4) vecchia_lik_kernel<false, 4, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-    else if (cfg.G == 8) vecchia_lik_kernel<false, 8, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-    else if (cfg.G == 16) vecchia_lik_kernel<false, 16, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-    else vecchia_lik_kernel<false, 32, SPHERE><<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
-  }
-}
-
 void launch_lik(const LaunchCfg& cfg, bool grad, const LikArgs& a, cudaStream_t stream) {
-  if (a.metric == 1) launch_lik_m<true>(cfg, grad, a, stream);
-  else launch_lik_m<false>(cfg, grad, a, stream);
+  lik_kernel(a.m + 1, grad, cfg.G, a.metric == 1)<<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
 }
 }  // namespace
 
@@ -760,7 +761,7 @@ constexpr int kNoAllocWarps = 4096;
 constexpr size_t kNoAllocPartialBytes = sizeof(double) * 4 * kNoAllocWarps;
 constexpr size_t kNoAllocErrOff = kNoAllocPartialBytes;
 constexpr size_t kNoAllocTabOff = kNoAllocErrOff + 256;
-constexpr size_t kNoAllocBytes = kNoAllocTabOff + (kTableBytes + 255) / 256 * 256;
+constexpr size_t kNoAllocBytes = kNoAllocTabOff + (kFixTableBytes + 255) / 256 * 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 namespace {

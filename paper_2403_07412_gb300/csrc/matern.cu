@@ -14,10 +14,12 @@
 // FP64/FP32 layout that matern.cuh evaluates.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
 #include "common.cuh"
+#include "fixtable.cuh"
 #include "matern.cuh"
 
 namespace vecchia {
@@ -59,11 +61,10 @@ __device__ double quad_I_warp(double u, double nu) {
 
 // One warp: I(0) and the small-u expansion constants (family Matérn), or the exponent
 // (power exponential).
-__global__ void matern_const_kernel(double nu, int family, double* tab) {
+__global__ void matern_const_kernel(double nu, int family, double* c) {
   if (blockIdx.x != 0 || threadIdx.x >= 32) return;
   const double I0 = family == kFamilyPowExp ? 1.0 : quad_I_warp(0.0, nu);
   if (threadIdx.x != 0) return;
-  double* c = tab + 2 * kIntWords * kNInt;
   if (family == kFamilyPowExp) {
     c[0] = __longlong_as_double(3LL);
     c[1] = nu;
@@ -172,8 +173,253 @@ __global__ void __launch_bounds__(kFitThreads) matern_fit_kernel(double nu, int 
   if (tid == 0) write_interval(mono, reinterpret_cast<float*>(tab) + (size_t)idx * 4 * kIntWords);
 }
 
+// ------------------------------------------------------------------ likelihood table
+// The likelihood kernels' table (fixtable.cuh) is wanted to 2^-60 or so of rho(0) = 1, and
+// an optimiser that moves nu builds one at every step, so it is built in 64-bit integers,
+// which cost a warp 2 to 5 cycles an instruction where FP64 costs 64:
+//   rho(u) = sum_k W_k exp(-u G_k),  W_k = h exp(nu tau_k - e^tau_k) / Gamma(nu),
+// G_k = e^-tau_k / 4, the trapezoidal rule for I(u) on one grid for all u.  h = ln 2 / p, so
+// that e^tau_k is a power of two times one of p numbers in [1, 2).  h <= 0.6 / sqrt(nu + 36)
+// resolves the integrand's peak (width 1 / sqrt(nu + x) or so) up to x = 36, beyond which
+// rho is below 2^-51 and the rule's relative error may grow; the grid ends where W_k, or
+// exp(-2^kELo G_k), has fallen below e^-44.
+// A fresh nu took 350 us beside the call's own work with a quadrature in FP64 of each
+// interval's Chebyshev values.
+struct FixSetup {
+  int family, p, klo, n;
+  unsigned long long lnp;    // ln 2 / p in units of 2^-64
+  double nu, norm, norm_lo;  // log Gamma(nu) - log h as a pair
+  double c[kNConst];         // small-u constants (matern.cuh)
+  FixSetup(int family_, double nu_) : family(family_), nu(nu_) {
+    p = 1;
+    klo = n = 0;
+    lnp = 0;
+    norm = norm_lo = 0.0;
+    for (double& v : c) v = 0.0;
+    c[1] = nu;
+    const bool integer = nu == std::floor(nu);
+    const long long kind = family == kFamilyPowExp ? 3 : integer ? (nu == 1.0 ? 1 : 2) : 0;
+    std::memcpy(&c[0], &kind, sizeof(kind));
+    if (family == kFamilyPowExp) return;
+    if (integer) {
+      c[2] = nu == 1.0 ? 0.0 : -0.25 / (nu - 1.0);
+    } else {
+      c[2] = 0.25 / (1.0 - nu);
+      c[3] = std::tgamma(1.0 - nu);
+      c[4] = 1.0 / std::tgamma(1.0 + nu);
+      c[5] = 0.25 / std::tgamma(2.0 + nu);
+    }
+    constexpr double kLn2 = 0.693147180559945309417;
+    const double hi = std::log(60.0 + nu + std::min(nu, 14.0 * std::sqrt(nu)));
+    const double lo = std::max(std::log(nu) - 45.0 / nu - std::sqrt(120.0 / nu), -26.5);
+    const double most = (kFixNodes - 3) * kLn2 / (hi - lo);
+    p = (int)std::max(1.0, std::min(std::ceil(kLn2 * std::sqrt(nu + 36.0) / 0.6), std::min(std::floor(most), 1e6)));
+    klo = (int)std::floor(lo * p / kLn2);
+    n = std::min(kFixNodes, (int)std::ceil(hi * p / kLn2) - klo + 1);
+    lnp = 0xB17217F7D1CF79ACull / p;
+    const long double v = std::lgamma((long double)nu) - std::log(0.693147180559945309417232121458L / p);
+    norm = (double)v;
+    norm_lo = (double)(v - norm);
+  }
+};
+
+// exp(-x 2^-58) in units of 2^-63, for x < 44 2^58: x = n ln 2 + 16 z; d = 1 - e^-z by its
+// Taylor polynomial of degree 9 (z < 0.0434; the terms from z^7 on in 32 bits), then four
+// times 1 - d <- (1 - d)^2.  Its error is a few units.
+__device__ __forceinline__ unsigned long long fix_exp(unsigned long long x) {
+  const unsigned n = __umulhi((unsigned)(x >> 32), 0xB8AA3B29u) >> 25;  // log2(e) 2^31
+  const unsigned long long z = ((x << 5) - n * 0x58B90BFBE8E7BCD6ull) >> 3;  // units of 2^-64
+  const unsigned zh = (unsigned)(z >> 32);
+  unsigned t = ~0u - __umulhi(zh, 0xFFFFFFFFu / 9);
+  t = ~0u - __umulhi(__umulhi(zh, 0xFFFFFFFFu / 8), t);
+  t = ~0u - __umulhi(__umulhi(zh, 0xFFFFFFFFu / 7), t);
+  constexpr unsigned long long one = ~0ull;
+  unsigned long long a = __umul64hi(one / 720, (unsigned long long)t << 32);
+  a = one / 120 - __umul64hi(z, a);
+  a = one / 24 - __umul64hi(z, a);
+  a = one / 6 - __umul64hi(z, a);
+  a = one / 2 - __umul64hi(z, a);
+  unsigned long long d = z - __umul64hi(z, __umul64hi(z, a));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) d = 2 * d - __umul64hi(d, d);
+  return (0x8000000000000000ull - (d >> 1)) >> n;
+}
+
+// 2^-tau/ln2 at node k: 2^q times 2^(b/p), 0 <= b < p.
+__device__ __forceinline__ void fix_node_power(const FixSetup& s, int k, int& q, int& b) {
+  const int K = -(s.klo + k);
+  q = K >= 0 ? K / s.p : -((s.p - 1 - K) / s.p);
+  b = K - q * s.p;
+}
+
+// Nodes (after the constants): W_k in units of 2^-65, and 2^(b/p - 1) in units of 2^-63.
+__global__ void fix_nodes_kernel(const FixSetup s, double* tab) {
+  double* c = fix_const(tab);
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  if (k < kNConst) c[k] = s.c[k];
+  if (k >= s.n) return;
+  int q, b;
+  fix_node_power(s, k, q, b);
+  const unsigned long long bl = b * s.lnp;
+  const unsigned long long et = fix_exp(bl >> 6);  // e^tau = et 2^(-63 - q)
+  const long long tau = -q * 0x162E42FEFA39EF3ll - (long long)(bl >> 7);  // units of 2^-57; and q ln 2's rest
+  const double th = (double)tau, tl = (double)(tau - (long long)th) - 0.34375 * q;
+  const double ph = s.nu * th, pl = fma(s.nu, tl, fma(s.nu, th, -ph));
+  const double sc = __longlong_as_double((long long)(1023 - 63 - q) << 52);
+  const double eh = (double)et, el = (double)(long long)(et - (unsigned long long)eh);
+  // x = norm - nu tau + e^tau >= 0, as a pair
+  Neumaier x;
+  x.add(s.norm);
+  x.add(-ph * 0x1p-57);
+  x.add(eh * sc);
+  x.add(s.norm_lo - pl * 0x1p-57 + el * sc);
+  const double xt = x.s + x.c;
+  unsigned long long w = 0;
+  if (xt < 44.0) {
+    const double xl = (x.s - xt) + x.c;
+    const unsigned long long xi = __double2ull_rn(fmax(xt, 0.0) * 0x1p58);
+    w = min(fix_exp(xi + (unsigned long long)__double2ll_rn(fmax(xl, -xt) * 0x1p58)), 0x1FFFFFFFFFFFFFFFull) << 2;
+  }
+  const unsigned long long mant = fix_exp(((s.p - b) * s.lnp) >> 6);
+  reinterpret_cast<ulonglong2*>(c + kNConst)[k] = make_ulonglong2(w, mant);
+}
+
+// v 2^sh as the argument of fix_exp; past its range (x >= 44): all ones.
+__device__ __forceinline__ unsigned long long fix_arg_shift(unsigned long long v, int sh) {
+  constexpr unsigned long long most = 44ull << 58;
+  if (sh >= 0) return sh >= 64 || v > (most >> min(sh, 63)) ? ~0ull : v << sh;
+  if (sh <= -64) return 0;
+  v >>= -sh;
+  return v >= most ? ~0ull : v;
+}
+__device__ __forceinline__ unsigned long long fix_exp_or_0(unsigned long long x) { return x == ~0ull ? 0 : fix_exp(x); }
+
+// cos(i pi / 16)
+constexpr double kCos16[9] = {1.0,
+                              0.98078528040323044913,
+                              0.92387953251128675613,
+                              0.83146961230254523708,
+                              0.70710678118654752440,
+                              0.55557023301960222474,
+                              0.38268343236508977173,
+                              0.19509032201612826785,
+                              0.0};
+constexpr double cos16(int i) {
+  i &= 31;
+  if (i > 16) i = 32 - i;
+  return i <= 8 ? kCos16[i] : -kCos16[16 - i];
+}
+static_assert(kFixDeg == 7, "the interpolation nodes are those of degree 7");
+// Interpolation at the eight Chebyshev points t_q = (1 + cos((2q + 1) pi / 16)) / 2: the
+// coefficient of T_j(2t - 1) is sum_q cheb[j][q] f(t_q), that of t^k sum_j mono[j][k] (it); t_q
+// in units of 2^-64.  (The product of the two matrices has entries up to 10^4 of either sign:
+// FP64 sums with it lose the small coefficients.)
+struct FixInterp {
+  double cheb[8][8], mono[8][8];
+  unsigned long long t[8];
+  constexpr FixInterp() : cheb(), mono(), t() {
+    mono[0][0] = 1.0;
+    mono[1][0] = -1.0;
+    mono[1][1] = 2.0;
+    for (int j = 2; j < 8; ++j)
+      for (int k = 0; k < 8; ++k)
+        mono[j][k] = 2.0 * ((k > 0 ? 2.0 * mono[j - 1][k - 1] : 0.0) - mono[j - 1][k]) - mono[j - 2][k];
+    for (int q = 0; q < 8; ++q) {
+      for (int j = 0; j < 8; ++j) cheb[j][q] = (j ? 0.25 : 0.125) * cos16(j * (2 * q + 1));
+      t[q] = (unsigned long long)((0.5 + 0.5 * cos16(2 * q + 1)) * 0x1p64);
+    }
+  }
+};
+__device__ const FixInterp kFixInterp = FixInterp();
+
+// One CTA per kFixGroup = 8 intervals [2^e (1 + j/32), ...) of an octave, 64 values u = 2^e
+// (1 + (j + t)/32).  exp(-u G) is the product of a factor for j, which takes W too, and one
+// for t: 16 exponentials a node for the 64 values, and a 64-bit product each (some 30
+// cycles of a warp; an exponential some 350, 1,400 in FP64).  Then the eight values of an
+// interval give its monomials: integer differences from one of them, exact, times the
+// matrix above in FP64, a thread per coefficient.
+constexpr int kFixGroup = 8;
+constexpr int kFixThreads = 256;
+constexpr int kFixChunk = 64;  // nodes at a time
+
+__global__ void __launch_bounds__(kFixThreads) fix_table_kernel(const FixSetup s, double* tab) {
+  __shared__ unsigned long long ea[kFixChunk][kFixGroup], eb[kFixChunk][8], part[4][64];
+  const int tid = threadIdx.x;
+  const int e = kELo + (blockIdx.x * kFixGroup >> kFixSub);
+  const int j0 = blockIdx.x * kFixGroup & ((1 << kFixSub) - 1);
+  if (s.family == kFamilyPowExp) {
+    if (tid < 64) {
+      const double t = (double)kFixInterp.t[tid & 7] * 0x1p-64;
+      const double u = ldexp(1.0 + (j0 + (tid >> 3) + t) / (1 << kFixSub), e);
+      part[0][tid] = __double2ull_rn(exp(-exp(0.5 * s.nu * log(u))) * 0x1p63);
+    }
+  } else {
+    const ulonglong2* __restrict__ nodes = reinterpret_cast<const ulonglong2*>(fix_const(tab) + kNConst);
+    const int k0 = max(0, (int)((e - 7.5f) * s.p) - s.klo - 1);  // 2^e G_k < 44 from here on
+    unsigned long long acc = 0;
+    const int out = tid & 63, slice = tid >> 6;
+    for (int kc = k0; kc < s.n; kc += kFixChunk) {
+      const int kk = tid & (kFixChunk - 1), k = kc + kk, r = 2 * (tid / kFixChunk);
+      ulonglong2 w = make_ulonglong2(0, 0);
+      int q = 0, b;
+      if (k < s.n) {
+        w = nodes[k];
+        fix_node_power(s, k, q, b);
+      }
+      // 2^e G = mant 2^(e + q - 1)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const unsigned long long xa = fix_arg_shift((w.y >> 6) * (32 + j0 + r + i), e + q - 5);
+        ea[kk][r + i] = __umul64hi(w.x, fix_exp_or_0(xa));
+        const unsigned long long xb = fix_arg_shift(__umul64hi(w.y, kFixInterp.t[r + i]), e + q - 11);
+        eb[kk][r + i] = fix_exp_or_0(xb);
+      }
+      __syncthreads();
+#pragma unroll 4
+      for (int i = slice * (kFixChunk / 4); i < (slice + 1) * (kFixChunk / 4); ++i)
+        acc += __umul64hi(ea[i][out >> 3], eb[i][out & 7]);
+      __syncthreads();
+    }
+    if (slice == 0 && s.n > k0) acc += (unsigned)(s.n - k0) / 2;  // the products are rounded down
+    part[slice][out] = acc;
+  }
+  __syncthreads();
+  if (tid >= 64) return;
+  if (s.family != kFamilyPowExp) part[0][tid] += part[1][tid] + part[2][tid] + part[3][tid];
+  __syncwarp();
+  const int k = tid & 7;
+  const unsigned long long* __restrict__ f = part[0] + (tid & ~7);
+  double a = 0.0, m = 0.0;
+#pragma unroll 1
+  for (int q = 0; q < 8; ++q) a = fma(kFixInterp.cheb[k][q], (double)(long long)(f[q] - f[4]) * 0x1p-63, a);
+#pragma unroll 1
+  for (int j = 7; j >= 0; --j) m = fma(kFixInterp.mono[j][k], __shfl_sync(0xffffffffu, a, j, 8), m);
+  // S = -exponent of the largest of c1..c4
+  int top = k >= 1 && k <= 4 ? (int)((__double_as_longlong(m) >> 52) & 0x7FF) : 0;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o, 8));
+  const int S = top > 0 ? 1022 - top : 0;
+  const double ms = m * __longlong_as_double((long long)(1023 + S) << 52);
+  float* w = reinterpret_cast<float*>(tab) + (size_t)(blockIdx.x * kFixGroup + (tid >> 3)) * 4 * kFixWords;
+  if (k == 0) {
+    const long long c0 = (long long)((f[4] + 1) >> 1) + __double2ll_rn(m * 0x1p62);
+    w[12] = __int_as_float((int)(unsigned)((unsigned long long)c0 & 0xFFFFFFFFull));
+    w[13] = __int_as_float((int)(c0 >> 32));
+    w[14] = ldexpf(1.0f, 36 - S);
+    w[15] = ldexpf(1.0f, -S);
+  } else if (k <= 4) {
+    split_float(ms, w + 2 * (k - 1));
+    if (k == 3) split_float(3.0 * ms, w + 16);
+  } else {
+    w[8 + k - 5] = (float)ms;
+    if (k == 5) w[18] = (float)(5.0 * ms);
+    if (k == 6) w[19] = (float)(6.0 * ms);
+    if (k == 7) w[11] = 0.0f;
+  }
+}
+
 // ------------------------------------------------------------------ table cache
-// Tables are cached per (device, family, nu), at most kMaxTables per process; a call that
+// Tables are cached per (device, kind, family, nu), at most kMaxTables of a kind per process; a call that
 // needs a table not in the cache builds it on its own stream.  Every launch that reads a
 // table records a use event on its stream afterwards (cov_table_used; one event per
 // stream that used the table).  When the cache is full, the least recently used table
@@ -187,6 +433,7 @@ struct TableUse {
 };
 struct TableEntry {
   int device = -1;
+  bool fixed = false;  // the likelihood kernels' table
   int family = 0;
   double nu = 0.0;
   double* d_tab = nullptr;
@@ -200,17 +447,29 @@ std::vector<TableEntry> g_tables;
 unsigned long long g_clock = 0;
 constexpr size_t kMaxTables = 32;
 constexpr size_t kMaxUseStreams = 8;
+
+void launch_cov_table(int family, double nu, double* tab, cudaStream_t stream, bool fixed) {
+  if (fixed) {
+    const FixSetup q(family, nu);
+    fix_nodes_kernel<<<kFixNodes / 32, 32, 0, stream>>>(q, tab);
+    fix_table_kernel<<<kFixInt / kFixGroup, kFixThreads, 0, stream>>>(q, tab);
+    return;
+  }
+  matern_const_kernel<<<1, 32, 0, stream>>>(nu, family, tab + 2 * kIntWords * kNInt);
+  matern_fit_kernel<<<kNInt, kFitThreads, 0, stream>>>(nu, family, tab);
+}
 }  // namespace
 
-// Returns (building on `stream` if needed) the device table for (family, nu) on the
+// Returns (building on `stream` if needed) the device table for (family, nu), the likelihood
+// kernels' (fixed) or the covariance evaluator's, on the
 // current device, and makes `stream` wait until it is built.  The caller launches its
 // kernels and then calls cov_table_used(table, stream).
-int get_cov_table(int family, double nu, cudaStream_t stream, const double** out) {
+int get_cov_table(int family, double nu, cudaStream_t stream, const double** out, bool fixed) {
   int dev = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_mu);
   for (auto& t : g_tables) {
-    if (t.device == dev && t.family == family && t.nu == nu) {
+    if (t.device == dev && t.fixed == fixed && t.family == family && t.nu == nu) {
       VECCHIA_CUDA_TRY(cudaStreamWaitEvent(stream, t.ready, 0));
       t.last_use = ++g_clock;
       t.pending += 1;
@@ -220,9 +479,11 @@ int get_cov_table(int family, double nu, cudaStream_t stream, const double** out
   }
   TableEntry* slot = nullptr;
   TableEntry* victim = nullptr;
+  size_t of_kind = 0;
+  for (auto& t : g_tables) of_kind += t.fixed == fixed;
   for (auto& t : g_tables)  // least recently used table of this device not pinned by a call
-    if (t.device == dev && t.pending == 0 && (!victim || t.last_use < victim->last_use)) victim = &t;
-  if (g_tables.size() >= kMaxTables && victim) {
+    if (t.device == dev && t.fixed == fixed && t.pending == 0 && (!victim || t.last_use < victim->last_use)) victim = &t;
+  if (of_kind >= kMaxTables && victim) {
     // Rebuild in place once every earlier reader of the old contents has finished.
     for (const TableUse& u : victim->uses) {
       VECCHIA_CUDA_TRY(cudaStreamWaitEvent(stream, u.done, 0));
@@ -232,7 +493,7 @@ int get_cov_table(int family, double nu, cudaStream_t stream, const double** out
     slot = victim;
   } else {
     double* d = nullptr;
-    if (cudaMalloc(&d, kTableBytes) != cudaSuccess) return VECCHIA_ENOMEM;
+    if (cudaMalloc(&d, fixed ? kFixTableBytes : kTableBytes) != cudaSuccess) return VECCHIA_ENOMEM;
     cudaEvent_t ev;
     if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
       cudaFree(d);
@@ -243,11 +504,11 @@ int get_cov_table(int family, double nu, cudaStream_t stream, const double** out
     slot->d_tab = d;
     slot->ready = ev;
   }
-  matern_const_kernel<<<1, 32, 0, stream>>>(nu, family, slot->d_tab);
-  matern_fit_kernel<<<kNInt, kFitThreads, 0, stream>>>(nu, family, slot->d_tab);
+  launch_cov_table(family, nu, slot->d_tab, stream, fixed);
   VECCHIA_CUDA_TRY(cudaGetLastError());
   VECCHIA_CUDA_TRY(cudaEventRecord(slot->ready, stream));
   slot->device = dev;
+  slot->fixed = fixed;
   slot->family = family;
   slot->nu = nu;
   slot->pending = 1;
@@ -281,15 +542,10 @@ void cov_table_used(const double* tab, cudaStream_t stream) {
   }
 }
 
-int get_matern_table(double nu, cudaStream_t stream, const double** out) {
-  return get_cov_table(kFamilyMatern, nu, stream, out);
-}
-
-// Builds the Matérn table for nu into caller-provided device memory (kTableBytes,
-// 16-byte aligned) on `stream`, without touching the cache.
+// Builds the likelihood kernels' Matérn table for nu into caller-provided device memory
+// (kFixTableBytes, 16-byte aligned) on `stream`, without touching the cache.
 int launch_matern_table(double nu, double* tab, cudaStream_t stream) {
-  matern_const_kernel<<<1, 32, 0, stream>>>(nu, kFamilyMatern, tab);
-  matern_fit_kernel<<<kNInt, kFitThreads, 0, stream>>>(nu, kFamilyMatern, tab);
+  launch_cov_table(kFamilyMatern, nu, tab, stream, true);
   VECCHIA_CUDA_TRY(cudaGetLastError());
   return VECCHIA_OK;
 }
@@ -332,7 +588,7 @@ static int covariance(int family, const double* d_dev, int64_t count, const doub
   if (count < 0 || (count > 0 && (!d_dev || !c_dev)) || !theta_ok_family(theta, family)) return VECCHIA_EINVAL;
   if (count == 0) return VECCHIA_OK;
   const double* tab = nullptr;
-  int rc = get_cov_table(family, theta[2], s, &tab);
+  int rc = get_cov_table(family, theta[2], s, &tab, false);
   if (rc) return rc;
   const int64_t blocks = std::min<int64_t>((count + 255) / 256, 4096);
   matern_eval_kernel<<<(int)blocks, 256, 0, s>>>(d_dev, count, theta[0], theta[1], family, tab, c_dev,

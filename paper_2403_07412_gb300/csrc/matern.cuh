@@ -40,8 +40,7 @@ __device__ __forceinline__ const float4* table_iv(const double* tab) {
 }
 __device__ __forceinline__ const double* table_c(const double* tab) { return tab + 2 * kIntWords * kNInt; }
 
-__device__ __forceinline__ MaternConst load_matern_const(const double* __restrict__ tab) {
-  const double* c = table_c(tab);
+__device__ __forceinline__ MaternConst matern_const_at(const double* __restrict__ c) {
   MaternConst mc;
   mc.kind = (int)__double_as_longlong(c[0]);
   mc.nu = c[1];
@@ -50,6 +49,9 @@ __device__ __forceinline__ MaternConst load_matern_const(const double* __restric
   mc.b0 = c[4];
   mc.b1 = c[5];
   return mc;
+}
+__device__ __forceinline__ MaternConst load_matern_const(const double* __restrict__ tab) {
+  return matern_const_at(table_c(tab));
 }
 
 // f 2^adj as a double, exactly, with integer operations (0 for zero, subnormal f, or
@@ -244,54 +246,9 @@ __device__ __forceinline__ double h_fix(double u, const MaternConst& mc, double 
   return h;
 }
 
-// ---- evaluation from a double-float argument u = uh + ul (likelihood kernels)
-// The interval index and t come from uh's float bits: u / 2^e = 1.m, t = 32 u / 2^e -
-// 33 - 2j, so th = (m mod 2^19) 2^-18 - 1 exactly and tl = ul 2^(5-e); 32 M = u dt/du is
-// (uh, ul) 2^(5-e).  Outside [2^kELo, 2^kEHi) the clamped index gives a finite value that
-// the rare path below replaces.
-struct PolyArgF {
-  int idx, ex;
-  float th, tl, mh, ml;  // t and 32 M as float pairs
-};
-
-__device__ __forceinline__ PolyArgF poly_arg_df(float uh, float ul) {
-  PolyArgF a;
-  const unsigned ub = __float_as_uint(uh);
-  a.ex = (int)((ub >> 23) & 0xFF) - 127;
-  const int ec = min(max(a.ex, kELo), kEHi - 1);
-  a.idx = ((ec - kELo) << kSub) | (int)((ub >> 19) & ((1u << kSub) - 1));
-  a.th = fmaf(__uint_as_float(0x3F800000u | ((ub & 0x7FFFFu) << 4)), 2.0f, -3.0f);
-  const float sc = __uint_as_float((unsigned)(127 + 5 - ec) << 23);
-  a.tl = __fmul_rn(ul, sc);
-  a.mh = __fmul_rn(uh, sc);
-  a.ml = a.tl;
-  return a;
-}
-
 // u outside the tabulated range as a double (rare path).
 __device__ __forceinline__ double df_to_double(float uh, float ul) {
   return f2d_scaled(uh, 0) + f2d_scaled(ul, 0);
-}
-
-__device__ __forceinline__ double rho_df(float uh, float ul, const double* __restrict__ tab, const MaternConst& mc) {
-  const PolyArgF a = poly_arg_df(uh, ul);
-  const float4* __restrict__ w = table_iv(tab) + a.idx * kIntWords;
-  const float4 w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3);
-  const int S = __float_as_int(w3.z);
-  const float t5 = fmaf(fmaf(fmaf(w2.w, a.th, w2.z), a.th, w2.y), a.th, w2.x);
-  float ph, pl, xh, xl;
-  df_start(ph, pl, t5, a.th, w1.z, w1.w);
-  df_horner(ph, pl, a.th, a.tl, w1.x, w1.y);
-  df_horner(ph, pl, a.th, a.tl, w0.z, w0.w);
-  df_horner(ph, pl, a.th, a.tl, w0.x, w0.y);
-  df_mul(ph, pl, a.th, a.tl, xh, xl);
-  const double c0 = __hiloint2double(__float_as_int(w3.y), __float_as_int(w3.x));
-  double rho = (c0 + f2d_scaled(xh, -S)) + f2d_scaled(xl, -S);
-  if (a.ex < kELo || a.ex >= kEHi) {
-    double h = 0.0;
-    rho_fix(df_to_double(uh, ul), mc, rho, h);
-  }
-  return rho;
 }
 
 // f 2^k for a float, by its exponent field; 0 when the result falls below the normal
@@ -301,31 +258,6 @@ __device__ __forceinline__ float fscale(float f, int k) {
   const int ne = (int)((fb >> 23) & 0xFF) + k;
   if ((fb & 0x7F800000u) == 0u || ne <= 0) return 0.0f;
   return __uint_as_float((fb & 0x807FFFFFu) | ((unsigned)ne << 23));
-}
-
-// h(u) as a float pair (about 2^-46 relative), no FP64 instruction on the common path.
-__device__ __forceinline__ void h_df(float uh, float ul, const double* __restrict__ tab, const MaternConst& mc,
-                                     float& hh, float& hl) {
-  const PolyArgF a = poly_arg_df(uh, ul);
-  const float4* __restrict__ w = table_iv(tab) + a.idx * kIntWords;
-  const float4 w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3), w4 = __ldg(w + 4);
-  const int S = __float_as_int(w3.z);
-  const float d5 = fmaf(fmaf(fmaf(8.0f * w2.w, a.th, 7.0f * w2.z), a.th, w4.w), a.th, w4.z);
-  float qh, ql;
-  df_start(qh, ql, d5, a.th, 4.0f * w1.z, 4.0f * w1.w);
-  df_horner(qh, ql, a.th, a.tl, w4.x, w4.y);
-  df_horner(qh, ql, a.th, a.tl, 2.0f * w0.z, 2.0f * w0.w);
-  df_horner(qh, ql, a.th, a.tl, w0.x, w0.y);
-  df_mul(qh, ql, a.mh, a.ml, hh, hl);  // 32 M P'(t), times 2^S
-  hh = fscale(hh, -S);
-  hl = fscale(hl, -S);
-  if (a.ex < kELo || a.ex >= kEHi) {
-    double r = 0.0, h = 0.0;
-    rho_fix(df_to_double(uh, ul), mc, r, h);
-    const float hi = __double2float_rn(h);
-    hh = hi;
-    hl = __double2float_rn(h - (double)hi);
-  }
 }
 
 template <bool DERIV>
@@ -339,6 +271,34 @@ __device__ __forceinline__ double rho_only(double u, const double* __restrict__ 
   double r, h;
   rho_eval<false>(u, tab, mc, r, h);
   return r;
+}
+
+// x as a float pair hi + lo (hi: x's leading 24 bits, lo: the next 24, about 2^-48
+// relative), with integer operations; exponents far from 0 take the FP64 route.
+__device__ __forceinline__ float2 d2f_pair(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7FF) - 1023;
+  if (e < -90 || e > 90) {
+    const float hi = __double2float_rn(x);
+    return make_float2(hi, __double2float_rn(x - (double)hi));
+  }
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  const float hi = __uint_as_float(sign | ((unsigned)(e + 127) << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
+  // remainder: mantissa bits 28..5, v 2^(e-47) = (v 2^-24) 2^(e-23)
+  const float lo = fscale(u24_float((unsigned)(b >> 5) & 0xFFFFFFu), e - 23);
+  return make_float2(hi, __uint_as_float(__float_as_uint(lo) | sign));
+}
+
+// x as a float pair (hi: x's leading 24 bits, lo: the next 24), by integer operations
+// only; |x| below 2^-100 gives (0, 0).  For values of moderate exponent (factor entries).
+__device__ __forceinline__ float2 d2f_trunc(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7FF) - 1023;
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  const float hi = __uint_as_float(sign | ((unsigned)(e + 127) << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
+  const float lo = fscale(u24_float((unsigned)(b >> 5) & 0xFFFFFFu), e - 23);
+  const bool z = e < -100;
+  return make_float2(z ? 0.0f : hi, z ? 0.0f : __uint_as_float(__float_as_uint(lo) | sign));
 }
 
 }  // namespace vecchia

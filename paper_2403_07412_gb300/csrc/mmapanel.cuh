@@ -1,0 +1,441 @@
+// Elimination of a full-warp block in 64-bit fixed point: panels of eight columns in integer
+// arithmetic, the updates between panels on the tensor cores.
+//
+// On GB300 a warp's FP64 instruction holds its sub-partition's pipe for 64 cycles; at m = 60
+// the elimination's 1,270 of them per location were the kernels' bound (FP64 pipe 81-85%
+// busy).  A multiply-accumulate of 31-bit limbs takes about 16 cycles of the integer pipes,
+// an mma.m16n8k16 (half precision, FP32 accumulation) 7.4 for 2,048 products.  So the block
+// is factored without FP64, as a left-looking Cholesky A = Lc Lc^T:
+//   - entries below the diagonal, and Schur complements, in units of 2^-60 (they are at most
+//     1 in magnitude), the diagonal (up to 1 + gamma) in units of 2^(2f - 60), f =
+//     floor(log2(1 + gamma) / 2);
+//   - V = Lc 2^62.  Off-diagonal entries of Lc are at most 2^-f in magnitude: a Schur
+//     complement of R + gamma I is gamma I plus a positive semidefinite matrix with diagonal
+//     at most 1, hence Lc_rk^2 <= 1 / (1 + gamma);
+//   - the data row y and its factor entries z = Lc^-1 y in units of 2^(ky - 60) and
+//     2^(ky - 62) (PanelScale).
+// FP64's column-by-column update rounds entries of size 1 to 2^-54 at every step; here every
+// entry carries absolute errors of about 2^-58 and 2^-56.
+//
+// Updates between panels: A_rc -= sum_{k < c0} Lc_rk Lc_ck, for the eight columns of the next
+// panel at once, as exact products of integers.  V is stored as its eight bytes, V +
+// 0x8080808080808080 = sum_i b_i 256^(7-i): digits d_i = b_i - 128, each a half exactly.  The
+// products d_i d'_j of one diagonal i + j = s add up to integers below 2^22 (63 terms of at
+// most 2^14 for each pair), exact in an FP32 accumulator; it starts at 1.5 2^23, so that the
+// integer is read off the accumulator's bits.  Kept are i <= 7, j <= 6, i + j <= 7.
+//
+// The bytes take the factor entries' own places: the four entries (r, 4w .. 4w+3) of a row
+// become eight words, one per digit plane, each with the digit of the four columns; so the
+// panels need no memory of their own (12 locations an SM, as with FP64).  A lane's four k of
+// a k16 step are the four columns of one word group (the MMA's k order is free as long as
+// both operands share it), so a fragment register is one byte permute (1024 + b as a half)
+// and one packed subtraction.
+//
+// All loops over columns and rows stay rolled: the phases of a location then run from the
+// instruction cache (unrolled over a panel's columns, instruction fetch was the largest
+// stall and the kernel 1.5 times slower).
+#pragma once
+
+#include "common.cuh"
+#include "fixtable.cuh"
+#include "matern.cuh"
+
+namespace vecchia {
+
+constexpr int kPanelCols = 8;
+constexpr int kPanelWords = kPanelCols / 4;
+constexpr unsigned long long kByteBias = 0x8080808080808080ull;
+constexpr float kAccZero = 12582912.0f;  // 1.5 2^23
+constexpr unsigned kAccZeroBits = 0x4B400000u;
+
+__device__ __forceinline__ unsigned exponent_field(double x) {
+  return (unsigned)(__double_as_longlong(x) >> 52) & 0x7FFu;
+}
+
+// 2^k, -1022 <= k <= 1023 (clamped).
+__device__ __forceinline__ double pow2_double(int k) {
+  return __longlong_as_double((long long)(min(max(k, -1022), 1023) + 1023) << 52);
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const unsigned (&a)[4], const unsigned (&b)[2]) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// Two digits (bytes of w picked by sel) as a pair of halves.
+__device__ __forceinline__ unsigned digit_pair(unsigned w, unsigned sel) {
+  const unsigned p = __byte_perm(w, 0x64646464u, sel);  // 1024 + b
+  unsigned r;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(p), "r"(0x64806480u));  // - 1152
+  return r;
+}
+
+// Digit planes of four columns' integers.
+__device__ __forceinline__ void digit_planes(const long long (&v)[4], unsigned (&out)[8]) {
+  unsigned lo[4], hi[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const unsigned long long b = (unsigned long long)v[k] + kByteBias;
+    lo[k] = (unsigned)b;
+    hi[k] = (unsigned)(b >> 32);
+  }
+  const unsigned a = __byte_perm(lo[0], lo[1], 0x5140), b = __byte_perm(lo[2], lo[3], 0x5140);  // bytes 0, 1
+  const unsigned c = __byte_perm(lo[0], lo[1], 0x7362), d = __byte_perm(lo[2], lo[3], 0x7362);  // bytes 2, 3
+  out[7] = __byte_perm(a, b, 0x5410);
+  out[6] = __byte_perm(a, b, 0x7632);
+  out[5] = __byte_perm(c, d, 0x5410);
+  out[4] = __byte_perm(c, d, 0x7632);
+  const unsigned e = __byte_perm(hi[0], hi[1], 0x5140), f = __byte_perm(hi[2], hi[3], 0x5140);
+  const unsigned g = __byte_perm(hi[0], hi[1], 0x7362), h = __byte_perm(hi[2], hi[3], 0x7362);
+  out[3] = __byte_perm(e, f, 0x5410);
+  out[2] = __byte_perm(e, f, 0x7632);
+  out[1] = __byte_perm(g, h, 0x5410);
+  out[0] = __byte_perm(g, h, 0x7632);
+}
+
+// Integer of column x (0..3) from the digit planes of its word.
+__device__ __forceinline__ long long planes_value(const unsigned (&w)[8], int x) {
+  const unsigned s2 = ((4 + x) << 4) | x;
+  const unsigned lo = __byte_perm(__byte_perm(w[7], w[6], s2), __byte_perm(w[5], w[4], s2), 0x5410);
+  const unsigned hi = __byte_perm(__byte_perm(w[3], w[2], s2), __byte_perm(w[1], w[0], s2), 0x5410);
+  return (long long)((((unsigned long long)hi << 32) | lo) - kByteBias);
+}
+
+// Slots of the entries (row, k0 .. k0 + 3): slot of (row, k) is tri_off(K, k) + row - k.
+struct WordSlots {
+  int e[4];
+  __device__ __forceinline__ WordSlots(int K, int k0) {  // of row 0; add the row
+    e[0] = tri_off(K, k0) - k0;
+#pragma unroll
+    for (int i = 1; i < 4; ++i) e[i] = e[i - 1] - (K - k0 - i + 1) - 1;
+  }
+};
+
+// 1/sqrt(d) of a positive d < 2^62: with d 2^(2q) in [2^60, 2^62), 2^31 / sqrt(d 2^(2q)) =
+// (rh 2^31 + rl) 2^-60, in (1, 2].  FP32 seed y, then one third-order step y (1 + e/2 + 3
+// e^2/8), e = 1 - d y^2 in units of 2^-60 (|e| < 2^-20: the omitted 5 e^3/16 is below 2^-61).
+__device__ __forceinline__ void rsqrt_fixed(long long d, int& q, int& rh, int& rl) {
+  q = (__clzll(d) - 2) >> 1;
+  const long long dn = d << (2 * q);
+  const float g = __int2float_rn((int)(dn >> 32)) * 0x1p-30f;  // d 2^(2q) / 2^62 in [1/4, 1]
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(g));
+  r = fminf(fmaxf(r, 1.0f), 0x1.fffffep0f);
+  const int Y = (int)(((__float_as_uint(r) & 0x7FFFFFu) | 0x800000u) << 7);  // y 2^30
+  const long long t = (long long)(int)(dn >> 31) * Y + (((long long)((int)dn & 0x7FFFFFFF) * Y) >> 31);
+  const long long w = (long long)(int)(t >> 31) * Y + (((long long)((int)t & 0x7FFFFFFF) * Y) >> 31);
+  const long long e = (1LL << 60) - w;
+  const int e32 = (int)(e >> 8);
+  const int s = (int)(((long long)e32 * e32) >> 32);  // e^2 2^72
+  const long long de = e + ((3LL * s) >> 14);         // (e/2 + 3 e^2/8) 2^61
+  const long long R = ((long long)Y << 30) + (long long)Y * (int)(de >> 31) +
+                      (((long long)Y * ((int)de & 0x7FFFFFFF)) >> 31);
+  rh = (int)(R >> 31);
+  rl = (int)R & 0x7FFFFFFF;
+}
+
+// A finite double times 2^sh as a 64-bit integer, rounded to nearest; the result must stay
+// below 2^62 in magnitude (sh chosen from the largest exponent).
+__device__ __forceinline__ long long fixed_from_double(double x, int sh) {
+  const long long b = __double_as_longlong(x);
+  const int ef = (int)((b >> 52) & 0x7FF);
+  const unsigned long long mant = (unsigned long long)((b & 0xFFFFFFFFFFFFFLL) | (ef ? 0x10000000000000LL : 0LL)) << 9;
+  const int r = 9 - ((ef ? ef : 1) - 1075 + sh);  // x 2^sh = (mant << 9) >> r
+  const long long v = r <= 0 ? (long long)mant : r < 63 ? (long long)((mant + (1ull << (r - 1))) >> r) : 0LL;
+  return b < 0 ? -v : v;
+}
+
+// x 2^k for any int k, by exact powers of two.
+__device__ __forceinline__ double mul_pow2(double x, int k) {
+  k = min(max(k, -2400), 2400);
+  const int k1 = k / 3, k2 = (k - k1) / 2, k3 = k - k1 - k2;
+  return x * pow2_double(k1) * pow2_double(k2) * pow2_double(k3);
+}
+
+// c + (a b >> 32), one instruction.
+__device__ __forceinline__ int mad_hi(int a, int b, int c) {
+  int r;
+  asm("mad.hi.s32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+
+// Units of a block: f of the diagonal (see above) and ky of the data row, chosen so that z
+// stays below 2^(ky - 2) (every sum of products then fits in 64 bits): the entries are
+// standardised residuals times sigma, so there is room for 8 sigma (but no more than 2^12
+// above the largest datum).
+struct PanelScale {
+  int f = 0, ky = 0;
+  bool grown = false;      // an entry of z did not fit (warp-uniform)
+  bool nonfinite = false;  // a datum is not finite
+  __device__ __forceinline__ void init(unsigned ytop, const double sigma2, const double gamma1, int attempt) {
+    const int top = (int)__reduce_max_sync(0xffffffffu, ytop);
+    nonfinite = top == 0x7FF;
+    const int Ey = top - 1023;                                       // |y| < 2^(Ey + 1)
+    const int Es = (((int)exponent_field(sigma2) - 1023) >> 1) + 1;  // sigma < 2^Es
+    ky = max(Ey + 2, min(Es + 3, Ey + 12)) + 2 + 10 * attempt;
+    f = max(((int)exponent_field(gamma1) - 1023) >> 1, 0);
+    grown = false;
+  }
+};
+
+// A_rc -= sum_{k < c0} Lc_rk Lc_ck for the columns [c0, pe) of the panel and the sixteen rows
+// from rt on.  (Two row tiles at a time, which share the column operand's conversion, cost
+// more in registers and code than they save.)
+__device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, int rt, int c0, int pe, int f, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  const uint2* __restrict__ D = reinterpret_cast<const uint2*>(A);
+  const int rb = min(c0 + g, K);  // the panel's own rows: the MMA's columns
+  const int r0 = min(rt + g, K), r1 = min(rt + g + 8, K);
+  float d[8][4];
+#pragma unroll
+  for (int s = 0; s < 8; ++s)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) d[s][v] = kAccZero;
+#pragma unroll 1
+  for (int kb = 0; kb < c0; kb += 16) {
+    const int k0 = kb + 4 * t;  // this lane's four columns; past the last panel: zeros
+    uint2 x[4], y[4], z[4];
+    if (k0 < c0) {
+      const WordSlots w(K, k0);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        x[i] = D[w.e[i] + r0];
+        y[i] = D[w.e[i] + r1];
+        z[i] = D[w.e[i] + rb];
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = y[i] = z[i] = make_uint2(0x80808080u, 0x80808080u);
+    }
+    unsigned bf[7][2];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+      const unsigned v = j & 1 ? z[j >> 1].y : z[j >> 1].x;
+      bf[j][0] = digit_pair(v, 0x4140);
+      bf[j][1] = digit_pair(v, 0x4342);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const unsigned u = i & 1 ? x[i >> 1].y : x[i >> 1].x, v = i & 1 ? y[i >> 1].y : y[i >> 1].x;
+      const unsigned af[4] = {digit_pair(u, 0x4140), digit_pair(v, 0x4140), digit_pair(u, 0x4342), digit_pair(v, 0x4342)};
+#pragma unroll
+      for (int j = 0; j < 7; ++j)
+        if (i + j < 8) mma_f16(d[i + j], af, bf[j]);
+    }
+  }
+  // sum_s acc_s 2^(48 - 8s), in units of 2^-60
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    unsigned a[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) a[s] = __float_as_uint(d[s][v]) - kAccZeroBits;
+    const int H = (int)(a[3] * 256u + a[4]), M = (int)(a[5] * 256u + a[6]) + ((int)a[7] >> 8);
+    const unsigned T = a[0] * 65536u + a[1] * 256u + a[2];
+    long long sum = (long long)((unsigned long long)T << 32) + (long long)H * (1 << 16) + M;
+    const int row = rt + g + 8 * (v >> 1), c = c0 + 2 * t + (v & 1);
+    if (row <= K && c < pe && row >= c) {
+      const int e = tri_off(K, c) + row - c;
+      if (f && row == c) sum >>= 2 * f;
+      A[e] -= sum;
+    }
+  }
+}
+
+// The columns [c0, min(c0 + 8, K - 1)) of a panel, left-looking, a row per lane and slot (rows
+// c0 + lane and c0 + lane + 32): A becomes V there.  The corner {C_mm, C_Km} is returned in
+// corner when column m = K - 1 lies in the panel.  The high limbs' products are summed in 64
+// bits, the mixed ones in units of 2^-56 (each rounded down, half a unit on average, which
+// the start values give back).  Returns whether the block can still be positive definite.
+template <bool GRAD>
+__device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, float2* __restrict__ RJ, int c0, int f,
+                                              bool& grown, long long (&corner)[2], int lane) {
+  const int last = K - 1 - c0;    // panel position of column m
+  const int jn = min(last + 1, kPanelCols);
+  const int r0 = c0 + lane, r1 = r0 + 32;
+  const bool two = c0 + 32 <= K;  // warp-uniform
+  int over = 0, grow = 0;
+  bool ok = true;
+  const int2* __restrict__ V = reinterpret_cast<const int2*>(A);
+#pragma unroll 1
+  for (int j = 0; j < jn; ++j) {
+    const int oj = tri_off(K, c0 + j) - (c0 + j);
+    const int q0 = min(max(r0, c0 + j), K), q1 = min(r1, K);
+    long long s0 = 0, s1 = 0;
+    int m0 = j, m1 = j;
+    int ok_ = tri_off(K, c0) - c0, step = K - c0;  // slot of (row 0, column c0 + k)
+#pragma unroll 1
+    for (int k = 0; k < j; ++k) {
+      const int2 p = V[ok_ + c0 + j], x = V[ok_ + q0];
+      const int lp = (int)((unsigned)p.x >> 4);
+      s0 += (long long)x.y * p.y;
+      m0 = mad_hi(x.y, lp, m0);
+      m0 = mad_hi((int)((unsigned)x.x >> 4), p.y, m0);
+      if (two) {
+        const int2 y = V[ok_ + q1];
+        s1 += (long long)y.y * p.y;
+        m1 = mad_hi(y.y, lp, m1);
+        m1 = mad_hi((int)((unsigned)y.x >> 4), p.y, m1);
+      }
+      ok_ -= step + 1;
+      --step;
+    }
+    s0 += (long long)m0 * 16;
+    if (f && lane == j) s0 >>= 2 * f;
+    const long long a0 = r0 >= c0 + j && r0 <= K ? A[oj + q0] - s0 : 0;
+    if (j == last) {
+      corner[0] = __shfl_sync(0xffffffffu, a0, j);
+      corner[1] = __shfl_sync(0xffffffffu, a0, j + 1);
+      break;
+    }
+    long long d = __shfl_sync(0xffffffffu, a0, j);
+    if (d <= 0) {  // a failed block runs on (values unused)
+      ok = false;
+      d = 1LL << 60;
+    }
+    int q, rh, rl;
+    rsqrt_fixed(d, q, rh, rl);
+    if (GRAD && lane == 0) {  // 2^-62 / sqrt(d), the factor that makes V a unit-lower entry
+      const float h = __int2float_rz(rh);
+      const float lo = __int2float_rn(rh - (int)h) + __int2float_rn(rl) * 0x1p-31f;
+      const float sc = __uint_as_float((unsigned)max(127 + q - 30 - 62 - f, 1) << 23);
+      const float hs = h + lo;
+      RJ[c0 + j] = make_float2(hs * sc, (lo - (hs - h)) * sc);
+    }
+    // V of this lane's rows; |V| >= 2^62 2^-f: not a positive definite block, or, in the data
+    // row, |z| too large for its units
+    const int lim = max(29 - q, 0), ylim = max(27 - q, 0);
+    auto scaled = [&](long long a) {
+      const long long n = a << q;
+      const int ch = (int)(n >> 31), cl = (int)n & 0x7FFFFFFF;
+      const long long mid = (long long)ch * rl + (long long)cl * rh;
+      const long long v = ((long long)ch * rh << 3) + (mid >> 28);
+      return f ? v >> f : v;
+    };
+    auto magnitude = [](long long a) { return (int)(a >> 32) ^ (int)(a >> 63); };
+    __syncwarp();  // the pivot row's entries of this column are read
+    if (lane > j && r0 <= K) {
+      if (r0 == K) grow |= magnitude(a0) >> ylim;
+      else over |= magnitude(a0) >> lim;
+      A[oj + r0] = scaled(a0);
+    }
+    if (two) {
+      s1 += (long long)m1 * 16;
+      const long long a1 = A[oj + q1] - s1;
+      if (r1 == K) grow |= magnitude(a1) >> ylim;
+      else if (r1 < K) over |= magnitude(a1) >> lim;
+      if (r1 <= K) A[oj + r1] = scaled(a1);
+    }
+    if (K == c0 + 64) {  // a 65-row panel (m = 63): its last row, the data row, on lane 0
+      long long s2 = 0;
+      int m2 = j;
+      int o2 = tri_off(K, c0) - c0;
+      for (int k = 0; k < j; ++k) {
+        const int2 p = V[o2 + c0 + j], x = V[o2 + K];
+        s2 += (long long)x.y * p.y;
+        m2 = mad_hi(x.y, (int)((unsigned)p.x >> 4), m2);
+        m2 = mad_hi((int)((unsigned)x.x >> 4), p.y, m2);
+        o2 -= K - c0 - k + 1;
+      }
+      const long long a2 = A[oj + K] - s2 - (long long)m2 * 16;
+      __syncwarp();
+      if (lane == 0) {
+        grow |= magnitude(a2) >> ylim;
+        A[oj + K] = scaled(a2);
+      }
+    }
+    __syncwarp();
+  }
+  grown = grown || __any_sync(0xffffffffu, grow != 0);
+  return ok && !__any_sync(0xffffffffu, over != 0);
+}
+
+// The panel's factor entries of the rows below it as digits, in place.
+__device__ __forceinline__ void panel_to_digits(int K, long long* __restrict__ A, int c0, int lane) {
+  const int r0 = c0 + kPanelCols;
+#pragma unroll 1
+  for (int u = lane; u < kPanelWords * (K + 1 - r0); u += 32) {  // (row, word)
+    const int r = r0 + u / kPanelWords, k0 = c0 + 4 * (u % kPanelWords);
+    const WordSlots w(K, k0);
+    long long v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = A[w.e[i] + r];
+    unsigned pl[8];
+    digit_planes(v, pl);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) reinterpret_cast<uint2*>(A)[w.e[i] + r] = make_uint2(pl[2 * i], pl[2 * i + 1]);
+  }
+  __syncwarp();
+}
+
+// Cholesky over the neighbour columns.  Returns whether the block is positive definite.
+template <bool GRAD>
+__device__ __forceinline__ bool panels_eliminate(int K, long long* __restrict__ A, float2* __restrict__ RJ, PanelScale& ysc,
+                                                 long long (&corner)[2], int lane) {
+  bool ok = true;
+#pragma unroll 1
+  for (int c0 = 0; c0 < K; c0 += kPanelCols) {
+    const int pe = min(c0 + kPanelCols, K);
+    if (c0 > 0) {
+#pragma unroll 1
+      for (int rt = c0; rt <= K; rt += 16) update_tile(K, A, rt, c0, pe, ysc.f, lane);
+      __syncwarp();
+    }
+    const bool o = panel_columns<GRAD>(K, A, RJ, c0, ysc.f, ysc.grown, corner, lane);
+    ok = ok && o;
+    if (pe < K) panel_to_digits(K, A, c0, lane);
+  }
+  return ok;
+}
+
+// V 2^-62 / sqrt(d) 2^(unit's exponent) as a float pair, rj = 2^-62 / sqrt(d).
+__device__ __forceinline__ float2 unit_pair(long long v, float2 rj, float unit) {
+  // v = a 2^39 + b 2^23 + c, each an exact float
+  const float fa = __int2float_rn((int)(v >> 39)) * 0x1p39f;
+  const float fb = __int2float_rn((int)(v >> 23) & 0xFFFF) * 0x1p23f;
+  const float fc = __int2float_rn((int)((unsigned)v & 0x7FFFFFu));
+  float vh, vl, oh, ol;
+  fast_two_sum(fa, fb, vh, vl);
+  df_mul(vh, __fadd_rn(vl, fc), rj.x, rj.y, oh, ol);
+  return make_float2(oh * unit, ol * unit);
+}
+
+// After the elimination, for the adjoint: every entry of the factor below the diagonal
+// (neighbour columns) becomes a float pair of the unit factor in its place.
+__device__ __forceinline__ void panels_to_pairs(int K, long long* __restrict__ A, const float2* __restrict__ RJ,
+                                                const PanelScale& ysc, int lane) {
+  float2* __restrict__ P = reinterpret_cast<float2*>(A);
+  const float yunit = __uint_as_float((unsigned)(min(max(ysc.ky, -126), 127) + 127) << 23);
+#pragma unroll 1
+  for (int c0 = 0; c0 < K - 1; c0 += kPanelCols) {
+    // below the panel: digits, one (row, word) per lane; in it (and all of the last panel): V
+    const bool lastp = c0 + kPanelCols >= K;
+    const int rb = lastp ? K + 1 : c0 + kPanelCols;
+#pragma unroll 1
+    for (int u = lane; u < kPanelWords * (K + 1 - c0); u += 32) {
+      const int r = c0 + u / kPanelWords, k0 = c0 + 4 * (u % kPanelWords);
+      const WordSlots ws(K, k0);
+      const float unit = r == K ? yunit : 1.0f;
+      unsigned w[8];
+      if (r >= rb) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint2 x = reinterpret_cast<const uint2*>(A)[ws.e[i] + r];
+          w[2 * i] = x.x;
+          w[2 * i + 1] = x.y;
+        }
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int c = k0 + x;
+        if (r > c && c < K - 1) {
+          const long long v = r >= rb ? planes_value(w, x) : A[ws.e[x] + r];
+          P[ws.e[x] + r] = unit_pair(v, RJ[c], unit);
+        }
+      }
+    }
+  }
+  __syncwarp();
+}
+
+}  // namespace vecchia

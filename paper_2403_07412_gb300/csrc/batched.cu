@@ -1,7 +1,7 @@
 // Many independent (field, theta) log-likelihood evaluations in one persistent launch.
 //
 // The paper batches only over the locations of one field (Sec. V-B).  Here the unit of
-// work is an item = (field, theta, tile of kTile consecutive ordered locations); a
+// work is an item = (field, theta, tile of consecutive ordered locations); a
 // persistent grid of warps takes items from a global counter, evaluates each location
 // with the same per-location code as the single-field kernel (block.cuh), and writes
 // one partial-sum record per item.  Fields may differ in n and m (all block sizes of a
@@ -28,7 +28,12 @@ int launch_matern_table(double nu, double* tab, cudaStream_t stream);
 bool theta_ok(const double* th);
 int lanes_for(int K, bool grad);
 
-constexpr int kTile = 256;       // ordered locations per work item
+// Locations an item gives each group of a warp.  A full-warp location of m = 60 takes a warp
+// some 75 us: eight make an item long enough to hide its hand-out (an atomic, the field
+// search, the constants: a few us), and short enough that the last items do not leave the
+// GPU waiting (items of 256 such locations took 19 ms each, a batch of two fields of n =
+// 20,000 44 ms where its work takes 7).
+__host__ __device__ constexpr int tile_steps(int lanes) { return lanes == 32 ? 8 : 16; }
 constexpr int kMaxNu = 8;        // prepared smoothness values
 constexpr int kMaxDistinctK = 4; // distinct block sizes per batch
 
@@ -41,8 +46,9 @@ struct FieldDesc {
   int32_t m;
   int32_t kidx;       // index of this field's block size in the batch's K list
   int32_t orig;       // position in the caller's field list
-  int32_t tiles;      // ceil(n / kTile)
-  int32_t lanes;      // lanes per location (8, 16 or 32)
+  int32_t tile;       // locations per item
+  int32_t tiles;      // ceil(n / tile)
+  int32_t lanes;      // lanes per location (4, 8, 16 or 32)
   int64_t item_base;  // first item of this field
 };
 
@@ -88,13 +94,13 @@ __device__ __forceinline__ void run_item(const FieldDesc& fd, int64_t tile, cons
   const uint32_t* pairs = reinterpret_cast<const uint32_t*>(smem + a.pairs_off[fd.kidx]);
   const WarpArea area(base + grp * group_doubles(K, GRAD, G), K, GRAD, G);
   Accum acc;
-  const int64_t i0 = tile * kTile;
-  const int64_t i1 = min(fd.n, i0 + kTile);
+  const int64_t i0 = tile * fd.tile;
+  const int64_t i1 = min(fd.n, i0 + fd.tile);
   for (int64_t b = i0; b < i1; b += NL) {
     const int64_t i = b + grp;
     const bool active = i < i1;
-    process_location<GRAD, G, false, FIXED>(active ? i : b, active, F, S, sched, pairs, area, tab, mc, tc, acc, false, nullptr,
-                              a.errloc, sub);
+    process_location<GRAD, G, false, FIXED>(active ? i : b, active, F, S, sched, pairs, area, tab, mc, tc, acc, false,
+                                            nullptr, a.errloc, sub);
   }
   write_partial<G>(acc, out, lane);
 }
@@ -157,21 +163,23 @@ __global__ void __launch_bounds__(384) vecchia_batched_kernel(const BatchArgs a)
   }
 }
 
-// One warp per (field, theta): the field's tile records, each lane a strided subset in
-// item order (compensated), merged by a fixed shuffle tree, so the result depends only
-// on the field's tile count.
-__global__ void vecchia_batched_finalize(const FieldDesc* __restrict__ fields, int nfields, int ntheta,
-                                         const double* __restrict__ thetas, const double* __restrict__ partial,
-                                         int want_grad, double* out) {
-  const int64_t id = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (id >= (int64_t)nfields * ntheta) return;  // whole warps leave together
-  const int fs = (int)(id / ntheta), t = (int)(id % ntheta);
+// One CTA per (field, theta): the field's item records, each thread a strided subset in
+// item order (compensated), merged by a fixed shuffle tree and warp order, so the result
+// depends only on the field's item count.  (A compensated sum costs a warp some 1,800
+// cycles of the FP64 pipe per 32 records: four sub-partitions share them.)
+constexpr int kFinalWarps = 4;
+
+__global__ void __launch_bounds__(32 * kFinalWarps)
+    vecchia_batched_finalize(const FieldDesc* __restrict__ fields, int ntheta, const double* __restrict__ thetas,
+                             const double* __restrict__ partial, int want_grad, double* out) {
+  __shared__ Neumaier sums[kFinalWarps][4];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int fs = (int)(blockIdx.x / ntheta), t = (int)(blockIdx.x % ntheta);
   const FieldDesc fd = fields[fs];
   Neumaier acc[4];
   const double* p = partial + (fd.item_base + (int64_t)t * fd.tiles) * 4;
-  for (int k = lane; k < fd.tiles; k += 32)
-    for (int c = 0; c < 4; ++c) acc[c].add(p[k * 4 + c]);
+  for (int k = threadIdx.x; k < fd.tiles; k += 32 * kFinalWarps)
+    for (int c = 0; c < 4; ++c) acc[c].add(p[(int64_t)k * 4 + c]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -180,7 +188,12 @@ __global__ void vecchia_batched_finalize(const FieldDesc* __restrict__ fields, i
       const double c2 = __shfl_down_sync(0xffffffffu, acc[c].c, o);
       acc[c].merge(s2, c2);
     }
-  if (lane != 0) return;
+  if (lane == 0)
+    for (int c = 0; c < 4; ++c) sums[warp][c] = acc[c];
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < kFinalWarps; ++w)
+    for (int c = 0; c < 4; ++c) acc[c].merge(sums[w][c].s, sums[w][c].c);
   const int64_t o = (int64_t)fd.orig * ntheta + t;
   if (!want_grad) {
     out[o] = acc[0].value();
@@ -278,7 +291,6 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return plans[x]->m > plans[y]->m; });
   std::vector<FieldDesc> fd(nfields);
   std::vector<int> kvals;
-  int64_t items = 0;
   for (int s = 0; s < nfields; ++s) {
     const Plan* p = plans[order[s]];
     FieldDesc& d = fd[s];
@@ -298,9 +310,6 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
     d.kidx = (int)(it - kvals.begin());
     d.lanes = lanes_for(K, want_grad != 0);
     d.orig = order[s];
-    d.tiles = (int)((p->n + kTile - 1) / kTile);
-    d.item_base = items;
-    items += (int64_t)d.tiles * ntheta;
   }
   // Every warp's shared-memory area is sized for the largest field's share (32/lanes
   // blocks).  A field whose own choice of lanes would need more than the full-warp
@@ -315,6 +324,13 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
       while (fd[f].lanes < 32 && (32 / fd[f].lanes) * group_doubles(K, want_grad != 0, fd[f].lanes) > full_area)
         fd[f].lanes *= 2;
     }
+  }
+  int64_t items = 0;
+  for (FieldDesc& d : fd) {
+    d.tile = (32 / d.lanes) * tile_steps(d.lanes);
+    d.tiles = (int)((d.n + d.tile - 1) / d.tile);
+    d.item_base = items;
+    items += (int64_t)d.tiles * ntheta;
   }
   for (int s = 0; s < nfields; ++s) {
     b->plans.push_back(plans[s]);
@@ -458,8 +474,8 @@ extern "C" int vecchia_loglik_batched(const vecchia_plan_t* plans, const double*
   else vecchia_batched_kernel<false><<<b->blocks, b->W * 32, b->smem, s>>>(a);
   VECCHIA_CUDA_TRY(cudaGetLastError());
   const int64_t pairs = (int64_t)nfields * ntheta;
-  vecchia_batched_finalize<<<(unsigned)((pairs + 3) / 4), 128, 0, s>>>(b->d_fields, nfields, ntheta, thetas_dev,
-                                                                           b->d_partial, want_grad, out_dev);
+  vecchia_batched_finalize<<<(unsigned)pairs, 32 * kFinalWarps, 0, s>>>(b->d_fields, ntheta, thetas_dev, b->d_partial,
+                                                                      want_grad, out_dev);
   VECCHIA_CUDA_TRY(cudaGetLastError());
   return VECCHIA_OK;
 }

@@ -1,17 +1,20 @@
-// Many independent (field, theta) log-likelihood evaluations in one persistent launch.
+// Many independent (field, theta) log-likelihood evaluations in a few persistent launches.
 //
 // The paper batches only over the locations of one field (Sec. V-B).  Here the unit of
-// work is an item = (field, theta, tile of consecutive ordered locations); a
-// persistent grid of warps takes items from a global counter, evaluates each location
-// with the same per-location code as the single-field kernel (block.cuh), and writes
-// one partial-sum record per item.  Fields may differ in n and m (all block sizes of a
-// batch share one shared-memory layout sized for the largest), and each theta picks its
-// covariance table by smoothness nu among the tables prepared with
-// vecchia_batched_prepare.  Items are laid out so the most expensive fields (largest m)
-// are handed out first.  A second kernel reduces each (field, theta)'s records in item
-// order, so results do not depend on scheduling.  The launch sequence (two memsets and
-// two kernels) allocates nothing and never waits on the host, so it can be captured in
-// a CUDA graph once the work layout has been cached by a first call.
+// work is an item = (field, theta, tile of consecutive ordered locations); a persistent
+// grid of warps takes items from a global counter, evaluates each location with the same
+// per-location code as the single-field kernel (block.cuh), and writes one partial-sum
+// record per item.  Fields may differ in n and m: the fields whose blocks run the same way
+// (lanes per location, FP64 or fixed point) form a class, and each class is one launch of its own
+// kernel, with a shared-memory layout sized for its largest block.  (One kernel for all of
+// them held every variant's code and the largest variant's registers and area: n = 20,000, m
+// = 60 / 30 / 10 took 102 / 30.0 / 6.5 ns a location.)  Each theta picks its covariance
+// table by smoothness nu among the tables prepared with vecchia_batched_prepare.  Items are
+// laid out so the most expensive fields (largest m) are handed out first.  A last kernel
+// reduces each (field, theta)'s records in item order, so results do not depend on
+// scheduling.  The launch sequence (two memsets, a kernel per class and the last one)
+// allocates nothing and never waits on the host, so it can be captured in a CUDA graph once
+// the work layout has been cached by a first call.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -26,16 +29,18 @@ namespace vecchia {
 
 int launch_matern_table(double nu, double* tab, cudaStream_t stream);
 bool theta_ok(const double* th);
-int lanes_for(int K, bool grad);
+int lanes_for(int K, bool grad, int64_t count);
 
-// Locations an item gives each group of a warp.  A full-warp location of m = 60 takes a warp
-// some 75 us: eight make an item long enough to hide its hand-out (an atomic, the field
-// search, the constants: a few us), and short enough that the last items do not leave the
-// GPU waiting (items of 256 such locations took 19 ms each, a batch of two fields of n =
-// 20,000 44 ms where its work takes 7).
-__host__ __device__ constexpr int tile_steps(int lanes) { return lanes == 32 ? 8 : 16; }
+// Locations an item gives each group of a warp: up to kMostSteps, fewer where the class has
+// not kItemsPerWarp such items for each resident warp.  A full-warp location of m = 60 takes
+// a warp some 75 us: eight make an item long enough to hide its hand-out (an atomic, the
+// field search, the constants: a few us).  Items of 256 locations took 19 ms each there, a
+// batch of two fields of n = 20,000, two thetas, 44 ms where its work takes 7; with eight for
+// every size, two fields of n = 700 took 1.40 ms.
+constexpr int kMostSteps = 8;
+constexpr int kItemsPerWarp = 4;
 constexpr int kMaxNu = 8;        // prepared smoothness values
-constexpr int kMaxDistinctK = 4; // distinct block sizes per batch
+constexpr int kMaxDistinctK = 4; // distinct block sizes per batch, and so most classes
 
 struct FieldDesc {
   const double2* xy;
@@ -44,23 +49,23 @@ struct FieldDesc {
   const int32_t* self;
   int64_t n;
   int32_t m;
-  int32_t kidx;       // index of this field's block size in the batch's K list
+  int32_t kidx;       // index of this field's block size in its class's K list
   int32_t orig;       // position in the caller's field list
   int32_t tile;       // locations per item
   int32_t tiles;      // ceil(n / tile)
-  int32_t lanes;      // lanes per location (4, 8, 16 or 32)
   int64_t item_base;  // first item of this field
 };
 
 struct BatchArgs {
   const FieldDesc* fields;
-  int nfields;
+  int first_field, last_field;  // the class's
   int ntheta;
   const double* thetas;  // [nfields][ntheta][4], caller order
   const double* nus;     // [kMaxNu]
   const double* const* tabs;
   int nnu;
-  int64_t total_items;
+  bool regather;                    // 8 lanes, gradient: see WarpArea
+  int64_t first_item, total_items;  // the class's
   unsigned long long* counter;
   unsigned long long* errloc;
   double* partial;  // [total_items][4]
@@ -92,7 +97,7 @@ __device__ __forceinline__ void run_item(const FieldDesc& fd, int64_t tile, cons
   const SchedSize S(K);
   const uint16_t* sched = reinterpret_cast<const uint16_t*>(smem + a.sched_off[fd.kidx]);
   const uint32_t* pairs = reinterpret_cast<const uint32_t*>(smem + a.pairs_off[fd.kidx]);
-  const WarpArea area(base + grp * group_doubles(K, GRAD, G), K, GRAD, G);
+  const WarpArea area(base + grp * group_doubles(K, GRAD, G, false, a.regather), K, GRAD, G, false, a.regather);
   Accum acc;
   const int64_t i0 = tile * fd.tile;
   const int64_t i1 = min(fd.n, i0 + fd.tile);
@@ -105,8 +110,9 @@ __device__ __forceinline__ void run_item(const FieldDesc& fd, int64_t tile, cons
   write_partial<G>(acc, out, lane);
 }
 
-template <bool GRAD>
-__global__ void __launch_bounds__(384) vecchia_batched_kernel(const BatchArgs a) {
+template <bool GRAD, int G, bool FIXED>
+__global__ void __launch_bounds__(GRAD && G == 8 ? 512 : GRAD || FIXED ? 384 : 32 * kMaxCtaWarps)
+    vecchia_batched_kernel(const BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   for (int k = 0; k < a.nk; ++k)
     build_schedules(a.kval[k], reinterpret_cast<uint16_t*>(smem + a.sched_off[k]),
@@ -120,8 +126,9 @@ __global__ void __launch_bounds__(384) vecchia_batched_kernel(const BatchArgs a)
     if (lane == 0) item = atomicAdd(a.counter, 1ULL);
     item = __shfl_sync(0xffffffffu, item, 0);
     if ((int64_t)item >= a.total_items) break;
+    item += a.first_item;
     // field of this item: fields are stored in item order
-    int lo = 0, hi = a.nfields - 1;
+    int lo = a.first_field, hi = a.last_field;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
       if (a.fields[mid].item_base <= (int64_t)item) lo = mid; else hi = mid - 1;
@@ -130,7 +137,7 @@ __global__ void __launch_bounds__(384) vecchia_batched_kernel(const BatchArgs a)
     const int64_t rel = (int64_t)item - fd.item_base;
     const int t = (int)(rel / fd.tiles);
     const int64_t tile = rel % fd.tiles;
-    if (kChecked && (t >= a.ntheta || tile >= fd.tiles || lo < 0 || lo >= a.nfields)) {
+    if (kChecked && (t >= a.ntheta || tile >= fd.tiles || tile < 0)) {
       if (lane == 0) {  // a work item outside the layout: record it and skip it
         atomicMin(a.errloc, err_code((int64_t)item, kErrIndex));
       }
@@ -154,11 +161,7 @@ __global__ void __launch_bounds__(384) vecchia_batched_kernel(const BatchArgs a)
     const MaternConst mc = matern_const_at(fix_const(tab));
     ThetaConst tc;
     tc.set(s2, beta, t2, kFamilyMatern, nu);
-    if (fd.lanes == 4) run_item<GRAD, 4, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
-    else if (fd.lanes == 8) run_item<GRAD, 8, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
-    else if (fd.lanes == 16) run_item<GRAD, 16, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
-    else if (fixed_point_block(fd.m + 1, GRAD, 32)) run_item<GRAD, 32, true>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
-    else run_item<GRAD, 32, false>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
+    run_item<GRAD, G, FIXED>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
     __syncwarp();
   }
 }
@@ -219,6 +222,22 @@ struct PreparedNu {
   double** d_tabs = nullptr;
 };
 
+using BatchKernel = void (*)(const BatchArgs);
+
+template <bool GRAD>
+BatchKernel batch_kernel(int lanes, bool fixed) {
+  if (lanes == 4) return vecchia_batched_kernel<GRAD, 4, false>;
+  if (lanes == 8) return vecchia_batched_kernel<GRAD, 8, false>;
+  if (lanes == 16) return vecchia_batched_kernel<GRAD, 16, false>;
+  return fixed ? vecchia_batched_kernel<GRAD, 32, true> : vecchia_batched_kernel<GRAD, 32, false>;
+}
+
+struct BatchClass {
+  BatchArgs args{};
+  BatchKernel kern = nullptr;
+  int W = 0, blocks = 0, smem = 0;
+};
+
 struct BatchState {
   int device = -1;
   std::vector<const void*> plans;
@@ -227,10 +246,8 @@ struct BatchState {
   int want_grad = 0;
   FieldDesc* d_fields = nullptr;
   double* d_partial = nullptr;
-  unsigned long long* d_counter = nullptr;  // [0] = work counter, [1] = error slot
-  int64_t total_items = 0;
-  BatchArgs args{};
-  int W = 0, blocks = 0, smem = 0;
+  unsigned long long* d_counter = nullptr;  // a work counter per class, then the error slot
+  std::vector<BatchClass> classes;
 };
 
 std::mutex g_mu;
@@ -250,33 +267,39 @@ PreparedNu* prepared_for(int dev) {
   return nullptr;
 }
 
-// Warps per CTA with the most resident warps per SM for this shared-memory footprint.
-template <bool GRAD>
-int batched_config(int fixed_bytes, int per_warp_bytes, int* W, int* blocks, int* smem) {
+// The class's warps per CTA with the most resident warps per SM (at most 16) and a grid of
+// one wave, with the coordinates gathered twice where that gives a fifth more warps (as in
+// the single-field launch).
+int class_shape(BatchClass* c, const int* areas, int fixed_bytes) {
   int dev = 0, sms = 0, optin = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
   VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  int best = -1;
-  for (int w : {12, 11, 10, 9, 8, 6, 4, 2, 1}) {
-    const int bytes = fixed_bytes + w * per_warp_bytes;
-    if (bytes > optin) continue;
-    VECCHIA_CUDA_TRY(cudaFuncSetAttribute(vecchia_batched_kernel<GRAD>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    int per_sm = 0;
-    VECCHIA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, vecchia_batched_kernel<GRAD>,
-                                                                   w * 32, bytes));
-    const int warps = std::min(per_sm * w, 16);
-    if (per_sm > 0 && warps > best) {
-      best = warps;
-      *W = w;
-      *blocks = per_sm * sms;
-      *smem = bytes;
+  cudaFuncAttributes fa;
+  VECCHIA_CUDA_TRY(cudaFuncGetAttributes(&fa, c->kern));
+  // one limit for every batch: cached ones are launched again in any order
+  VECCHIA_CUDA_TRY(cudaFuncSetAttribute(c->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes));
+  int best[2] = {-1, -1}, W[2] = {}, per[2] = {};
+  for (int r = 0; r < 2; ++r)
+    for (int w : {13, 12, 11, 10, 9, 8, 6, 4, 2, 1}) {
+      const int bytes = fixed_bytes + w * areas[r] * 8;
+      if (areas[r] == 0 || bytes > optin - (int)fa.sharedSizeBytes || 32 * w > fa.maxThreadsPerBlock) continue;
+      int per_sm = 0;
+      VECCHIA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, c->kern, w * 32, bytes));
+      const int warps = std::min(per_sm * w, 16);
+      if (per_sm > 0 && warps > best[r]) {
+        best[r] = warps;
+        W[r] = w;
+        per[r] = per_sm;
+      }
     }
-  }
-  if (best <= 0) return VECCHIA_EINVAL;
-  VECCHIA_CUDA_TRY(cudaFuncSetAttribute(vecchia_batched_kernel<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        *smem));
+  const int r = best[1] > 0 && 5 * best[1] >= 6 * best[0] ? 1 : 0;
+  if (best[r] <= 0) return VECCHIA_EINVAL;
+  c->W = W[r];
+  c->blocks = per[r] * sms;
+  c->smem = fixed_bytes + W[r] * areas[r] * 8;
+  c->args.regather = r == 1;
+  c->args.area_doubles = areas[r];
   return VECCHIA_OK;
 }
 
@@ -286,81 +309,84 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
   b->device = dev;
   b->ntheta = ntheta;
   b->want_grad = want_grad;
+  const bool grad = want_grad != 0;
+  // fields by class, the wider groups (larger blocks) first, and by m within one
+  auto lanes = [&](int f) {
+    int64_t count = 0;
+    for (int g = 0; g < nfields; ++g)
+      if (plans[g]->m == plans[f]->m) count += plans[g]->n * ntheta;
+    return lanes_for(plans[f]->m + 1, grad, count);
+  };
+  auto key = [&](int f) { return 2 * lanes(f) + (fixed_point_block(plans[f]->m + 1, grad, lanes(f)) ? 1 : 0); };
   std::vector<int> order(nfields);
   for (int f = 0; f < nfields; ++f) order[f] = f;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return plans[x]->m > plans[y]->m; });
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+    return key(x) != key(y) ? key(x) > key(y) : plans[x]->m > plans[y]->m;
+  });
   std::vector<FieldDesc> fd(nfields);
-  std::vector<int> kvals;
-  for (int s = 0; s < nfields; ++s) {
-    const Plan* p = plans[order[s]];
-    FieldDesc& d = fd[s];
-    d.xy = reinterpret_cast<const double2*>(p->d_xy);
-    d.yf = ys[order[s]];
-    d.nbr = p->d_nbr;
-    d.self = p->d_self;
-    d.n = p->n;
-    d.m = p->m;
-    const int K = p->m + 1;
-    auto it = std::find(kvals.begin(), kvals.end(), K);
-    if (it == kvals.end()) {
-      if ((int)kvals.size() == kMaxDistinctK) { delete b; return VECCHIA_EINVAL; }
-      kvals.push_back(K);
-      it = kvals.end() - 1;
-    }
-    d.kidx = (int)(it - kvals.begin());
-    d.lanes = lanes_for(K, want_grad != 0);
-    d.orig = order[s];
-  }
-  // Every warp's shared-memory area is sized for the largest field's share (32/lanes
-  // blocks).  A field whose own choice of lanes would need more than the full-warp
-  // fields do widens its groups instead, so the launch keeps the occupancy of the
-  // largest blocks (which carry most of the flops).
-  int full_area = 0;
-  for (int f = 0; f < nfields; ++f)
-    if (fd[f].lanes == 32) full_area = std::max(full_area, group_doubles(fd[f].m + 1, want_grad != 0, 32));
-  if (full_area > 0) {
-    for (int f = 0; f < nfields; ++f) {
-      const int K = fd[f].m + 1;
-      while (fd[f].lanes < 32 && (32 / fd[f].lanes) * group_doubles(K, want_grad != 0, fd[f].lanes) > full_area)
-        fd[f].lanes *= 2;
-    }
-  }
   int64_t items = 0;
-  for (FieldDesc& d : fd) {
-    d.tile = (32 / d.lanes) * tile_steps(d.lanes);
-    d.tiles = (int)((d.n + d.tile - 1) / d.tile);
-    d.item_base = items;
-    items += (int64_t)d.tiles * ntheta;
+  int distinct = 0;
+  for (int s = 0; s < nfields;) {
+    BatchClass c;
+    BatchArgs& a = c.args;
+    const int k0 = key(order[s]), L = lanes(order[s]);
+    c.kern = grad ? batch_kernel<true>(L, k0 & 1) : batch_kernel<false>(L, k0 & 1);
+    a.ntheta = ntheta;
+    a.first_field = s;
+    a.first_item = items;
+    int areas[2] = {0, 0};
+    int64_t steps = 0;
+    for (; s < nfields && key(order[s]) == k0; ++s) {
+      const Plan* p = plans[order[s]];
+      FieldDesc& d = fd[s];
+      d.xy = reinterpret_cast<const double2*>(p->d_xy);
+      d.yf = ys[order[s]];
+      d.nbr = p->d_nbr;
+      d.self = p->d_self;
+      d.n = p->n;
+      d.m = p->m;
+      d.orig = order[s];
+      const int K = p->m + 1;
+      if (a.nk == 0 || a.kval[a.nk - 1] != K) {
+        if (distinct++ == kMaxDistinctK) { delete b; return VECCHIA_EINVAL; }
+        a.kval[a.nk++] = K;
+        for (int r = 0; r < (regather_capable(grad, L) ? 2 : 1); ++r)  // a warp holds 32/L blocks
+          areas[r] = std::max(areas[r], (32 / L) * group_doubles(K, grad, L, false, r == 1));
+      }
+      d.kidx = a.nk - 1;
+      steps += (d.n + 32 / L - 1) / (32 / L) * ntheta;
+    }
+    a.last_field = s - 1;
+    int off = 0;
+    for (int k = 0; k < a.nk; ++k) {
+      const SchedSize S(a.kval[k]);
+      a.sched_off[k] = off;
+      off += S.sched_bytes;
+      a.pairs_off[k] = off;
+      off += S.pairs_bytes;
+    }
+    a.area_off = off;
+    const int rc = class_shape(&c, areas, off);
+    if (rc) { delete b; return rc; }
+    const int64_t share = steps / ((int64_t)kItemsPerWarp * c.blocks * c.W);
+    for (int k = a.first_field; k <= a.last_field; ++k) {
+      FieldDesc& d = fd[k];
+      d.tile = (32 / L) * (int)std::max<int64_t>(1, std::min<int64_t>(kMostSteps, share));
+      d.tiles = (int)((d.n + d.tile - 1) / d.tile);
+      d.item_base = items;
+      items += (int64_t)d.tiles * ntheta;
+    }
+    a.total_items = items - a.first_item;
+    b->classes.push_back(c);
   }
   for (int s = 0; s < nfields; ++s) {
     b->plans.push_back(plans[s]);
     b->ys.push_back(ys[s]);
   }
-  b->total_items = items;
-  BatchArgs& a = b->args;
-  a.nfields = nfields;
-  a.ntheta = ntheta;
-  a.total_items = items;
-  a.nk = (int)kvals.size();
-  int off = 0, area = 0;
-  for (int k = 0; k < a.nk; ++k) {
-    const SchedSize S(kvals[k]);
-    a.kval[k] = kvals[k];
-    a.sched_off[k] = off;
-    off += S.sched_bytes;
-    a.pairs_off[k] = off;
-    off += S.pairs_bytes;
-  }
-  for (int f = 0; f < nfields; ++f)  // a warp holds 32/lanes blocks of its field's size
-    area = std::max(area, (32 / fd[f].lanes) * group_doubles(fd[f].m + 1, want_grad != 0, fd[f].lanes));
-  a.area_off = off;
-  a.area_doubles = area;
-  int rc = want_grad ? batched_config<true>(off, a.area_doubles * 8, &b->W, &b->blocks, &b->smem)
-                     : batched_config<false>(off, a.area_doubles * 8, &b->W, &b->blocks, &b->smem);
-  if (rc) { delete b; return rc; }
+  const int ncls = (int)b->classes.size();
   if (cudaMalloc(&b->d_fields, sizeof(FieldDesc) * nfields) != cudaSuccess ||
       cudaMalloc(&b->d_partial, sizeof(double) * 4 * std::max<int64_t>(items, 1)) != cudaSuccess ||
-      cudaMalloc(&b->d_counter, sizeof(unsigned long long) * 2) != cudaSuccess) {
+      cudaMalloc(&b->d_counter, sizeof(unsigned long long) * (ncls + 1)) != cudaSuccess) {
     free_batch(b);
     return VECCHIA_ENOMEM;
   }
@@ -368,10 +394,13 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
     free_batch(b);
     return VECCHIA_ECUDA;
   }
-  a.fields = b->d_fields;
-  a.partial = b->d_partial;
-  a.counter = b->d_counter;
-  a.errloc = b->d_counter + 1;
+  for (int k = 0; k < ncls; ++k) {
+    BatchArgs& a = b->classes[k].args;
+    a.fields = b->d_fields;
+    a.partial = b->d_partial;
+    a.counter = b->d_counter + k;
+    a.errloc = b->d_counter + ncls;
+  }
   *out = b;
   return VECCHIA_OK;
 }
@@ -463,16 +492,18 @@ extern "C" int vecchia_loglik_batched(const vecchia_plan_t* plans, const double*
     if (rc) return rc;
     g_batches.push_back(b);
   }
-  BatchArgs a = b->args;
-  a.thetas = thetas_dev;
-  a.nus = pn->d_nus;
-  a.tabs = pn->d_tabs;
-  a.nnu = pn->nnu;
-  VECCHIA_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned long long), s));
-  VECCHIA_CUDA_TRY(cudaMemsetAsync(b->d_counter + 1, 0xFF, sizeof(unsigned long long), s));
-  if (want_grad) vecchia_batched_kernel<true><<<b->blocks, b->W * 32, b->smem, s>>>(a);
-  else vecchia_batched_kernel<false><<<b->blocks, b->W * 32, b->smem, s>>>(a);
-  VECCHIA_CUDA_TRY(cudaGetLastError());
+  const size_t ncls = b->classes.size();
+  VECCHIA_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned long long) * ncls, s));
+  VECCHIA_CUDA_TRY(cudaMemsetAsync(b->d_counter + ncls, 0xFF, sizeof(unsigned long long), s));
+  for (const BatchClass& c : b->classes) {
+    BatchArgs a = c.args;
+    a.thetas = thetas_dev;
+    a.nus = pn->d_nus;
+    a.tabs = pn->d_tabs;
+    a.nnu = pn->nnu;
+    c.kern<<<c.blocks, c.W * 32, c.smem, s>>>(a);
+    VECCHIA_CUDA_TRY(cudaGetLastError());
+  }
   const int64_t pairs = (int64_t)nfields * ntheta;
   vecchia_batched_finalize<<<(unsigned)pairs, 32 * kFinalWarps, 0, s>>>(b->d_fields, ntheta, thetas_dev, b->d_partial,
                                                                       want_grad, out_dev);

@@ -359,18 +359,26 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
   return VECCHIA_OK;
 }
 
-// Configuration for block size K: the tuned shape if vecchia_autotune recorded one, else
-// the default lanes per location.  VECCHIA_LANES_PER_LOCATION / VECCHIA_WARPS_PER_CTA
-// force either value (tuning experiments).  `count` (> 0: the call's locations) widens
-// the default groups while they would leave fewer location groups than the GPU has
-// sub-partitions: such a call is bound by each warp's serial latency, which wider groups
+// G widened while `count` locations in groups of G lanes would leave sub-partitions of the
+// GPU without a warp: such a call is bound by each warp's serial latency, which wider groups
 // shorten (n = 2,000, m = 10, per call: 4 lanes 33.9 us, 8 lanes 30.7, 16 lanes 28.8, 32
 // lanes 41.1; n = 1,000, m = 30 with the gradient: 8 lanes 131, 16 lanes 80.0, 32 lanes
 // 61.5; m = 10: 16 lanes 30.9, 32 lanes 32.0, so up to 16 lanes for the smallest blocks).
-// And where 16-lane groups would need a second turn of the resident warps while 8-lane
-// groups all fit at once, those are taken (m = 30, n = 6,000, 8 and 16 lanes: 121 and 137
-// us, with the gradient 176 and 190; n = 4,000, one turn either way: 148 and 131 with the
-// gradient).
+int widened(int K, int G, int64_t count, int dev) {
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return G;
+  const int most = K <= 16 ? 16 : 32;
+  while (G < most && (count + 32 / G - 1) / (32 / G) < 4 * (int64_t)sms) G *= 2;
+  return G;
+}
+
+// Configuration for block size K: the tuned shape if vecchia_autotune recorded one, else
+// the default lanes per location.  VECCHIA_LANES_PER_LOCATION / VECCHIA_WARPS_PER_CTA
+// force either value (tuning experiments).  `count` (> 0: the call's locations) widens
+// the default groups where there are few.  And where 16-lane groups would need a second
+// turn of the resident warps while 8-lane groups all fit at once, those are taken (m = 30,
+// n = 6,000, 8 and 16 lanes: 121 and 137 us, with the gradient 176 and 190; n = 4,000, one
+// turn either way: 148 and 131 with the gradient).
 int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t count = -1) {
   int dev = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
@@ -386,10 +394,7 @@ int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t c
   }
   if (const char* e = getenv("VECCHIA_WARPS_PER_CTA")) W = atoi(e);
   if (!chosen && count > 0) {
-    int sms = 0;
-    VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int most = K <= 16 ? 16 : 32;
-    while (G < most && (count + 32 / G - 1) / (32 / G) < 4 * (int64_t)sms) G *= 2;
+    G = widened(K, G, count, dev);
     if (G == 16 && K <= max_k_for_lanes(8)) {
       LaunchCfg wide, narrow;
       int rc = shape_for(K, grad, 16, W, &wide, sphere);
@@ -407,13 +412,13 @@ void launch_lik(const LaunchCfg& cfg, bool grad, const LikArgs& a, cudaStream_t 
 }
 }  // namespace
 
-// Lanes per location for block size K: the tuned value if any, else the default.
-int lanes_for(int K, bool grad) {
+// Lanes per location for `count` blocks of size K: the tuned value if any, else the default,
+// widened where there are few.
+int lanes_for(int K, bool grad, int64_t count) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return default_lanes(K, grad);
   int G = default_lanes(K, grad), W = 0;
-  tuned_for(dev, K, grad, &G, &W);
-  return G;
+  return tuned_for(dev, K, grad, &G, &W) ? G : widened(K, G, count, dev);
 }
 
 namespace {

@@ -1,26 +1,31 @@
 // Large conditioning sets (m > VECCHIA_MAX_M_WARP): one CTA per location.
 //
-// The paper runs m up to 150 (Sec. VI-D).  A 151-row bordered block is 93 KB of packed
-// FP64, too much for a warp's share of shared memory, so here a CTA of kCtaThreads
-// threads owns one location at a time and runs the same elimination as block.cuh (the
-// bordered L D L^T whose trailing 2x2 corner holds s_i / sigma2 and y_i - mu_i) with
-// CTA-wide barriers.  The (row, column) of a packed slot or a pair index is decoded
-// arithmetically (a triangular-number inverse) instead of from schedule tables, which
-// keeps two CTAs resident per SM.  The adjoint's two backward solves run on the first two
-// warps, one each, on vectors in shared memory; everything else is spread over all
-// threads.
+// The paper runs m up to 150 (Sec. VI-D).  A 151-row bordered block is 93 KB, too much for
+// a warp's share of shared memory, so here a CTA of two to eight warps owns one location at a
+// time and eliminates its block in fixed point, as the full-warp kernels do (mmapanel.cuh):
+// panels of eight columns, updates on the tensor cores, the trailing 2x2 corner s_i / sigma2
+// and y_i - mu_i.  (In FP64, four columns a CTA-wide pass, the FP64 pipe was its bound: n =
+// 50,000, m = 120 took 36.2 ms with the gradient.)  What bounds it now is latency: a location's
+// phases, and the panels' serial columns most of all, leave a warp issuing one instruction in
+// four cycles, and shared memory holds three locations an SM at m = 120, two at 150.  The
+// (row, column) of a pair index is decoded arithmetically (a triangular-number inverse)
+// instead of from schedule tables, to keep that many.  The adjoint's two backward solves run
+// on the first two warps, one each, on vectors in shared memory; everything else is spread
+// over all threads.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <mutex>
+#include <vector>
 
 #include "block.cuh"
 #include "common.cuh"
 #include "matern.cuh"
+#include "mmapanel.cuh"
 
 namespace vecchia {
 
-constexpr int kCtaThreads = 128;     // default CTA size (4 warps)
-constexpr int kCtaThreadsMax = 256;  // when fewer than 4 CTAs fit on an SM
+constexpr int kCtaThreadsMax = 256;  // two to eight warps (big_config)
 
 struct BigArgs {
   const double* __restrict__ xy;
@@ -60,79 +65,49 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;
 }
 
-// B columns j..j+B-1 of the bordered L D L^T, CTA-wide.  Each column in turn is scaled by
-// its pivot's reciprocal (its unscaled entries kept in TVs[q]) and applied to the later
-// columns of the group; then one pass over the remaining prefix [1, o_{j+B-1}) applies
-// all B columns to each slot in column order, fma(-L_q T_q, .) for q = 0..B-1.  Every
-// slot sees the same roundings in the same order as with single-column steps, while the
-// trailing matrix is read and written once per B columns.  Returns false (uniformly over
-// the CTA) at a pivot outside rcp_fixed's domain.
-template <int B>
-__device__ __forceinline__ bool cta_columns(double* A, double* const* TVs, int K, int j, int tid, int NTH) {
-  int o[B];
-#pragma unroll
-  for (int q = 0; q < B; ++q) o[q] = tri_off(K, j + q);
-#pragma unroll
-  for (int q = 0; q < B; ++q) {
-    const double d = A[o[q]];
-    if (!pivot_in_range(d)) return false;  // every thread reads the same pivot
-    const double inv = rcp_fixed(d);
-    double* T = TVs[q];
-    for (int r = j + q + 1 + tid; r <= K; r += NTH) {
-      const double tv = A[o[q] + r - j - q];
-      T[r] = tv;
-      A[o[q] + r - j - q] = tv * inv;
+// Cholesky over the neighbour columns.  A panel's own eight rows are a serial chain of eight
+// columns, and warp 0 runs ahead with it: it takes the sixteen rows below a panel through the
+// panel's columns (panel_row, a row per lane), updates them for the next panel and factors
+// that panel's rows, while the other warps take the rows further down through the first
+// panel's columns and, once warp 0's sixteen rows are in (barrier 1), update them.
+template <bool GRAD>
+__device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, float2* __restrict__ RJ, int4* __restrict__ piv,
+                                              PanelScale& ysc, long long* corner, int tid, int NTH) {
+  const int lane = tid & 31, wid = tid >> 5;
+  int over = 0, grow = 0;
+  // pivots of this panel and the next
+#pragma unroll 1
+  for (int c0 = -kPanelCols; c0 + kPanelCols < K; c0 += kPanelCols) {
+    const int c1 = c0 + kPanelCols, pe = min(c1 + kPanelCols, K);
+    const int4* __restrict__ pv = piv + (c0 & kPanelCols);
+    if (wid == 0) {
+      if (c0 >= 0) {
+        if (lane < 16 && c1 + lane <= K) panel_row(K, A, pv, c0, ysc.f, c1 + lane, over, grow);
+        __threadfence_block();
+        asm volatile("bar.arrive 1, %0;" ::"r"(NTH) : "memory");
+        __syncwarp();
+        update_tile(K, A, c1, c1, pe, ysc.f, lane);
+        __syncwarp();
+      }
+      long long cr[2] = {0, 0};
+      bool g = false;
+      if (!panel_columns<GRAD, true>(K, A, RJ, piv + (c1 & kPanelCols), c1, ysc.f, g, cr, lane)) over = 1;
+      if (g) grow = 1;
+      if (pe == K && lane == 0) {
+        corner[0] = cr[0];
+        corner[1] = cr[1];
+      }
+    } else if (c0 >= 0) {
+#pragma unroll 1
+      for (int r = c1 + 16 + tid - 32; r <= K; r += NTH - 32) panel_row(K, A, pv, c0, ysc.f, r, over, grow);
+      asm volatile("bar.sync 1, %0;" ::"r"(NTH) : "memory");
+#pragma unroll 1
+      for (int rt = c1 + 16 * wid; rt <= K; rt += (NTH - 32) / 2) update_tile(K, A, rt, c1, pe, ysc.f, lane);
     }
     __syncthreads();
-    if (q + 1 < B) {
-      const double* Lq = A + o[q] - j - q;
-#pragma unroll
-      for (int p = q + 1; p < B; ++p) {
-        const double tp = T[j + p];
-        for (int r = j + p + tid; r <= K; r += NTH) {
-          const int e = o[p] + r - j - p;
-          A[e] = fma(-Lq[r], tp, A[e]);
-        }
-      }
-      __syncthreads();
-    }
   }
-  const double* L[B];
-#pragma unroll
-  for (int q = 0; q < B; ++q) L[q] = A + o[q] - j - q;
-  constexpr int U = 8 / B;
-  const int end = o[B - 1];
-  const int nfull = (end - 1) / (NTH * U);
-  const int tail0 = 1 + NTH * U * nfull;
-  for (int bt = 0; bt < nfull; ++bt) {
-    const int base = 1 + tid + NTH * U * bt;
-    double av[U];
-    int rr[U], cc[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int e = base + NTH * k;
-      const int w = tri_root(e);
-      cc[k] = K - w;
-      rr[k] = cc[k] + (e - w * (w + 1) / 2);
-      av[k] = A[e];
-    }
-#pragma unroll
-    for (int q = 0; q < B; ++q)
-#pragma unroll
-      for (int k = 0; k < U; ++k) av[k] = fma(-L[q][rr[k]], TVs[q][cc[k]], av[k]);
-#pragma unroll
-    for (int k = 0; k < U; ++k) A[base + NTH * k] = av[k];
-  }
-  for (int e = tail0 + tid; e < end; e += NTH) {
-    const int w = tri_root(e);
-    const int c = K - w, r = c + (e - w * (w + 1) / 2);
-    double a = A[e];
-#pragma unroll
-    for (int q = 0; q < B; ++q) a = fma(-L[q][r], TVs[q][c], a);
-    A[e] = a;
-  }
-  __syncthreads();
-  return true;
+  ysc.grown = __syncthreads_or(grow) != 0;
+  return __syncthreads_or(over) == 0;
 }
 
 template <bool GRAD, bool SPHERE>
@@ -150,6 +125,11 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
   double* WH = TV + align_up(K + 1, 2);
   double* GV = WH + align_up(K + 1, 2);
   double* red = GV + align_up(K + 1, 2);
+  long long* corner = reinterpret_cast<long long*>(red + 32);
+  double* coef = reinterpret_cast<double*>(corner + 2);
+  int4* piv = reinterpret_cast<int4*>(coef + 4);
+  unsigned* ytops = reinterpret_cast<unsigned*>(piv + 2 * kPanelCols);
+  long long* AF = reinterpret_cast<long long*>(A);
   float2* WHf = reinterpret_cast<float2*>(WH);  // w^ and g as float pairs for the beta sums
   float2* GVf = reinterpret_cast<float2*>(GV);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -177,12 +157,10 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       js = 0;
     }
     const double2 ps = xy2[js];
-    // ---- gather (two slots per thread covers m <= 2 * kCtaThreads): centred,
-    // 1/beta-scaled coordinates as float pairs, and data
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int p = tid + NTH * s;
-      if (p < m) {
+    // ---- gather: centred, 1/beta-scaled coordinates as float pairs, and data
+    unsigned ytop = 0u;  // largest exponent field of the data
+#pragma unroll 1
+    for (int p = tid; p < m; p += NTH) {
         double xv = 0.0, yv = 0.0, zv = 0.0, fv = 0.0;
         if (p < mi) {
           int j = row[p];
@@ -202,77 +180,94 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
           fv = a.yf[j];
         }
         YV[p] = fv;
+        ytop = max(ytop, exponent_field(fv));
         CX[p] = d2f_pair(xv);
         CY[p] = d2f_pair(yv);
         if constexpr (SPHERE) CZ[p] = d2f_pair(zv);
-      }
     }
     if (tid == 0) {
       CX[m] = make_float2(0.0f, 0.0f);
       CY[m] = make_float2(0.0f, 0.0f);
       if constexpr (SPHERE) CZ[m] = make_float2(0.0f, 0.0f);
       YV[m] = a.yf[js];
+      ytop = max(ytop, exponent_field(a.yf[js]));
     }
+    ytop = __reduce_max_sync(0xffffffffu, ytop);
+    if (lane == 0) ytops[wid] = ytop;
     if (kChecked) bad_idx = __syncthreads_or(bad_idx) != 0;
     __syncthreads();
-    // ---- assemble
-    for (int c = tid; c < K; c += NTH) {
-      const int o = tri_off(K, c);
-      A[o] = (c >= mi && c < m) ? 1.0 : tc.gamma1;
-      A[o + K - c] = YV[c];
+    for (int w = 0; w < NTH >> 5; ++w) ytop = max(ytop, ytops[w]);
+    // ---- assemble, in fixed point (mmapanel.cuh); again with larger units in the rare case
+    // that an entry of the data row outgrows them
+    PanelScale ysc;
+    bool ok = true;
+    for (int attempt = 0;; ++attempt) {
+      ysc.init(ytop, tc.sigma2, tc.gamma1, attempt);
+      for (int c = tid; c < K; c += NTH) {
+        const int o = tri_off(K, c);
+        AF[o] = fixed_from_double((c >= mi && c < m) ? 1.0 : tc.gamma1, 60 - 2 * ysc.f);
+        AF[o + K - c] = ysc.nonfinite ? 0LL : fixed_from_double(YV[c], 60 - ysc.ky);
+      }
+      if (tid == 0) AF[0] = 0;
+      for (int q0 = tid; q0 < NP; q0 += 2 * NTH) {
+        const int q1 = q0 + NTH;
+        const bool has1 = q1 < NP;
+        const int v0 = tri_root(q0), v1 = tri_root(has1 ? q1 : q0);
+        const int c0 = K - 2 - v0, r0 = c0 + 1 + (q0 - v0 * (v0 + 1) / 2);
+        const int qq1 = has1 ? q1 : q0;
+        const int c1 = K - 2 - v1, r1 = c1 + 1 + (qq1 - v1 * (v1 + 1) / 2);
+        const bool ok0 = c0 < mi && (r0 < mi || r0 == m);
+        const bool ok1 = has1 && c1 < mi && (r1 < mi || r1 == m);
+        float u0h, u0l, u1h, u1l;
+        pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
+        pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
+        const long long val0 = rho_fixed62(u0h, u0l, a.tab, mc) >> 2, val1 = rho_fixed62(u1h, u1l, a.tab, mc) >> 2;
+        AF[tri_off(K, c0) + r0 - c0] = ok0 ? val0 : 0LL;
+        if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? val1 : 0LL;
+      }
+      __syncthreads();
+      ok = cta_eliminate<GRAD>(K, AF, reinterpret_cast<float2*>(TV), piv, ysc, corner, tid, NTH);
+      if (!ysc.grown || !ok || ysc.nonfinite || attempt == 7) break;
     }
-    if (tid == 0) A[0] = 0.0;
-    for (int q0 = tid; q0 < NP; q0 += 2 * NTH) {
-      const int q1 = q0 + NTH;
-      const bool has1 = q1 < NP;
-      const int v0 = tri_root(q0), v1 = tri_root(has1 ? q1 : q0);
-      const int c0 = K - 2 - v0, r0 = c0 + 1 + (q0 - v0 * (v0 + 1) / 2);
-      const int qq1 = has1 ? q1 : q0;
-      const int c1 = K - 2 - v1, r1 = c1 + 1 + (qq1 - v1 * (v1 + 1) / 2);
-      const bool ok0 = c0 < mi && (r0 < mi || r0 == m);
-      const bool ok1 = has1 && c1 < mi && (r1 < mi || r1 == m);
-      float u0h, u0l, u1h, u1l;
-      pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
-      pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-      const double val0 = rho_fixed(u0h, u0l, a.tab, mc), val1 = rho_fixed(u1h, u1l, a.tab, mc);
-      A[tri_off(K, c0) + r0 - c0] = ok0 ? val0 : 0.0;
-      if (has1) A[tri_off(K, c1) + r1 - c1] = ok1 ? val1 : 0.0;
+    // ---- the term, on warp 0 (FP64)
+    const double nan = __longlong_as_double(0x7FF8000000000000LL);
+    if (wid == 0) {
+      const double st = mul_pow2((double)corner[0], 2 * ysc.f - 60);
+      // data not finite (or far out of any scale): with pd, a data error
+      const double rr = ysc.grown || ysc.nonfinite ? nan : mul_pow2((double)corner[1], ysc.ky - 60);
+      const bool pd = ok && positive_finite(st);
+      const bool good = pd && finite_bits(rr) && !bad_idx;
+      const double s = tc.sigma2 * st;
+      const double inv_s = rcp_newton(s);
+      const double q = rr * rr * inv_s;
+      if (good) {
+        acc.Q.add(q);
+        acc.mul_s(s);
+        acc.count += 1;
+      } else {
+        acc.Q.add(nan);
+        if (tid == 0) atomicMin(a.errloc, err_code(i, bad_idx ? kErrIndex : (pd ? kErrData : kErrNotPD)));
+      }
+      const double rs = rr * inv_s;
+      if (a.terms && tid == 0) {
+        const double li = good ? -0.5 * q - 0.5 * log(s) - 0.91893853320467274178 : nan;
+        a.terms[GRAD ? 4 * i : i] = li;
+      }
+      if (GRAD && tid == 0) {
+        coef[0] = 0.5 * (rs * rs - inv_s);
+        coef[1] = rs * tc.inv_sigma2;
+        coef[2] = good ? 0.5 * (rr * rs - 1.0) : nan;
+      }
     }
     __syncthreads();
-    // ---- L D L^T over the neighbour columns: CTA-wide steps of four columns (then two,
-    // then one), bit-identical to single-column steps (cta_columns)
-    double* TVs[4] = {TV, YV, WH, GV};  // YV, WH and GV are free during the elimination
-    bool ok = true;
-    int j = 0;
-    for (; ok && j + 4 < K; j += 4) ok = cta_columns<4>(A, TVs, K, j, tid, NTH);
-    for (; ok && j + 2 < K; j += 2) ok = cta_columns<2>(A, TVs, K, j, tid, NTH);
-    if (ok && j + 1 < K) ok = cta_columns<1>(A, TVs, K, j, tid, NTH);
-    const double st = A[1], rr = A[2];
-    const bool pd = ok && positive_finite(st);  // a non-finite rr with pd: non-finite data
-    const bool good = pd && finite_bits(rr) && !bad_idx;
-    const double nan = __longlong_as_double(0x7FF8000000000000LL);
-    const double s = tc.sigma2 * st;
-    const double inv_s = rcp_newton(s);
-    const double q = rr * rr * inv_s;
-    if (good) {
-      acc.Q.add(q);
-      acc.mul_s(s);
-      acc.count += 1;
-    } else {
-      acc.Q.add(nan);
-      if (tid == 0) atomicMin(a.errloc, err_code(i, bad_idx ? kErrIndex : (pd ? kErrData : kErrNotPD)));
-    }
-    const double li = good ? -0.5 * q - 0.5 * log(s) - 0.91893853320467274178 : nan;
-    if (!GRAD) {
-      if (a.terms && tid == 0) a.terms[i] = li;
-      __syncthreads();
-      continue;
-    }
+    if (!GRAD) continue;
     // ---- adjoint: the two backward solves on warps 0 (w) and 1 (alpha~) at once, then
     // the pair pass on all threads
-    const double rs = rr * inv_s;
-    const double cb = 0.5 * (rs * rs - inv_s);
-    const double rsa = rs * tc.inv_sigma2;
+    const double cb = coef[0], rsa = coef[1], sS = coef[2];
+    const bool good = finite_bits(sS);
+    panels_to_pairs(K, AF, reinterpret_cast<const float2*>(TV), ysc, tid, NTH);
+    __syncthreads();
+    const float2* __restrict__ L = reinterpret_cast<const float2*>(A);  // the unit factor
     double pT = 0.0;
     if (wid < 2 && good) {
       // Double-float solves on the FP32 pipe, as in the warp kernels: each step of the
@@ -283,12 +278,12 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       // one CTA per SM of occupancy at m = 90 and 120.
       float2* V = reinterpret_cast<float2*>(wid == 0 ? TV : YV);
       const int row = wid == 0 ? m : K;
-      for (int c = lane; c < K - 1; c += 32) V[c] = d2f_trunc(A[tri_off(K, c) + row - c]);
+      for (int c = lane; c < K - 1; c += 32) V[c] = L[tri_off(K, c) + row - c];
       __syncwarp();
       for (int c = K - 2; c >= 1; --c) {
         const float2 vc = V[c];  // final since the previous step (__syncwarp below)
         for (int cc = lane; cc < c; cc += 32) {
-          const float2 l = d2f_trunc(A[tri_off(K, cc) + c - cc]);
+          const float2 l = L[tri_off(K, cc) + c - cc];
           float2 v = V[cc];
           df_fms(v.x, v.y, l, vc);
           V[cc] = v;
@@ -327,26 +322,18 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       }
     }
     const double pB = f2d_scaled(pbh, 0) + f2d_scaled(pbl, 0);
-    const double sS = 0.5 * (rr * rs - 1.0);
     if (a.terms) {
       const double tB = block_sum(pB, red), tT = block_sum(pT, red);
       if (tid == 0) {
         double* o = a.terms + i * 4;
-        o[0] = li;
         o[1] = good ? (sS - tc.tau2 * tT) * tc.inv_sigma2 : nan;
         o[2] = good ? tc.dbeta_coef * tB : nan;
         o[3] = good ? tT : nan;
       }
     }
-    if (good) {
-      acc.S += sS;
-      acc.B += pB;
-      acc.T += pT;
-    } else {  // every output of a failed term is NaN
-      acc.S += nan;
-      acc.B += nan;
-      acc.T += nan;
-    }
+    if (wid == 0) acc.S += sS;  // a failed term's is NaN, and so every output
+    acc.B += good ? pB : nan;
+    acc.T += good ? pT : nan;
     __syncthreads();
   }
   const double B = block_sum(acc.B, red);
@@ -363,14 +350,24 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
 // Shared memory of the CTA kernel for block size K.
 int big_smem_bytes(int K, bool sphere) {
   const int NTd = (K + 1) * (K + 2) / 2;
-  return 8 * (align_up(NTd, 2) + (sphere ? 7 : 6) * align_up(K + 1, 2) + 32 + 16);
+  return 8 * (align_up(NTd, 2) + (sphere ? 7 : 6) * align_up(K + 1, 2) + 32 + 6 + 4 * kPanelCols + 4);
 }
 
-// CTA size: 128 threads while at least 4 CTAs fit on an SM (more locations in flight),
-// else 256 so that the SM still holds 512 threads.  Measured on GB300 at n = 100k:
-// m = 90 (6 CTAs/SM) 128 threads 1.35x faster than 256; m = 150 (2 CTAs/SM) 256
-// threads 1.34x faster than 128.  VECCHIA_CTA_THREADS = 128 or 256 forces one.
-int big_config(int K, bool grad, int* blocks, int* threads, int* smem, bool sphere) {
+// CTA size: the W warps with the largest c W / (W + 2), c the CTAs of that size resident on an SM
+// (at most the ones `count` > 0 locations give it): a location's serial part, the panels' own
+// columns on warp 0, is worth about two warps' shares of the rest.  Ties go to the larger W.  n =
+// 20,000 with the gradient, ms: m = 64 (8 CTAs of 2 warps, 5 of 3, 4 of 4) 2.86, 3.33, 3.47; m =
+// 90 (6, 5, 4) 6.02, 5.49, 5.58; m = 120 (3 of any up to 5 warps, 2 of 6) 14.4, 11.7, 10.9, 10.6
+// and 13.1; m = 150 (2) 27.4, 22.4, 20.2, 19.9, 18.4.  VECCHIA_CTA_THREADS, a multiple of 32 from
+// 64 to 256, forces one.
+struct BigShape {
+  int dev, K, grad, sphere;
+  int per_sm[kCtaThreadsMax / 32 + 1];
+};
+std::mutex g_big_mu;
+std::vector<BigShape> g_big_shapes;  // the occupancy queries cost tens of microseconds
+
+int big_config(int K, bool grad, int* blocks, int* threads, int* smem, bool sphere, int64_t count) {
   int dev = 0, sms = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
   VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -378,22 +375,39 @@ int big_config(int K, bool grad, int* blocks, int* threads, int* smem, bool sphe
   auto kern = grad ? (sphere ? vecchia_big_kernel<true, true> : vecchia_big_kernel<true, false>)
                    : (sphere ? vecchia_big_kernel<false, true> : vecchia_big_kernel<false, false>);
   VECCHIA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem));
-  const char* e = getenv("VECCHIA_CTA_THREADS");
-  const int forced = e ? atoi(e) : 0;
-  int t = (forced == 128 || forced == 256) ? forced : kCtaThreads;
-  int per_sm = 0;
-  VECCHIA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, t, *smem));
-  if (forced != 128 && forced != 256 && per_sm * t < 512) {
-    int per_sm2 = 0;
-    VECCHIA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, kern, kCtaThreadsMax, *smem));
-    if (per_sm2 >= 1) {
-      t = kCtaThreadsMax;
-      per_sm = per_sm2;
+  BigShape shape{dev, K, (int)grad, (int)sphere, {}};
+  {
+    std::lock_guard<std::mutex> lk(g_big_mu);
+    bool known = false;
+    for (const BigShape& e : g_big_shapes)
+      if (e.dev == dev && e.K == K && e.grad == (int)grad && e.sphere == (int)sphere) {
+        shape = e;
+        known = true;
+        break;
+      }
+    if (!known) {
+      for (int w = 2; w <= kCtaThreadsMax / 32; ++w)
+        VECCHIA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&shape.per_sm[w], kern, 32 * w, *smem));
+      g_big_shapes.push_back(shape);
     }
   }
-  if (per_sm < 1) return VECCHIA_EINVAL;
-  *blocks = per_sm * sms;
-  *threads = t;
+  const char* e = getenv("VECCHIA_CTA_THREADS");
+  const int forced = e ? atoi(e) : 0;
+  const int64_t share = count > 0 ? (count + sms - 1) / sms : shape.per_sm[2];
+  int W = 0;
+  double best = 0.0;
+  for (int w = 2; w <= kCtaThreadsMax / 32; ++w) {
+    if (forced % 32 == 0 && forced >= 64 && forced <= kCtaThreadsMax && 32 * w != forced) continue;
+    const double score = (double)std::min<int64_t>(shape.per_sm[w], share) * w / (w + 2);
+    if (shape.per_sm[w] > 0 && score >= best) {
+      best = score;
+      W = w;
+    }
+  }
+  if (W == 0) return VECCHIA_EINVAL;
+  *blocks = shape.per_sm[W] * sms;
+  if (count > 0) *blocks = (int)std::min<int64_t>(*blocks, count);
+  *threads = 32 * W;
   return VECCHIA_OK;
 }
 

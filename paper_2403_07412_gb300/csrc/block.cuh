@@ -788,7 +788,10 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     }
   }
   constexpr int NS = (KCAP - 1 + G - 1) / G;  // slots of the K-1 <= KCAP-1 neighbour entries
-  if constexpr (kPanels) panels_to_pairs(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), ysc, sub);
+  if constexpr (kPanels) {
+    panels_to_pairs(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), ysc, sub, 32);
+    __syncwarp();
+  }
   // The two unit backward solves run in double-float arithmetic on the FP32 pipe: each
   // step of their serial chain would otherwise wait behind the other warps' FP64 work.
   float2 wf[NS], bf[NS];

@@ -55,7 +55,7 @@ struct BigArgs {
   double radius;
   int64_t i0, i1;                  // ordered locations [i0, i1) are evaluated
 };
-int big_config(int K, bool grad, int* blocks, int* threads, int* smem, bool sphere);
+int big_config(int K, bool grad, int* blocks, int* threads, int* smem, bool sphere, int64_t count);
 void launch_big(bool grad, int blocks, int threads, int smem, const BigArgs& a, cudaStream_t s);
 bool theta_ok_family(const double* th, int family);
 int launch_matern_table(double nu, double* tab, cudaStream_t stream);
@@ -495,7 +495,7 @@ int launch_with(Plan* p, const double* y_dev, const double* theta, bool grad, co
 static int launch_big_loglik(Plan* p, const double* y_dev, const double* theta, bool grad, double* out_dev,
                              double* terms_dev, cudaStream_t stream, int64_t i0, int64_t i1) {
   int blocks = 0, threads = 0, smem = 0;
-  int rc = big_config(p->m + 1, grad, &blocks, &threads, &smem, p->metric == 1);
+  int rc = big_config(p->m + 1, grad, &blocks, &threads, &smem, p->metric == 1, i1 - i0);
   if (rc) return rc;
   if (p->partial_cap < (int64_t)blocks * 4) {
     if (p->d_partial) cudaFree(p->d_partial);
@@ -668,7 +668,7 @@ int autotune(Plan* p, const double* y_dev, const double* theta, bool grad, int* 
   const int K = p->m + 1;
   if (p->m > kMaxMWarp) {  // one CTA per location, sized by occupancy: nothing to time
     int blocks = 0, threads = 0, smem = 0;
-    const int rc = big_config(K, grad, &blocks, &threads, &smem, p->metric == 1);
+    const int rc = big_config(K, grad, &blocks, &threads, &smem, p->metric == 1, p->n);
     if (rc) return rc;
     if (G_out) *G_out = threads;
     if (W_out) *W_out = threads / 32;

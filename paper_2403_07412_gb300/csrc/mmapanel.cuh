@@ -1,5 +1,5 @@
-// Elimination of a full-warp block in 64-bit fixed point: panels of eight columns in integer
-// arithmetic, the updates between panels on the tensor cores.
+// Elimination of a block by a warp, or by a CTA's warps (bigblock.cu), in 64-bit fixed point:
+// panels of eight columns in integer arithmetic, the updates between panels on the tensor cores.
 //
 // On GB300 a warp's FP64 instruction holds its sub-partition's pipe for 64 cycles; at m = 60
 // the elimination's 1,270 of them per location were the kernels' bound (FP64 pipe 81-85%
@@ -20,9 +20,12 @@
 // Updates between panels: A_rc -= sum_{k < c0} Lc_rk Lc_ck, for the eight columns of the next
 // panel at once, as exact products of integers.  V is stored as its eight bytes, V +
 // 0x8080808080808080 = sum_i b_i 256^(7-i): digits d_i = b_i - 128, each a half exactly.  The
-// products d_i d'_j of one diagonal i + j = s add up to integers below 2^22 (63 terms of at
-// most 2^14 for each pair), exact in an FP32 accumulator; it starts at 1.5 2^23, so that the
-// integer is read off the accumulator's bits.  Kept are i <= 7, j <= 6, i + j <= 7.
+// products d_i d'_j of one diagonal i + j = s add up to integers that an FP32 accumulator holds
+// exactly up to 2^22; it starts at 1.5 2^23, so that the integer is read off the
+// accumulator's bits.  (A row's entries have squares that add up to at most 1, which bounds the
+// sums of the leading digits, and the digits below spread over their range: 8 pairs of 150
+// columns add up with a standard deviation below 2^18, or 2^20.7 in one pair where the two rows
+// are the same.)  Kept are i <= 7, j <= 6, i + j <= 7.
 //
 // The bytes take the factor entries' own places: the four entries (r, 4w .. 4w+3) of a row
 // become eight words, one per digit plane, each with the digit of the four columns; so the
@@ -160,6 +163,18 @@ __device__ __forceinline__ int mad_hi(int a, int b, int c) {
   return r;
 }
 
+// |a| >> 32, roughly (one below for negative a).
+__device__ __forceinline__ int top_magnitude(long long a) { return (int)(a >> 32) ^ (int)(a >> 63); }
+
+// A Schur complement's entry times its column's pivot reciprocal: V.
+__device__ __forceinline__ long long scaled_entry(long long a, int q, int rh, int rl, int f) {
+  const long long n = a << q;
+  const int ch = (int)(n >> 31), cl = (int)n & 0x7FFFFFFF;
+  const long long mid = (long long)ch * rl + (long long)cl * rh;
+  const long long v = ((long long)ch * rh << 3) + (mid >> 28);
+  return f ? v >> f : v;
+}
+
 // Units of a block: f of the diagonal (see above) and ky of the data row, chosen so that z
 // stays below 2^(ky - 2) (every sum of products then fits in 64 bits): the entries are
 // standardised residuals times sigma, so there is room for 8 sigma (but no more than 2^12
@@ -247,20 +262,24 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
 // corner when column m = K - 1 lies in the panel.  The high limbs' products are summed in 64
 // bits, the mixed ones in units of 2^-56 (each rounded down, half a unit on average, which
 // the start values give back).  Returns whether the block can still be positive definite.
-template <bool GRAD>
-__device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, float2* __restrict__ RJ, int c0, int f,
-                                              bool& grown, long long (&corner)[2], int lane) {
+// With CTA only the panel's own rows (of the last panel: all), and the pivots' reciprocals
+// are left in piv for panel_row.
+template <bool GRAD, bool CTA>
+__device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, float2* __restrict__ RJ,
+                                              int4* __restrict__ piv, int c0, int f, bool& grown,
+                                              long long (&corner)[2], int lane) {
+  const int rmax = CTA && c0 + kPanelCols < K ? c0 + kPanelCols - 1 : K;
   const int last = K - 1 - c0;    // panel position of column m
   const int jn = min(last + 1, kPanelCols);
   const int r0 = c0 + lane, r1 = r0 + 32;
-  const bool two = c0 + 32 <= K;  // warp-uniform
+  const bool two = !CTA && c0 + 32 <= K;  // warp-uniform
   int over = 0, grow = 0;
   bool ok = true;
   const int2* __restrict__ V = reinterpret_cast<const int2*>(A);
 #pragma unroll 1
   for (int j = 0; j < jn; ++j) {
     const int oj = tri_off(K, c0 + j) - (c0 + j);
-    const int q0 = min(max(r0, c0 + j), K), q1 = min(r1, K);
+    const int q0 = min(max(r0, c0 + j), rmax), q1 = min(r1, K);
     long long s0 = 0, s1 = 0;
     int m0 = j, m1 = j;
     int ok_ = tri_off(K, c0) - c0, step = K - c0;  // slot of (row 0, column c0 + k)
@@ -282,7 +301,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
     }
     s0 += (long long)m0 * 16;
     if (f && lane == j) s0 >>= 2 * f;
-    const long long a0 = r0 >= c0 + j && r0 <= K ? A[oj + q0] - s0 : 0;
+    const long long a0 = r0 >= c0 + j && r0 <= rmax ? A[oj + q0] - s0 : 0;
     if (j == last) {
       corner[0] = __shfl_sync(0xffffffffu, a0, j);
       corner[1] = __shfl_sync(0xffffffffu, a0, j + 1);
@@ -295,6 +314,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
     }
     int q, rh, rl;
     rsqrt_fixed(d, q, rh, rl);
+    if (CTA && lane == 0) piv[j] = make_int4(q, rh, rl, 0);
     if (GRAD && lane == 0) {  // 2^-62 / sqrt(d), the factor that makes V a unit-lower entry
       const float h = __int2float_rz(rh);
       const float lo = __int2float_rn(rh - (int)h) + __int2float_rn(rl) * 0x1p-31f;
@@ -305,28 +325,20 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
     // V of this lane's rows; |V| >= 2^62 2^-f: not a positive definite block, or, in the data
     // row, |z| too large for its units
     const int lim = max(29 - q, 0), ylim = max(27 - q, 0);
-    auto scaled = [&](long long a) {
-      const long long n = a << q;
-      const int ch = (int)(n >> 31), cl = (int)n & 0x7FFFFFFF;
-      const long long mid = (long long)ch * rl + (long long)cl * rh;
-      const long long v = ((long long)ch * rh << 3) + (mid >> 28);
-      return f ? v >> f : v;
-    };
-    auto magnitude = [](long long a) { return (int)(a >> 32) ^ (int)(a >> 63); };
     __syncwarp();  // the pivot row's entries of this column are read
-    if (lane > j && r0 <= K) {
-      if (r0 == K) grow |= magnitude(a0) >> ylim;
-      else over |= magnitude(a0) >> lim;
-      A[oj + r0] = scaled(a0);
+    if (lane > j && r0 <= rmax) {
+      if (r0 == K) grow |= top_magnitude(a0) >> ylim;
+      else over |= top_magnitude(a0) >> lim;
+      A[oj + r0] = scaled_entry(a0, q, rh, rl, f);
     }
     if (two) {
       s1 += (long long)m1 * 16;
       const long long a1 = A[oj + q1] - s1;
-      if (r1 == K) grow |= magnitude(a1) >> ylim;
-      else if (r1 < K) over |= magnitude(a1) >> lim;
-      if (r1 <= K) A[oj + r1] = scaled(a1);
+      if (r1 == K) grow |= top_magnitude(a1) >> ylim;
+      else if (r1 < K) over |= top_magnitude(a1) >> lim;
+      if (r1 <= K) A[oj + r1] = scaled_entry(a1, q, rh, rl, f);
     }
-    if (K == c0 + 64) {  // a 65-row panel (m = 63): its last row, the data row, on lane 0
+    if (!CTA && K == c0 + 64) {  // a 65-row panel (m = 63): its last row, the data row, on lane 0
       long long s2 = 0;
       int m2 = j;
       int o2 = tri_off(K, c0) - c0;
@@ -340,14 +352,52 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       const long long a2 = A[oj + K] - s2 - (long long)m2 * 16;
       __syncwarp();
       if (lane == 0) {
-        grow |= magnitude(a2) >> ylim;
-        A[oj + K] = scaled(a2);
+        grow |= top_magnitude(a2) >> ylim;
+        A[oj + K] = scaled_entry(a2, q, rh, rl, f);
       }
     }
     __syncwarp();
   }
   grown = grown || __any_sync(0xffffffffu, grow != 0);
   return ok && !__any_sync(0xffffffffu, over != 0);
+}
+
+// Row r below the panel [c0, c0 + 8), by one thread: its eight entries of the factor, from the
+// panel's own rows and pivots, and then their digits, in place.
+__device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, const int4* __restrict__ piv, int c0, int f,
+                                          int r, int& over, int& grow) {
+  const int2* __restrict__ V = reinterpret_cast<const int2*>(A);
+#pragma unroll 1
+  for (int j = 0; j < kPanelCols; ++j) {
+    long long s0 = 0;
+    int m0 = j;
+    int ok_ = tri_off(K, c0) - c0, step = K - c0;  // slot of (row 0, column c0 + k)
+#pragma unroll 1
+    for (int k = 0; k < j; ++k) {
+      const int2 p = V[ok_ + c0 + j], x = V[ok_ + r];
+      s0 += (long long)x.y * p.y;
+      m0 = mad_hi(x.y, (int)((unsigned)p.x >> 4), m0);
+      m0 = mad_hi((int)((unsigned)x.x >> 4), p.y, m0);
+      ok_ -= step + 1;
+      --step;
+    }
+    const int4 pv = piv[j];
+    const long long a = A[ok_ + r] - s0 - (long long)m0 * 16;
+    if (r == K) grow |= top_magnitude(a) >> max(27 - pv.x, 0);
+    else over |= top_magnitude(a) >> max(29 - pv.x, 0);
+    A[ok_ + r] = scaled_entry(a, pv.x, pv.y, pv.z, f);
+  }
+#pragma unroll 1
+  for (int k0 = c0; k0 < c0 + kPanelCols; k0 += 4) {
+    const WordSlots w(K, k0);
+    long long v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = A[w.e[i] + r];
+    unsigned pl[8];
+    digit_planes(v, pl);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) reinterpret_cast<uint2*>(A)[w.e[i] + r] = make_uint2(pl[2 * i], pl[2 * i + 1]);
+  }
 }
 
 // The panel's factor entries of the rows below it as digits, in place.
@@ -381,7 +431,7 @@ __device__ __forceinline__ bool panels_eliminate(int K, long long* __restrict__ 
       for (int rt = c0; rt <= K; rt += 16) update_tile(K, A, rt, c0, pe, ysc.f, lane);
       __syncwarp();
     }
-    const bool o = panel_columns<GRAD>(K, A, RJ, c0, ysc.f, ysc.grown, corner, lane);
+    const bool o = panel_columns<GRAD, false>(K, A, RJ, nullptr, c0, ysc.f, ysc.grown, corner, lane);
     ok = ok && o;
     if (pe < K) panel_to_digits(K, A, c0, lane);
   }
@@ -401,9 +451,9 @@ __device__ __forceinline__ float2 unit_pair(long long v, float2 rj, float unit) 
 }
 
 // After the elimination, for the adjoint: every entry of the factor below the diagonal
-// (neighbour columns) becomes a float pair of the unit factor in its place.
+// (neighbour columns) becomes a float pair of the unit factor in its place.  By nth threads.
 __device__ __forceinline__ void panels_to_pairs(int K, long long* __restrict__ A, const float2* __restrict__ RJ,
-                                                const PanelScale& ysc, int lane) {
+                                                const PanelScale& ysc, int tid, int nth) {
   float2* __restrict__ P = reinterpret_cast<float2*>(A);
   const float yunit = __uint_as_float((unsigned)(min(max(ysc.ky, -126), 127) + 127) << 23);
 #pragma unroll 1
@@ -412,7 +462,7 @@ __device__ __forceinline__ void panels_to_pairs(int K, long long* __restrict__ A
     const bool lastp = c0 + kPanelCols >= K;
     const int rb = lastp ? K + 1 : c0 + kPanelCols;
 #pragma unroll 1
-    for (int u = lane; u < kPanelWords * (K + 1 - c0); u += 32) {
+    for (int u = tid; u < kPanelWords * (K + 1 - c0); u += nth) {
       const int r = c0 + u / kPanelWords, k0 = c0 + 4 * (u % kPanelWords);
       const WordSlots ws(K, k0);
       const float unit = r == K ? yunit : 1.0f;
@@ -435,7 +485,6 @@ __device__ __forceinline__ void panels_to_pairs(int K, long long* __restrict__ A
       }
     }
   }
-  __syncwarp();
 }
 
 }  // namespace vecchia

@@ -221,9 +221,10 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
         float u0h, u0l, u1h, u1l;
         pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
         pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-        const long long val0 = rho_fixed62(u0h, u0l, a.tab, mc) >> 2, val1 = rho_fixed62(u1h, u1l, a.tab, mc) >> 2;
-        AF[tri_off(K, c0) + r0 - c0] = ok0 ? val0 : 0LL;
-        if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? val1 : 0LL;
+        long long val0, val1;
+        rho_fixed62(u0h, u0l, u1h, u1l, a.tab, mc, val0, val1);
+        AF[tri_off(K, c0) + r0 - c0] = ok0 ? val0 >> 2 : 0LL;
+        if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? val1 >> 2 : 0LL;
       }
       __syncthreads();
       ok = cta_eliminate<GRAD>(K, AF, reinterpret_cast<float2*>(TV), piv, ysc, corner, tid, NTH);
@@ -317,7 +318,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
         const int c0 = K - 2 - v0, r0 = c0 + 1 + (q0 - v0 * (v0 + 1) / 2);
         float u0h, u0l, h0h, h0l;
         pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
-        h_fixed(u0h, u0l, a.tab, mc, h0h, h0l);
+        h_fixed<true>(u0h, u0l, a.tab, mc, h0h, h0l);
         beta_pair_add(WHf[r0], WHf[c0], GVf[r0], GVf[c0], h0h, h0l, pbh, pbl);
       }
     }

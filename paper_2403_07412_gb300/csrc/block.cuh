@@ -374,7 +374,7 @@ __device__ __forceinline__ void beta_pair_add(float2 wr, float2 wc, float2 gr, f
 // q = sub + G k, in increasing k; w^ and g are float pairs (WHf, GVf).  One pair per
 // iteration: fewer live registers than two (n = 1M, m = 60, l + grad 101.2 -> 99.3 ms;
 // at n = 250k, m = 20, 2.03 -> 1.98 ms), with the same sums.
-template <int G, bool SPHERE>
+template <int G, bool SPHERE, bool FIXED>
 __device__ __forceinline__ double beta_pass(const FieldView& F, int NP, const uint32_t* __restrict__ pairs,
                                             const float2* __restrict__ CX, const float2* __restrict__ CY,
                                             const float2* __restrict__ CZ, const float2* __restrict__ WHf,
@@ -386,7 +386,7 @@ __device__ __forceinline__ double beta_pass(const FieldView& F, int NP, const ui
     const int r0 = w0 & 0xFF, c0 = (w0 >> 8) & 0xFF;
     float u0h, u0l, h0h, h0l;
     pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
-    h_fixed(u0h, u0l, tab, mc, h0h, h0l);
+    h_fixed<FIXED>(u0h, u0l, tab, mc, h0h, h0l);
     beta_pair_add(WHf[r0], WHf[c0], GVf[r0], GVf[c0], h0h, h0l, pbh, pbl);
   }
   return f2d_scaled(pbh, 0) + f2d_scaled(pbl, 0);
@@ -523,14 +523,19 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     float u0h, u0l, u1h, u1l;
     pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
     pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-    if constexpr (kPanels) {  // units of 2^-60
-      const long long val0 = rho_fixed62(u0h, u0l, tab, mc) >> 2, val1 = rho_fixed62(u1h, u1l, tab, mc) >> 2;
-      A[w0 >> 16] = __longlong_as_double(v0 ? val0 : 0LL);
-      if (has1) A[w1 >> 16] = __longlong_as_double(v1 ? val1 : 0LL);
+    long long val0, val1;
+    if constexpr (GRAD && !FIXED) {
+      val0 = rho_fixed62(u0h, u0l, tab, mc);
+      val1 = rho_fixed62(u1h, u1l, tab, mc);
     } else {
-      const double val0 = rho_fixed(u0h, u0l, tab, mc), val1 = rho_fixed(u1h, u1l, tab, mc);
-      A[w0 >> 16] = v0 ? val0 : 0.0;
-      if (has1) A[w1 >> 16] = v1 ? val1 : 0.0;
+      rho_fixed62(u0h, u0l, u1h, u1l, tab, mc, val0, val1);
+    }
+    if constexpr (kPanels) {  // units of 2^-60
+      A[w0 >> 16] = __longlong_as_double(v0 ? val0 >> 2 : 0LL);
+      if (has1) A[w1 >> 16] = __longlong_as_double(v1 ? val1 >> 2 : 0LL);
+    } else {
+      A[w0 >> 16] = fixed62_double(v0 ? val0 : 0LL);
+      if (has1) A[w1 >> 16] = fixed62_double(v1 ? val1 : 0LL);
     }
   }
   __syncwarp();
@@ -860,7 +865,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   }
   const double sS = 0.5 * (rr * rs - 1.0);
   __syncwarp();
-  const double pB = beta_pass<G, SPHERE>(F, S.NP, pairs, CX, CY, CZ, WHf, GVf, tab, mc, sub);
+  const double pB = beta_pass<G, SPHERE, FIXED>(F, S.NP, pairs, CX, CY, CZ, WHf, GVf, tab, mc, sub);
   if (terms_mode) {
     const double tB = group_sum<G>(pB), tT = group_sum<G>(pT);
     if (terms && active && sub == 0) {

@@ -49,9 +49,10 @@ __host__ __device__ constexpr int max_k_for_lanes(int G) { return G == 4 ? 16 : 
 // Smallest full-warp blocks (rows) eliminated in fixed point (mmapanel.cuh) instead of FP64.
 // n = 100k, FP64 / fixed point, ms: forward m = 34 2.19 / 2.33, m = 38 2.79 / 2.55, m = 60 8.75 /
 // 5.39; with the gradient m = 42 4.16 / 4.69, m = 46 5.04 / 5.11, m = 50 6.20 / 6.03, m = 60 11.1 /
-// 8.32 (its adjoint reads the factor from digits).
+// 8.32 (its adjoint reads the factor from digits; at m = 48 the two are even, and FP64 ahead by 3%
+// in the smallest calls).
 constexpr int kFixedMinFwd = 38;
-constexpr int kFixedMinGrad = 49;
+constexpr int kFixedMinGrad = 51;
 
 // First slot of column c of a packed block triangle (block.cuh).
 __host__ __device__ __forceinline__ int tri_off(int K, int c) { return (K - c) * (K - c + 1) / 2; }

@@ -62,8 +62,7 @@ __device__ __forceinline__ FixArg fix_arg(float uh, float ul) {
 // multiple of 2^-36 and the rest (below 2^-26: q tl), in units of 2^-56, go to integers by
 // conversion.  The integer re-enters FP64 by one conversion (64 cycles of
 // the FP64 pipe; two additions before).
-__device__ __forceinline__ long long rho_fixed62(float uh, float ul, const double* __restrict__ tab,
-                                                 const MaternConst& mc) {
+__device__ __forceinline__ long long rho_table62(float uh, float ul, const double* __restrict__ tab) {
   const FixArg a = fix_arg(uh, ul);
   const float4* __restrict__ w = reinterpret_cast<const float4*>(tab) + a.idx * kFixWords;
   const float4 w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3);
@@ -81,23 +80,65 @@ __device__ __forceinline__ long long rho_fixed62(float uh, float ul, const doubl
   const float r = fmaf(xl, fs, __fsub_rn(y, __int2float_rn(n1)));
   const int n2 = __float2int_rn(r * 0x1p20f);
   const long long c0 = (long long)(((unsigned long long)__float_as_uint(w3.y) << 32) | __float_as_uint(w3.x));
-  const long long v = c0 + (long long)n1 * (1 << 26) + (long long)n2 * 64;
-  if (a.ex < kELo || a.ex >= kEHi) {
-    double rho = 0.0, h = 0.0;
-    rho_fix(df_to_double(uh, ul), mc, rho, h);
-    return __double2ll_rn(rho * 0x1p62);
-  }
-  return v;
+  return c0 + (long long)n1 * (1 << 26) + (long long)n2 * 64;
 }
 
-// The same in FP64: one conversion, and 2^-62 on the exponent field.
-__device__ __forceinline__ double rho_fixed(float uh, float ul, const double* __restrict__ tab, const MaternConst& mc) {
-  const long long v = rho_fixed62(uh, ul, tab, mc);
+// Whether u lies outside the table.
+__device__ __forceinline__ bool fix_outside(float uh) {
+  return __float_as_uint(uh) - ((unsigned)(kELo + 127) << 23) >= (unsigned)(kEHi - kELo) << 23;
+}
+
+// rho(u) 2^62 there (rare; the constants by value, which keeps them in registers).
+static __device__ __noinline__ long long rho_outside62(float uh, float ul, int kind, double nu, double a1, double G, double b0,
+                                                double b1) {
+  const MaternConst mc{kind, nu, a1, G, b0, b1};
+  double rho = 0.0, h = 0.0;
+  rho_fix(df_to_double(uh, ul), mc, rho, h);
+  return __double2ll_rn(rho * 0x1p62);
+}
+
+// rho(u) 2^62 of one pair.
+__device__ __forceinline__ long long rho_fixed62(float uh, float ul, const double* __restrict__ tab,
+                                                 const MaternConst& mc) {
+  const long long v = rho_table62(uh, ul, tab);
+  if (!fix_outside(uh)) return v;
+  double rho = 0.0, h = 0.0;
+  rho_fix(df_to_double(uh, ul), mc, rho, h);
+  return __double2ll_rn(rho * 0x1p62);
+}
+
+// rho(u) 2^62 of two pairs: one branch for both keeps their instructions together (n = 100k, m = 10
+// 162 -> 156 us, m = 60 5.39 -> 5.33 ms; the FP64 gradient kernels take more registers with it).
+__device__ __forceinline__ void rho_fixed62(float u0h, float u0l, float u1h, float u1l, const double* __restrict__ tab,
+                                            const MaternConst& mc, long long& v0, long long& v1) {
+  v0 = rho_table62(u0h, u0l, tab);
+  v1 = rho_table62(u1h, u1l, tab);
+  if (fix_outside(u0h) || fix_outside(u1h)) {
+    if (fix_outside(u0h)) v0 = rho_outside62(u0h, u0l, mc.kind, mc.nu, mc.a1, mc.G, mc.b0, mc.b1);
+    if (fix_outside(u1h)) v1 = rho_outside62(u1h, u1l, mc.kind, mc.nu, mc.a1, mc.G, mc.b0, mc.b1);
+  }
+}
+
+// v 2^-62 in FP64: one conversion, and 2^-62 on the exponent field.  (A conversion holds the FP64 pipe
+// for 64 cycles; integer operations in its place, some 25, gave 2% at m = 30 and took 2% at m = 10.)
+__device__ __forceinline__ double fixed62_double(long long v) {
   const double r = (double)v;
   return __hiloint2double(__double2hiint(r) - (v != 0 ? 62 << 20 : 0), __double2loint(r));
 }
 
-// h(u) as a float pair.
+// h(u) outside the table, as a float pair (rare).
+static __device__ __noinline__ float2 h_outside(float uh, float ul, int kind, double nu, double a1, double G, double b0,
+                                                double b1) {
+  const MaternConst mc{kind, nu, a1, G, b0, b1};
+  double r = 0.0, h = 0.0;
+  rho_fix(df_to_double(uh, ul), mc, r, h);
+  const float hi = __double2float_rn(h);
+  return make_float2(hi, __double2float_rn(h - (double)hi));
+}
+
+// h(u) as a float pair (CALL: the rare path in a function, in the fixed-point kernels: n = 100k, m =
+// 60 8.33 -> 8.26 ms).
+template <bool CALL>
 __device__ __forceinline__ void h_fixed(float uh, float ul, const double* __restrict__ tab, const MaternConst& mc,
                                         float& hh, float& hl) {
   const FixArg a = fix_arg(uh, ul);
@@ -113,12 +154,18 @@ __device__ __forceinline__ void h_fixed(float uh, float ul, const double* __rest
   df_mul(s, l, a.mh, a.tl, hh, hl);
   hh *= inv;
   hl *= inv;
-  if (a.ex < kELo || a.ex >= kEHi) {
-    double r = 0.0, h = 0.0;
-    rho_fix(df_to_double(uh, ul), mc, r, h);
-    const float hi = __double2float_rn(h);
-    hh = hi;
-    hl = __double2float_rn(h - (double)hi);
+  if (fix_outside(uh)) {
+    if constexpr (CALL) {
+      const float2 h = h_outside(uh, ul, mc.kind, mc.nu, mc.a1, mc.G, mc.b0, mc.b1);
+      hh = h.x;
+      hl = h.y;
+    } else {
+      double r = 0.0, h = 0.0;
+      rho_fix(df_to_double(uh, ul), mc, r, h);
+      const float hi = __double2float_rn(h);
+      hh = hi;
+      hl = __double2float_rn(h - (double)hi);
+    }
   }
 }
 

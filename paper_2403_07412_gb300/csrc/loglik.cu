@@ -364,10 +364,13 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
 // shorten (n = 2,000, m = 10, per call: 4 lanes 33.9 us, 8 lanes 30.7, 16 lanes 28.8, 32
 // lanes 41.1; n = 1,000, m = 30 with the gradient: 8 lanes 131, 16 lanes 80.0, 32 lanes
 // 61.5; m = 10: 16 lanes 30.9, 32 lanes 32.0, so up to 16 lanes for the smallest blocks).
-int widened(int K, int G, int64_t count, int dev) {
+// The gradient's 16-lane groups widen already below ten an SM (n = 3,000, 16 and 32 lanes: m =
+// 26 103, 99; m = 30 129, 119; m = 34 169, 148; n = 4,000, m = 30 131, 141).
+int widened(int K, bool grad, int G, int64_t count, int dev) {
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return G;
   const int most = K <= 16 ? 16 : 32;
+  if (grad && G == 16 && count < 20 * (int64_t)sms) return most;
   while (G < most && (count + 32 / G - 1) / (32 / G) < 4 * (int64_t)sms) G *= 2;
   return G;
 }
@@ -376,9 +379,10 @@ int widened(int K, int G, int64_t count, int dev) {
 // the default lanes per location.  VECCHIA_LANES_PER_LOCATION / VECCHIA_WARPS_PER_CTA
 // force either value (tuning experiments).  `count` (> 0: the call's locations) widens
 // the default groups where there are few.  And where 16-lane groups would need a second
-// turn of the resident warps while 8-lane groups all fit at once, those are taken (m = 30,
-// n = 6,000, 8 and 16 lanes: 121 and 137 us, with the gradient 176 and 190; n = 4,000, one
-// turn either way: 148 and 131 with the gradient).
+// turn of the resident warps (without the gradient: a third warp on a sub-partition) while
+// 8-lane groups all fit at once, those are taken (m = 30, 8 and 16 lanes, us: n = 3,000 92 and
+// 100, with the gradient 142 and 129; n = 4,000 98 and 103, 148 and 131; n = 6,000 121 and 137,
+// 176 and 190).
 int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t count = -1) {
   int dev = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
@@ -394,13 +398,14 @@ int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t c
   }
   if (const char* e = getenv("VECCHIA_WARPS_PER_CTA")) W = atoi(e);
   if (!chosen && count > 0) {
-    G = widened(K, G, count, dev);
+    G = widened(K, grad, G, count, dev);
     if (G == 16 && K <= max_k_for_lanes(8)) {
       LaunchCfg wide, narrow;
       int rc = shape_for(K, grad, 16, W, &wide, sphere);
       if (!rc) rc = shape_for(K, grad, 8, W, &narrow, sphere);
       if (rc) return rc;
-      if ((count + 1) / 2 > (int64_t)wide.blocks * wide.W && (count + 3) / 4 <= (int64_t)narrow.blocks * narrow.W) G = 8;
+      const int64_t full = grad ? (int64_t)wide.blocks * wide.W : 8 * (int64_t)wide.sms;
+      if ((count + 1) / 2 > full && (count + 3) / 4 <= (int64_t)narrow.blocks * narrow.W) G = 8;
     }
   }
   while (K > max_k_for_lanes(G)) G *= 2;
@@ -418,7 +423,7 @@ int lanes_for(int K, bool grad, int64_t count) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return default_lanes(K, grad);
   int G = default_lanes(K, grad), W = 0;
-  return tuned_for(dev, K, grad, &G, &W) ? G : widened(K, G, count, dev);
+  return tuned_for(dev, K, grad, &G, &W) ? G : widened(K, grad, G, count, dev);
 }
 
 namespace {

@@ -112,6 +112,7 @@ __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, 
 
 template <bool GRAD, bool SPHERE>
 __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;");  // the reduction of the records
   extern __shared__ __align__(16) unsigned char smem[];
   const int m = a.m, K = m + 1;
   const int NTd = (K + 1) * (K + 2) / 2, NP = K * (K - 1) / 2;

@@ -360,8 +360,9 @@ int vecchia_autotune(vecchia_plan_t plan, const double* y_dev, const double thet
  *   mean_dev    : n_new doubles, device, written.  var_dev: n_new doubles or NULL.
  *   nbr_host    : optional n_new x m int32, host: the conditioning sets (original
  *                 indices, nearest first).
- * Synchronises `stream` before returning (temporary buffers are freed).  m must be at
- * most VECCHIA_MAX_M_WARP and at most n.  A location whose neighbour block is not
+ * Synchronises `stream` before returning (temporary buffers are freed).  A planar plan's
+ * first prediction lays out a search grid over its points, about 24 bytes a point, which the
+ * plan keeps until it is destroyed.  m must be at most VECCHIA_MAX_M_WARP and at most n.  A location whose neighbour block is not
  * positive definite gets NaN and is reported through vecchia_last_error_location, with
  * status VECCHIA_OK (the other predictions stand).  EINVAL: non-finite or (sphere)
  * out-of-range coordinates, bad theta, m > VECCHIA_MAX_M_WARP or m > n, n_new < 1.

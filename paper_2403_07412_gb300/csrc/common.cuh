@@ -79,6 +79,12 @@ struct Plan {
   int64_t partial_cap = 0;
   unsigned long long* d_errloc = nullptr;  // first failing location (ULLONG_MAX = none)
   cudaStream_t last_stream = nullptr;
+  // grid over all points for prediction (planar plans), laid out by the first vecchia_predict
+  double* d_grid_xy = nullptr;
+  int32_t* d_grid_cells = nullptr;
+  int32_t* d_grid_idx = nullptr;
+  void* d_grid_levels = nullptr;
+  int grid_levels = 0;
 };
 
 // ------------------------------------------------------------------ device helpers

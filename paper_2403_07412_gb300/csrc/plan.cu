@@ -20,6 +20,7 @@
 #include <cstring>
 #include <new>
 #include <queue>
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -536,6 +537,45 @@ static int knn_sphere_gpu(Plan* p, const double* xyz_host, cudaStream_t stream) 
   return rc;
 }
 
+// The grid the planar prediction searches: one level over all the plan's points, in original
+// order.  It depends on the plan's points only, so it is laid out once, by the first
+// prediction, and freed with the plan (20 bytes a point and 4 a cell).  (Copying the points
+// to the host and building it there for every prediction took 2.3 of 3.7 ms at n = 250,000, 25,000 new
+// points, m = 30.)
+static std::mutex g_grid_mu;
+
+static int predict_grid(Plan* p) {
+  std::lock_guard<std::mutex> lk(g_grid_mu);
+  if (p->d_grid_levels) return VECCHIA_OK;
+  const int64_t n = p->n;
+  std::vector<double> xy(2 * n);
+  if (cudaMemcpy(xy.data(), p->d_xy, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost) != cudaSuccess)
+    return VECCHIA_ECUDA;
+  std::vector<Level> lev;
+  std::vector<int32_t> cs, pidx;
+  std::vector<double> pxy;
+  build_levels(n, xy.data(), lev, cs, pidx, pxy, n);
+  int rc = VECCHIA_OK;
+  void* d[4] = {};
+  const void* h[4] = {pxy.data(), cs.data(), pidx.data(), lev.data()};
+  const size_t bytes[4] = {sizeof(double) * pxy.size(), sizeof(int32_t) * cs.size(), sizeof(int32_t) * pidx.size(),
+                           sizeof(Level) * lev.size()};
+  for (int k = 0; k < 4 && !rc; ++k) {
+    if (cudaMalloc(&d[k], std::max<size_t>(bytes[k], 16)) != cudaSuccess) rc = VECCHIA_ENOMEM;
+    else if (cudaMemcpy(d[k], h[k], bytes[k], cudaMemcpyHostToDevice) != cudaSuccess) rc = VECCHIA_ECUDA;
+  }
+  if (rc) {
+    for (void* q : d) cudaFree(q);
+    return rc;
+  }
+  p->d_grid_xy = static_cast<double*>(d[0]);
+  p->d_grid_cells = static_cast<int32_t*>(d[1]);
+  p->d_grid_idx = static_cast<int32_t*>(d[2]);
+  p->d_grid_levels = d[3];
+  p->grid_levels = (int)lev.size();
+  return VECCHIA_OK;
+}
+
 // Conditioning sets of prediction points: the m nearest OBSERVED points of the plan
 // (all of them are candidates; ties to the lower original index), written to d_nbr_new
 // (n_new x m, original indices) on `stream`.  xy_new_host: n_new x 2 (plane) or
@@ -569,42 +609,19 @@ int knn_predict(Plan* p, const double* xy_new_host, int64_t n_new, int32_t* d_nb
     cudaFree(d_q);
     return rc;
   }
-  std::vector<double> xy(2 * n);
-  if (cudaMemcpy(xy.data(), p->d_xy, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost) != cudaSuccess)
-    return VECCHIA_ECUDA;
-  std::vector<Level> lev;
-  std::vector<int32_t> cs, pidx;
-  std::vector<double> pxy;
-  build_levels(n, xy.data(), lev, cs, pidx, pxy, n);  // one level over all points, original order
-  double *d_pxy = nullptr, *d_q = nullptr;
-  int32_t *d_cs = nullptr, *d_pidx = nullptr;
-  Level* d_lev = nullptr;
-  auto alloc = [&](void** ptr, size_t bytes) {
-    if (rc) return;
-    if (cudaMalloc(ptr, std::max<size_t>(bytes, 16)) != cudaSuccess) rc = VECCHIA_ENOMEM;
-  };
-  alloc((void**)&d_pxy, sizeof(double) * pxy.size());
-  alloc((void**)&d_cs, sizeof(int32_t) * cs.size());
-  alloc((void**)&d_pidx, sizeof(int32_t) * pidx.size());
-  alloc((void**)&d_lev, sizeof(Level) * lev.size());
-  alloc((void**)&d_q, sizeof(double) * 2 * n_new);
-  auto up = [&](void* dst, const void* src, size_t bytes) {
-    if (rc) return;
-    if (cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) rc = VECCHIA_ECUDA;
-  };
-  up(d_pxy, pxy.data(), sizeof(double) * pxy.size());
-  up(d_cs, cs.data(), sizeof(int32_t) * cs.size());
-  up(d_pidx, pidx.data(), sizeof(int32_t) * pidx.size());
-  up(d_lev, lev.data(), sizeof(Level) * lev.size());
-  up(d_q, xy_new_host, sizeof(double) * 2 * n_new);
+  rc = predict_grid(p);
+  double* d_q = nullptr;
+  if (!rc && cudaMalloc(&d_q, sizeof(double) * 2 * n_new) != cudaSuccess) rc = VECCHIA_ENOMEM;
+  if (!rc && cudaMemcpyAsync(d_q, xy_new_host, sizeof(double) * 2 * n_new, cudaMemcpyHostToDevice, stream) != cudaSuccess)
+    rc = VECCHIA_ECUDA;
   if (!rc) {
     KnnArgs a;
     a.xyo = nullptr;
-    a.cell_start = d_cs;
-    a.pt_idx = d_pidx;
-    a.pt_xy = reinterpret_cast<const double2*>(d_pxy);
-    a.levels = d_lev;
-    a.nlev = (int)lev.size();
+    a.cell_start = p->d_grid_cells;
+    a.pt_idx = p->d_grid_idx;
+    a.pt_xy = reinterpret_cast<const double2*>(p->d_grid_xy);
+    a.levels = static_cast<const Level*>(p->d_grid_levels);
+    a.nlev = p->grid_levels;
     a.n = n;
     a.m = p->m;
     a.perm = nullptr;
@@ -614,10 +631,6 @@ int knn_predict(Plan* p, const double* xy_new_host, int64_t n_new, int32_t* d_nb
     if (cudaGetLastError() != cudaSuccess) rc = VECCHIA_ECUDA;
   }
   if (!rc && cudaStreamSynchronize(stream) != cudaSuccess) rc = VECCHIA_ECUDA;
-  cudaFree(d_pxy);
-  cudaFree(d_cs);
-  cudaFree(d_pidx);
-  cudaFree(d_lev);
   cudaFree(d_q);
   return rc;
 }
@@ -631,6 +644,10 @@ static void plan_free(Plan* p) {
   cudaFree(p->d_inv);
   cudaFree(p->d_partial);
   cudaFree(p->d_errloc);
+  cudaFree(p->d_grid_xy);
+  cudaFree(p->d_grid_cells);
+  cudaFree(p->d_grid_idx);
+  cudaFree(p->d_grid_levels);
   delete[] p->h_perm;
   delete p;
 }

@@ -20,7 +20,9 @@
 // Storage: the triangle is packed column by column from the last column (K) to the
 // first, so the columns still to be updated at step j form a prefix [0, off(j)),
 // off(c) = (K-c)(K-c+1)/2.  Every FP64 instruction is issued with as many active lanes
-// as the trailing prefix allows; pivots use one reciprocal (no square root).
+// as the trailing prefix allows; pivots use one reciprocal (no square root).  The larger
+// blocks run a Cholesky factorisation in fixed point instead, in the same storage
+// (fixed_point_block, mmapanel.cuh).
 //
 // Adjoint (not in the paper).  With w = Sigma_JJ^{-1} v, alpha = Sigma_JJ^{-1} y_J,
 // r = y_i - mu_i and s = s_i, write w^ = [-w; 1], a^ = [alpha; 0] and

@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       ysc.init(ytop, tc.sigma2, tc.gamma1, attempt);
       for (int c = tid; c < K; c += NTH) {
         const int o = tri_off(K, c);
-        AF[o] = fixed_from_double((c >= mi && c < m) ? 1.0 : tc.gamma1, 60 - 2 * ysc.f);
+        AF[o] = fixed_from_double(tc.gamma1, 60 - 2 * ysc.f);  // a pad's is any positive number
         AF[o + K - c] = ysc.nonfinite ? 0LL : fixed_from_double(YV[c], 60 - ysc.ky);
       }
       if (tid == 0) AF[0] = 0;

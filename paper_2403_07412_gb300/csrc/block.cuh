@@ -502,9 +502,9 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   for (int c = sub; c < K; c += G) {
     const int o = tri_off(K, c);
     const double dg = (c >= mi && c < m) ? 1.0 : tc.gamma1;
-    if constexpr (kPanels) {  // in fixed point (mmapanel.cuh)
+    if constexpr (kPanels) {  // in fixed point (mmapanel.cuh); a pad's diagonal is any positive number
       const double yc = sep_buffers ? W.TV1[c] : A[o + K - c];
-      A[o] = __longlong_as_double(fixed_from_double(dg, 60 - 2 * ysc.f));
+      A[o] = __longlong_as_double(fixed_from_double(tc.gamma1, 60 - 2 * ysc.f));
       A[o + K - c] = __longlong_as_double(ysc.nonfinite ? 0LL : fixed_from_double(yc, 60 - ysc.ky));
     } else {
       A[o] = dg;

@@ -172,7 +172,7 @@ __device__ __forceinline__ long long scaled_entry(long long a, int q, int rh, in
   const int ch = (int)(n >> 31), cl = (int)n & 0x7FFFFFFF;
   const long long mid = (long long)ch * rl + (long long)cl * rh;
   const long long v = ((long long)ch * rh << 3) + (mid >> 28);
-  return f ? v >> f : v;
+  return f ? v >> min(f, 63) : v;
 }
 
 // Units of a block: f of the diagonal (see above) and ky of the data row, chosen so that z
@@ -251,7 +251,7 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
     const int row = rt + g + 8 * (v >> 1), c = c0 + 2 * t + (v & 1);
     if (row <= K && c < pe && row >= c) {
       const int e = tri_off(K, c) + row - c;
-      if (f && row == c) sum >>= 2 * f;
+      if (f && row == c) sum >>= min(2 * f, 63);
       A[e] -= sum;
     }
   }
@@ -300,7 +300,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       --step;
     }
     s0 += (long long)m0 * 16;
-    if (f && lane == j) s0 >>= 2 * f;
+    if (f && lane == j) s0 >>= min(2 * f, 63);
     const long long a0 = r0 >= c0 + j && r0 <= rmax ? A[oj + q0] - s0 : 0;
     if (j == last) {
       corner[0] = __shfl_sync(0xffffffffu, a0, j);
@@ -318,7 +318,8 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
     if (GRAD && lane == 0) {  // 2^-62 / sqrt(d), the factor that makes V a unit-lower entry
       const float h = __int2float_rz(rh);
       const float lo = __int2float_rn(rh - (int)h) + __int2float_rn(rl) * 0x1p-31f;
-      const float sc = __uint_as_float((unsigned)max(127 + q - 30 - 62 - f, 1) << 23);
+      const int se = 127 + q - 30 - 62 - f;  // below the floats' range past gamma = 2^70: 0
+      const float sc = se > 0 ? __uint_as_float((unsigned)se << 23) : 0.0f;
       const float hs = h + lo;
       RJ[c0 + j] = make_float2(hs * sc, (lo - (hs - h)) * sc);
     }

@@ -541,15 +541,18 @@ static int knn_sphere_gpu(Plan* p, const double* xyz_host, cudaStream_t stream) 
 // order.  It depends on the plan's points only, so it is laid out once, by the first
 // prediction, and freed with the plan (20 bytes a point and 4 a cell).  (Copying the points
 // to the host and building it there for every prediction took 2.3 of 3.7 ms at n = 250,000, 25,000 new
-// points, m = 30.)
+// points, m = 30.)  All copies go to the caller's stream, which may be one that does not wait for
+// the legacy default stream, and have finished before the plan holds the grid: a prediction on
+// another stream, or from another thread, finds it complete.
 static std::mutex g_grid_mu;
 
-static int predict_grid(Plan* p) {
+static int predict_grid(Plan* p, cudaStream_t stream) {
   std::lock_guard<std::mutex> lk(g_grid_mu);
   if (p->d_grid_levels) return VECCHIA_OK;
   const int64_t n = p->n;
   std::vector<double> xy(2 * n);
-  if (cudaMemcpy(xy.data(), p->d_xy, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost) != cudaSuccess)
+  if (cudaMemcpyAsync(xy.data(), p->d_xy, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess)
     return VECCHIA_ECUDA;
   std::vector<Level> lev;
   std::vector<int32_t> cs, pidx;
@@ -562,8 +565,9 @@ static int predict_grid(Plan* p) {
                            sizeof(Level) * lev.size()};
   for (int k = 0; k < 4 && !rc; ++k) {
     if (cudaMalloc(&d[k], std::max<size_t>(bytes[k], 16)) != cudaSuccess) rc = VECCHIA_ENOMEM;
-    else if (cudaMemcpy(d[k], h[k], bytes[k], cudaMemcpyHostToDevice) != cudaSuccess) rc = VECCHIA_ECUDA;
+    else if (cudaMemcpyAsync(d[k], h[k], bytes[k], cudaMemcpyHostToDevice, stream) != cudaSuccess) rc = VECCHIA_ECUDA;
   }
+  if (cudaStreamSynchronize(stream) != cudaSuccess && !rc) rc = VECCHIA_ECUDA;
   if (rc) {
     for (void* q : d) cudaFree(q);
     return rc;
@@ -609,7 +613,7 @@ int knn_predict(Plan* p, const double* xy_new_host, int64_t n_new, int32_t* d_nb
     cudaFree(d_q);
     return rc;
   }
-  rc = predict_grid(p);
+  rc = predict_grid(p, stream);
   double* d_q = nullptr;
   if (!rc && cudaMalloc(&d_q, sizeof(double) * 2 * n_new) != cudaSuccess) rc = VECCHIA_ENOMEM;
   if (!rc && cudaMemcpyAsync(d_q, xy_new_host, sizeof(double) * 2 * n_new, cudaMemcpyHostToDevice, stream) != cudaSuccess)

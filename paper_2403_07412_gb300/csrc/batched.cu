@@ -304,7 +304,7 @@ int class_shape(BatchClass* c, const int* areas, int fixed_bytes) {
 }
 
 int build_batch(const Plan* const* plans, const double* const* ys, int nfields, int ntheta, int want_grad,
-                int dev, BatchState** out) {
+                int dev, cudaStream_t stream, BatchState** out) {
   BatchState* b = new BatchState();
   b->device = dev;
   b->ntheta = ntheta;
@@ -390,7 +390,10 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
     free_batch(b);
     return VECCHIA_ENOMEM;
   }
-  if (cudaMemcpy(b->d_fields, fd.data(), sizeof(FieldDesc) * nfields, cudaMemcpyHostToDevice) != cudaSuccess) {
+  // on the caller's stream (it may not wait for the legacy default stream), and finished before
+  // the layout is cached, where a call on another stream may find it
+  if (cudaMemcpyAsync(b->d_fields, fd.data(), sizeof(FieldDesc) * nfields, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess) {
     free_batch(b);
     return VECCHIA_ECUDA;
   }
@@ -488,7 +491,7 @@ extern "C" int vecchia_loglik_batched(const vecchia_plan_t* plans, const double*
     if (cs != cudaStreamCaptureStatusNone) return VECCHIA_EINVAL;
     std::vector<const Plan*> pp(nfields);
     for (int f = 0; f < nfields; ++f) pp[f] = plans[f];
-    int rc = build_batch(pp.data(), y_devs, nfields, ntheta, want_grad, dev, &b);
+    int rc = build_batch(pp.data(), y_devs, nfields, ntheta, want_grad, dev, s, &b);
     if (rc) return rc;
     g_batches.push_back(b);
   }

@@ -1,6 +1,7 @@
-"""A plan's first prediction on a stream that does not wait for the legacy default stream: the search grid it
-lays out has to be in place before the kernel that reads it, on that stream and on any other that comes
-next.  The grid's contents are exact, so conditioning sets are equal bit for bit."""
+"""A plan's first prediction and a batch's first call on streams that do not wait for the legacy default
+stream: what those calls lay out on the device once has to be in place before the kernels that read it, on
+that stream and on any other that comes next.  The search grid's and the layout's contents are exact, so
+conditioning sets are equal bit for bit and results equal those of a later call."""
 import numpy as np
 import pytest
 import torch
@@ -41,3 +42,19 @@ def test_first_prediction_on_side_streams(V, n):
             assert np.all(np.abs(mean.cpu().numpy() - want[0]) <= 1e-9 * np.maximum(np.abs(want[0]), 1.0))
             assert np.all(np.abs(var.cpu().numpy() - want[1]) <= 1e-9)
         plan.close()
+
+
+def test_first_batched_call_on_a_side_stream(V):
+    sizes = [(700, 10), (400, 30), (300, 60)]
+    V.vecchia_batched_prepare([0.5, 1.5])
+    thetas = torch.as_tensor(np.tile([THETA, (0.8, 0.1, 0.5, 0.1)], (3, 1, 1)), device="cuda").contiguous()
+    plans = [V.Plan(datagen.uniform_locations(n, 40 + m), m, order=V.ORDER_RANDOM, seed=4) for n, m in sizes]
+    ys = [torch.as_tensor(datagen.rng(50 + m).standard_normal(n), device="cuda") for n, m in sizes]
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        batch = V.Batch(plans, ys, 2, want_grad=True)
+        first = batch.run(thetas).clone()
+        side.synchronize()
+    again = batch.run(thetas).cpu().numpy()
+    assert np.array_equal(first.cpu().numpy(), again) and np.isfinite(again).all()

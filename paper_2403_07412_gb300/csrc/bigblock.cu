@@ -222,10 +222,10 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
         float u0h, u0l, u1h, u1l;
         pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
         pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-        long long val0, val1;
+        FixRho val0, val1;
         rho_fixed62(u0h, u0l, u1h, u1l, a.tab, mc, val0, val1);
-        AF[tri_off(K, c0) + r0 - c0] = ok0 ? val0 >> 2 : 0LL;
-        if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? val1 >> 2 : 0LL;
+        AF[tri_off(K, c0) + r0 - c0] = ok0 ? fixed60(val0) : 0LL;
+        if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? fixed60(val1) : 0LL;
       }
       __syncthreads();
       ok = cta_eliminate<GRAD>(K, AF, reinterpret_cast<float2*>(TV), piv, ysc, corner, tid, NTH);

@@ -525,7 +525,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     float u0h, u0l, u1h, u1l;
     pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
     pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-    long long val0, val1;
+    FixRho val0, val1;
     if constexpr (GRAD && !FIXED) {
       val0 = rho_fixed62(u0h, u0l, tab, mc);
       val1 = rho_fixed62(u1h, u1l, tab, mc);
@@ -533,11 +533,13 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
       rho_fixed62(u0h, u0l, u1h, u1l, tab, mc, val0, val1);
     }
     if constexpr (kPanels) {  // units of 2^-60
-      A[w0 >> 16] = __longlong_as_double(v0 ? val0 >> 2 : 0LL);
-      if (has1) A[w1 >> 16] = __longlong_as_double(v1 ? val1 >> 2 : 0LL);
+      A[w0 >> 16] = __longlong_as_double(v0 ? fixed60(val0) : 0LL);
+      if (has1) A[w1 >> 16] = __longlong_as_double(v1 ? fixed60(val1) : 0LL);
     } else {
-      A[w0 >> 16] = fixed62_double(v0 ? val0 : 0LL);
-      if (has1) A[w1 >> 16] = fixed62_double(v1 ? val1 : 0LL);
+      if (!v0) val0.v = 0;
+      if (!v1) val1.v = 0;
+      A[w0 >> 16] = fixed_to_double(val0);
+      if (has1) A[w1 >> 16] = fixed_to_double(val1);
     }
   }
   __syncwarp();

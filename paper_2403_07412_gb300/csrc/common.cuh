@@ -33,7 +33,7 @@ constexpr int kFixDeg = 7;
 constexpr int kFixWords = 5;
 constexpr int kFixInt = (kEHi - kELo) << kFixSub;
 constexpr int kFixNodes = 512;
-constexpr size_t kFixTableBytes = (size_t)16 * kFixWords * kFixInt + sizeof(double) * kNConst + 16 * (size_t)kFixNodes;
+constexpr size_t kFixTableBytes = (size_t)16 * kFixWords * kFixInt + sizeof(double) * kNConst + 20 * (size_t)kFixNodes;
 
 // Largest conditioning sets: overall (CTA-per-location kernel) and for the warp kernels.
 constexpr int kMaxM = VECCHIA_MAX_M;

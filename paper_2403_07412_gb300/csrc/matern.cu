@@ -174,27 +174,32 @@ __global__ void __launch_bounds__(kFitThreads) matern_fit_kernel(double nu, int 
 }
 
 // ------------------------------------------------------------------ likelihood table
-// The likelihood kernels' table (fixtable.cuh) is wanted to 2^-60 or so of rho(0) = 1, and
-// an optimiser that moves nu builds one at every step, so it is built in 64-bit integers,
-// which cost a warp 2 to 5 cycles an instruction where FP64 costs 64:
-//   rho(u) = sum_k W_k exp(-u G_k),  W_k = h exp(nu tau_k - e^tau_k) / Gamma(nu),
-// G_k = e^-tau_k / 4, the trapezoidal rule for I(u) on one grid for all u.  h = ln 2 / p, so
-// that e^tau_k is a power of two times one of p numbers in [1, 2).  h <= 0.6 / sqrt(nu + 36)
-// resolves the integrand's peak (width 1 / sqrt(nu + x) or so) up to x = 36, beyond which
-// rho is below 2^-51 and the rule's relative error may grow; the grid ends where W_k, or
-// exp(-2^kELo G_k), has fallen below e^-44.
+// The likelihood kernels' table (fixtable.cuh) is wanted to 2^-60 or so of rho(0) = 1, and where rho
+// is small to 2^-50 of itself, and an optimiser that moves nu builds one at every step, so it is
+// built in 64-bit integers, which cost a warp 2 to 5 cycles an instruction where FP64 costs 64:
+//   rho(u) = sum_k exp(-(x_k + u G_k)),  x_k = e^tau_k - nu tau_k + log Gamma(nu) - log h,
+// G_k = e^-tau_k / 4, the trapezoidal rule for I(u) on one grid for all u; an interval whose
+// values are small takes exp(E ln 2 - x_k - u G_k).  h = ln 2 / p, so
+// that e^tau_k is a power of two times one of p numbers in [1, 2).  h <= 0.6 / sqrt(nu + 47)
+// resolves the integrand's peak (width (nu^2 + u)^(-1/4)) to a relative 2^-50 up to sqrt(u) = 67,
+// beyond which the polynomials' own relative error (2^-30 there) grows faster.  The integrand falls
+// below e^-44 of its peak within acosh(1 + 44 / R) above the peak t* = (nu + R) / 2, R =
+// sqrt(nu^2 + u): with s = tau - log t* it is exp(-R (cosh s - 1) - nu (sinh s - s)) of the peak.
+// The grid ends where that has happened at the largest u, and where x_k, or 2^kELo G_k, exceeds 44.
 // A fresh nu took 350 us beside the call's own work with a quadrature in FP64 of each
 // interval's Chebyshev values.
 struct FixSetup {
   int family, p, klo, n;
   unsigned long long lnp;    // ln 2 / p in units of 2^-64
   double nu, norm, norm_lo;  // log Gamma(nu) - log h as a pair
+  float stirling;            // Stirling's log Gamma(nu), to order 1 / nu^0, less log Gamma(nu)
   double c[kNConst];         // small-u constants (matern.cuh)
   FixSetup(int family_, double nu_) : family(family_), nu(nu_) {
     p = 1;
     klo = n = 0;
     lnp = 0;
     norm = norm_lo = 0.0;
+    stirling = 0.0f;
     for (double& v : c) v = 0.0;
     c[1] = nu;
     const bool integer = nu == std::floor(nu);
@@ -210,16 +215,20 @@ struct FixSetup {
       c[5] = 0.25 / std::tgamma(2.0 + nu);
     }
     constexpr double kLn2 = 0.693147180559945309417;
-    const double hi = std::log(60.0 + nu + std::min(nu, 14.0 * std::sqrt(nu)));
+    const double R = std::sqrt(nu * nu + std::ldexp(1.0, kEHi));
+    const double hi = std::max(std::log(60.0 + nu + std::min(nu, 14.0 * std::sqrt(nu))),
+                               std::log(0.5 * (nu + R)) + std::acosh(1.0 + 44.0 / R));
     const double lo = std::max(std::log(nu) - 45.0 / nu - std::sqrt(120.0 / nu), -26.5);
     const double most = (kFixNodes - 3) * kLn2 / (hi - lo);
-    p = (int)std::max(1.0, std::min(std::ceil(kLn2 * std::sqrt(nu + 36.0) / 0.6), std::min(std::floor(most), 1e6)));
+    p = (int)std::max(1.0, std::min(std::ceil(kLn2 * std::sqrt(nu + 47.0) / 0.6), std::min(std::floor(most), 1e6)));
     klo = (int)std::floor(lo * p / kLn2);
     n = std::min(kFixNodes, (int)std::ceil(hi * p / kLn2) - klo + 1);
     lnp = 0xB17217F7D1CF79ACull / p;
-    const long double v = std::lgamma((long double)nu) - std::log(0.693147180559945309417232121458L / p);
+    const long double lg = std::lgamma((long double)nu);
+    const long double v = lg - std::log(0.693147180559945309417232121458L / p);
     norm = (double)v;
     norm_lo = (double)(v - norm);
+    stirling = (float)(nu * std::log((long double)nu) - nu - 0.5L * std::log(nu / 6.283185307179586477L) - lg);
   }
 };
 
@@ -252,7 +261,8 @@ __device__ __forceinline__ void fix_node_power(const FixSetup& s, int k, int& q,
   b = K - q * s.p;
 }
 
-// Nodes (after the constants): W_k in units of 2^-65, and 2^(b/p - 1) in units of 2^-63.
+// Nodes (after the constants): x_k modulo 64 in units of 2^-58, and 2^(b/p - 1) in units of 2^-63;
+// then x_k as floats.
 __global__ void fix_nodes_kernel(const FixSetup s, double* tab) {
   double* c = fix_const(tab);
   const int k = blockIdx.x * 32 + threadIdx.x;
@@ -273,26 +283,19 @@ __global__ void fix_nodes_kernel(const FixSetup s, double* tab) {
   x.add(-ph * 0x1p-57);
   x.add(eh * sc);
   x.add(s.norm_lo - pl * 0x1p-57 + el * sc);
-  const double xt = x.s + x.c;
-  unsigned long long w = 0;
-  if (xt < 44.0) {
-    const double xl = (x.s - xt) + x.c;
-    const unsigned long long xi = __double2ull_rn(fmax(xt, 0.0) * 0x1p58);
-    w = min(fix_exp(xi + (unsigned long long)__double2ll_rn(fmax(xl, -xt) * 0x1p58)), 0x1FFFFFFFFFFFFFFFull) << 2;
-  }
+  const double xt = x.s + x.c, xl = (x.s - xt) + x.c;
+  const double xm = xt < 1024.0 ? xt - 64.0 * floor(xt * 0x1p-6) : 0.0;  // beyond, the float says enough
+  const unsigned long long xi = __double2ull_rz(xm * 0x1p58) + (unsigned long long)__double2ll_rn(xl * 0x1p58);
   const unsigned long long mant = fix_exp(((s.p - b) * s.lnp) >> 6);
-  reinterpret_cast<ulonglong2*>(c + kNConst)[k] = make_ulonglong2(w, mant);
+  ulonglong2* nodes = reinterpret_cast<ulonglong2*>(c + kNConst);
+  nodes[k] = make_ulonglong2(xi, mant);
+  reinterpret_cast<float*>(nodes + kFixNodes)[k] = (float)xt;
 }
 
-// v 2^sh as the argument of fix_exp; past its range (x >= 44): all ones.
-__device__ __forceinline__ unsigned long long fix_arg_shift(unsigned long long v, int sh) {
-  constexpr unsigned long long most = 44ull << 58;
-  if (sh >= 0) return sh >= 64 || v > (most >> min(sh, 63)) ? ~0ull : v << sh;
-  if (sh <= -64) return 0;
-  v >>= -sh;
-  return v >= most ? ~0ull : v;
+// v 2^sh modulo 2^64.
+__device__ __forceinline__ unsigned long long fix_shift(unsigned long long v, int sh) {
+  return sh >= 0 ? (sh < 64 ? v << sh : 0) : (sh > -64 ? v >> -sh : 0);
 }
-__device__ __forceinline__ unsigned long long fix_exp_or_0(unsigned long long x) { return x == ~0ull ? 0 : fix_exp(x); }
 
 // cos(i pi / 16)
 constexpr double kCos16[9] = {1.0,
@@ -333,55 +336,89 @@ struct FixInterp {
 __device__ const FixInterp kFixInterp = FixInterp();
 
 // One CTA per kFixGroup = 8 intervals [2^e (1 + j/32), ...) of an octave, 64 values u = 2^e
-// (1 + (j + t)/32).  exp(-u G) is the product of a factor for j, which takes W too, and one
-// for t: 16 exponentials a node for the 64 values, and a 64-bit product each (some 30
-// cycles of a warp; an exponential some 350, 1,400 in FP64).  Then the eight values of an
+// (1 + (j + t)/32).  exp(-u G) is the product of a factor for j, which takes x_k and the
+// interval's E too, and one for t: 16 exponentials a node for the 64 values, and a 64-bit product each (some 30
+// cycles of a warp; an exponential some 350, 1,400 in FP64).  The sum x_k + u G_k - E ln 2 is formed
+// modulo 64, and beside it in floats, which say whether it exceeds 44 (and the term is left out).
+// E comes from rho's estimate by Laplace's method at the interval's lower end, (nu / t*)^-nu
+// exp(nu - R) sqrt(nu / R) over Stirling's error: within 2% for nu >= 0.05 where rho < 2^-7.  Then the eight values of an
 // interval give its monomials: integer differences from one of them, exact, times the
 // matrix above in FP64, a thread per coefficient.
 constexpr int kFixGroup = 8;
 constexpr int kFixThreads = 256;
 constexpr int kFixChunk = 64;  // nodes at a time
+constexpr int kFixMostE = 960;  // (62 + E) 2^20 is subtracted from an exponent field
 
 __global__ void __launch_bounds__(kFixThreads) fix_table_kernel(const FixSetup s, double* tab) {
   __shared__ unsigned long long ea[kFixChunk][kFixGroup], eb[kFixChunk][8], part[4][64];
+  __shared__ int scale[kFixGroup];  // E
   const int tid = threadIdx.x;
   const int e = kELo + (blockIdx.x * kFixGroup >> kFixSub);
   const int j0 = blockIdx.x * kFixGroup & ((1 << kFixSub) - 1);
+  const float nu = (float)s.nu;
+  if (tid < kFixGroup) {
+    const float u = ldexpf((float)(32 + j0 + tid), e - kFixSub);
+    float bits;  // -log2 rho
+    if (s.family == kFamilyPowExp) {
+      bits = 1.442695041f * expf(0.5f * nu * logf(u));
+    } else {
+      const float R = sqrtf(fmaf(nu, nu, u)), d = u / (R + nu);  // R - nu
+      bits = 1.442695041f * (d - nu * log1pf(0.5f * d / nu) - 0.5f * logf(nu / R) - s.stirling);
+    }
+    scale[tid] = (int)fminf(fmaxf(floorf(bits) - 6.0f, 0.0f), (float)kFixMostE);
+  }
+  __syncthreads();
   if (s.family == kFamilyPowExp) {
     if (tid < 64) {
       const double t = (double)kFixInterp.t[tid & 7] * 0x1p-64;
       const double u = ldexp(1.0 + (j0 + (tid >> 3) + t) / (1 << kFixSub), e);
-      part[0][tid] = __double2ull_rn(exp(-exp(0.5 * s.nu * log(u))) * 0x1p63);
+      const double x = exp(0.5 * s.nu * log(u)) - 0.693147180559945309417 * scale[tid >> 3];
+      part[0][tid] = __double2ull_rn(exp(-x) * 0x1p63);
     }
   } else {
     const ulonglong2* __restrict__ nodes = reinterpret_cast<const ulonglong2*>(fix_const(tab) + kNConst);
-    const int k0 = max(0, (int)((e - 7.5f) * s.p) - s.klo - 1);  // 2^e G_k < 44 from here on
+    const float* __restrict__ xf = reinterpret_cast<const float*>(nodes + kFixNodes);
+    // outside [k0, k1) a term is below e^-44
+    const float eln2 = 0.6931472f * (float)scale[kFixGroup - 1], u1 = ldexpf(1.0f, e + 1);
+    const int k0 = max(0, (int)(((float)e - log2f(4.0f * (44.0f + eln2))) * s.p) - s.klo - 2);
+    const float R1 = sqrtf(fmaf(nu, nu, u1));
+    const float top = logf(0.5f * (nu + R1)) + acoshf(1.0f + 44.0f / R1);
+    const int k1 = min(s.n, max(k0, (int)(1.442695041f * top * s.p) - s.klo + 3));
     unsigned long long acc = 0;
+    unsigned terms = 0;
     const int out = tid & 63, slice = tid >> 6;
-    for (int kc = k0; kc < s.n; kc += kFixChunk) {
+    for (int kc = k0; kc < k1; kc += kFixChunk) {
       const int kk = tid & (kFixChunk - 1), k = kc + kk, r = 2 * (tid / kFixChunk);
       ulonglong2 w = make_ulonglong2(0, 0);
+      float x = INFINITY, g = 0.0f;
       int q = 0, b;
-      if (k < s.n) {
+      if (k < k1) {
         w = nodes[k];
+        x = xf[k];
         fix_node_power(s, k, q, b);
+        g = ldexpf(__ull2float_rn(w.y), e + q - 64 - kFixSub);  // 2^e G / 32 = mant 2^(e + q - 1) / 32
       }
-      // 2^e G = mant 2^(e + q - 1)
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const unsigned long long xa = fix_arg_shift((w.y >> 6) * (32 + j0 + r + i), e + q - 5);
-        ea[kk][r + i] = __umul64hi(w.x, fix_exp_or_0(xa));
-        const unsigned long long xb = fix_arg_shift(__umul64hi(w.y, kFixInterp.t[r + i]), e + q - 11);
-        eb[kk][r + i] = fix_exp_or_0(xb);
+        const int E = scale[r + i];
+        const float about = fmaf(g, (float)(32 + j0 + r + i), x) - 0.6931472f * (float)E;
+        unsigned long long xa = w.x + fix_shift((w.y >> 6) * (32 + j0 + r + i), e + q - 5) -
+                                (unsigned long long)E * 0x2C5C85FDF473DE7ull;
+        if (about < 1.0f && (long long)xa < 0) xa = 0;  // rounded below 0
+        ea[kk][r + i] = about < 44.0f ? min(2 * fix_exp(xa), 0xFFFFFFFFFFFFFFFEull) : 0;
+        const unsigned long long xb = fix_shift(__umul64hi(w.y, kFixInterp.t[r + i]), e + q - 11);
+        eb[kk][r + i] = g < 44.0f ? fix_exp(xb) : 0;
       }
       __syncthreads();
 #pragma unroll 4
-      for (int i = slice * (kFixChunk / 4); i < (slice + 1) * (kFixChunk / 4); ++i)
-        acc += __umul64hi(ea[i][out >> 3], eb[i][out & 7]);
+      for (int i = slice * (kFixChunk / 4); i < (slice + 1) * (kFixChunk / 4); ++i) {
+        const unsigned long long x1 = ea[i][out >> 3];
+        acc += __umul64hi(x1, eb[i][out & 7]);
+        terms += x1 != 0;
+      }
       __syncthreads();
     }
-    if (slice == 0 && s.n > k0) acc += (unsigned)(s.n - k0) / 2;  // the products are rounded down
-    part[slice][out] = acc;
+    part[slice][out] = acc + terms / 2;  // the products are rounded down
   }
   __syncthreads();
   if (tid >= 64) return;
@@ -400,13 +437,14 @@ __global__ void __launch_bounds__(kFixThreads) fix_table_kernel(const FixSetup s
   for (int o = 4; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o, 8));
   const int S = top > 0 ? 1022 - top : 0;
   const double ms = m * __longlong_as_double((long long)(1023 + S) << 52);
+  const int E = scale[tid >> 3];
   float* w = reinterpret_cast<float*>(tab) + (size_t)(blockIdx.x * kFixGroup + (tid >> 3)) * 4 * kFixWords;
   if (k == 0) {
     const long long c0 = (long long)((f[4] + 1) >> 1) + __double2ll_rn(m * 0x1p62);
     w[12] = __int_as_float((int)(unsigned)((unsigned long long)c0 & 0xFFFFFFFFull));
     w[13] = __int_as_float((int)(c0 >> 32));
     w[14] = ldexpf(1.0f, 36 - S);
-    w[15] = ldexpf(1.0f, -S);
+    w[15] = ldexpf(1.0f, -S - E);
   } else if (k <= 4) {
     split_float(ms, w + 2 * (k - 1));
     if (k == 3) split_float(3.0 * ms, w + 16);
@@ -414,7 +452,7 @@ __global__ void __launch_bounds__(kFixThreads) fix_table_kernel(const FixSetup s
     w[8 + k - 5] = (float)ms;
     if (k == 5) w[18] = (float)(5.0 * ms);
     if (k == 6) w[19] = (float)(6.0 * ms);
-    if (k == 7) w[11] = 0.0f;
+    if (k == 7) w[11] = __int_as_float((62 + E) << 20);
   }
 }
 

@@ -111,7 +111,7 @@ __device__ __forceinline__ void run_item(const FieldDesc& fd, int64_t tile, cons
 }
 
 template <bool GRAD, int G, bool FIXED>
-__global__ void __launch_bounds__(GRAD && G == 8 ? 512 : GRAD || FIXED ? 384 : 32 * kMaxCtaWarps)
+__global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : (FIXED ? 512 : 32 * kMaxCtaWarps))
     vecchia_batched_kernel(const BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   for (int k = 0; k < a.nk; ++k)

@@ -72,41 +72,36 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // panel's columns and, once warp 0's sixteen rows are in (barrier 1), update them.
 template <bool GRAD>
 __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, float2* __restrict__ RJ, int4* __restrict__ piv,
-                                              PanelScale& ysc, long long* corner, int tid, int NTH) {
+                                              double* __restrict__ zs, int f, long long* corner, int tid, int NTH) {
   const int lane = tid & 31, wid = tid >> 5;
-  int over = 0, grow = 0;
-  // pivots of this panel and the next
+  int over = 0;
+  // piv and zs hold those of this panel and the next
 #pragma unroll 1
   for (int c0 = -kPanelCols; c0 + kPanelCols < K; c0 += kPanelCols) {
     const int c1 = c0 + kPanelCols, pe = min(c1 + kPanelCols, K);
     const int4* __restrict__ pv = piv + (c0 & kPanelCols);
+    const double* __restrict__ pz = zs + (c0 & kPanelCols);
     if (wid == 0) {
       if (c0 >= 0) {
-        if (lane < 16 && c1 + lane <= K) panel_row(K, A, pv, c0, ysc.f, c1 + lane, over, grow);
+        if (lane < 16 && c1 + lane < K) panel_row(K, A, pv, pz, c0, f, c1 + lane, over);
         __threadfence_block();
         asm volatile("bar.arrive 1, %0;" ::"r"(NTH) : "memory");
         __syncwarp();
-        update_tile(K, A, c1, c1, pe, ysc.f, lane);
+        update_tile(K, A, c1, c1, pe, f, lane);
         __syncwarp();
       }
-      long long cr[2] = {0, 0};
-      bool g = false;
-      if (!panel_columns<GRAD, true>(K, A, RJ, piv + (c1 & kPanelCols), c1, ysc.f, g, cr, lane)) over = 1;
-      if (g) grow = 1;
-      if (pe == K && lane == 0) {
-        corner[0] = cr[0];
-        corner[1] = cr[1];
-      }
+      long long cr = 0;
+      if (!panel_columns<GRAD, true>(K, A, RJ, piv + (c1 & kPanelCols), zs + (c1 & kPanelCols), c1, f, cr, lane)) over = 1;
+      if (pe == K && lane == 0) *corner = cr;
     } else if (c0 >= 0) {
 #pragma unroll 1
-      for (int r = c1 + 16 + tid - 32; r <= K; r += NTH - 32) panel_row(K, A, pv, c0, ysc.f, r, over, grow);
+      for (int r = c1 + 16 + tid - 32; r < K; r += NTH - 32) panel_row(K, A, pv, pz, c0, f, r, over);
       asm volatile("bar.sync 1, %0;" ::"r"(NTH) : "memory");
 #pragma unroll 1
-      for (int rt = c1 + 16 * wid; rt <= K; rt += (NTH - 32) / 2) update_tile(K, A, rt, c1, pe, ysc.f, lane);
+      for (int rt = c1 + 16 * wid; rt < K; rt += (NTH - 32) / 2) update_tile(K, A, rt, c1, pe, f, lane);
     }
     __syncthreads();
   }
-  ysc.grown = __syncthreads_or(grow) != 0;
   return __syncthreads_or(over) == 0;
 }
 
@@ -129,7 +124,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
   long long* corner = reinterpret_cast<long long*>(red + 32);
   double* coef = reinterpret_cast<double*>(corner + 2);
   int4* piv = reinterpret_cast<int4*>(coef + 4);
-  unsigned* ytops = reinterpret_cast<unsigned*>(piv + 2 * kPanelCols);
+  double* zs = reinterpret_cast<double*>(piv + 2 * kPanelCols);
   long long* AF = reinterpret_cast<long long*>(A);
   float2* WHf = reinterpret_cast<float2*>(WH);  // w^ and g as float pairs for the beta sums
   float2* GVf = reinterpret_cast<float2*>(GV);
@@ -138,6 +133,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
   const MaternConst mc = matern_const_at(fix_const(a.tab));
   ThetaConst tc;
   tc.set(a.sigma2, a.beta, a.tau2, a.family, a.nu);
+  const int f = panel_shift(tc.gamma1);
   const double2* __restrict__ xy2 = reinterpret_cast<const double2*>(a.xy);
   FieldView F;  // the distance fields pair_u reads
   F.sphere = sphere;
@@ -159,7 +155,6 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
     }
     const double2 ps = xy2[js];
     // ---- gather: centred, 1/beta-scaled coordinates as float pairs, and data
-    unsigned ytop = 0u;  // largest exponent field of the data
 #pragma unroll 1
     for (int p = tid; p < m; p += NTH) {
         double xv = 0.0, yv = 0.0, zv = 0.0, fv = 0.0;
@@ -181,7 +176,6 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
           fv = a.yf[j];
         }
         YV[p] = fv;
-        ytop = max(ytop, exponent_field(fv));
         CX[p] = d2f_pair(xv);
         CY[p] = d2f_pair(yv);
         if constexpr (SPHERE) CZ[p] = d2f_pair(zv);
@@ -191,53 +185,40 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       CY[m] = make_float2(0.0f, 0.0f);
       if constexpr (SPHERE) CZ[m] = make_float2(0.0f, 0.0f);
       YV[m] = a.yf[js];
-      ytop = max(ytop, exponent_field(a.yf[js]));
     }
-    ytop = __reduce_max_sync(0xffffffffu, ytop);
-    if (lane == 0) ytops[wid] = ytop;
     if (kChecked) bad_idx = __syncthreads_or(bad_idx) != 0;
     __syncthreads();
-    for (int w = 0; w < NTH >> 5; ++w) ytop = max(ytop, ytops[w]);
-    // ---- assemble, in fixed point (mmapanel.cuh); again with larger units in the rare case
-    // that an entry of the data row outgrows them
-    PanelScale ysc;
-    bool ok = true;
-    for (int attempt = 0;; ++attempt) {
-      ysc.init(ytop, tc.sigma2, tc.gamma1, attempt);
-      for (int c = tid; c < K; c += NTH) {
-        const int o = tri_off(K, c);
-        AF[o] = fixed_from_double(tc.gamma1, 60 - 2 * ysc.f);  // a pad's is any positive number
-        AF[o + K - c] = ysc.nonfinite ? 0LL : fixed_from_double(YV[c], 60 - ysc.ky);
-      }
-      if (tid == 0) AF[0] = 0;
-      for (int q0 = tid; q0 < NP; q0 += 2 * NTH) {
-        const int q1 = q0 + NTH;
-        const bool has1 = q1 < NP;
-        const int v0 = tri_root(q0), v1 = tri_root(has1 ? q1 : q0);
-        const int c0 = K - 2 - v0, r0 = c0 + 1 + (q0 - v0 * (v0 + 1) / 2);
-        const int qq1 = has1 ? q1 : q0;
-        const int c1 = K - 2 - v1, r1 = c1 + 1 + (qq1 - v1 * (v1 + 1) / 2);
-        const bool ok0 = c0 < mi && (r0 < mi || r0 == m);
-        const bool ok1 = has1 && c1 < mi && (r1 < mi || r1 == m);
-        float u0h, u0l, u1h, u1l;
-        pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
-        pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-        FixRho val0, val1;
-        rho_fixed62(u0h, u0l, u1h, u1l, a.tab, mc, val0, val1);
-        AF[tri_off(K, c0) + r0 - c0] = ok0 ? fixed60(val0) : 0LL;
-        if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? fixed60(val1) : 0LL;
-      }
-      __syncthreads();
-      ok = cta_eliminate<GRAD>(K, AF, reinterpret_cast<float2*>(TV), piv, ysc, corner, tid, NTH);
-      if (!ysc.grown || !ok || ysc.nonfinite || attempt == 7) break;
+    // ---- assemble, in fixed point (mmapanel.cuh)
+    for (int c = tid; c < K; c += NTH) {
+      const int o = tri_off(K, c);
+      AF[o] = fixed_from_double(tc.gamma1, 60 - 2 * f);  // a pad's is any positive number
+      A[o + K - c] = YV[c];
     }
+    if (tid == 0) AF[0] = 0;
+    for (int q0 = tid; q0 < NP; q0 += 2 * NTH) {
+      const int q1 = q0 + NTH;
+      const bool has1 = q1 < NP;
+      const int v0 = tri_root(q0), v1 = tri_root(has1 ? q1 : q0);
+      const int c0 = K - 2 - v0, r0 = c0 + 1 + (q0 - v0 * (v0 + 1) / 2);
+      const int qq1 = has1 ? q1 : q0;
+      const int c1 = K - 2 - v1, r1 = c1 + 1 + (qq1 - v1 * (v1 + 1) / 2);
+      const bool ok0 = c0 < mi && (r0 < mi || r0 == m);
+      const bool ok1 = has1 && c1 < mi && (r1 < mi || r1 == m);
+      float u0h, u0l, u1h, u1l;
+      pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
+      pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
+      FixRho val0, val1;
+      rho_fixed62(u0h, u0l, u1h, u1l, a.tab, mc, val0, val1);
+      AF[tri_off(K, c0) + r0 - c0] = ok0 ? fixed60(val0) : 0LL;
+      if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? fixed60(val1) : 0LL;
+    }
+    __syncthreads();
+    const bool ok = cta_eliminate<GRAD>(K, AF, reinterpret_cast<float2*>(TV), piv, zs, f, corner, tid, NTH);
     // ---- the term, on warp 0 (FP64)
     const double nan = __longlong_as_double(0x7FF8000000000000LL);
     if (wid == 0) {
-      const double st = mul_pow2((double)corner[0], 2 * ysc.f - 60);
-      // data not finite (or far out of any scale): with pd, a data error
-      const double rr = ysc.grown || ysc.nonfinite ? nan : mul_pow2((double)corner[1], ysc.ky - 60);
-      const bool pd = ok && positive_finite(st);
+      const double st = mul_pow2((double)*corner, 2 * f - 60), rr = A[2];
+      const bool pd = ok && positive_finite(st);  // a non-finite rr with pd: non-finite data
       const bool good = pd && finite_bits(rr) && !bad_idx;
       const double s = tc.sigma2 * st;
       const double inv_s = rcp_newton(s);
@@ -267,7 +248,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
     // the pair pass on all threads
     const double cb = coef[0], rsa = coef[1], sS = coef[2];
     const bool good = finite_bits(sS);
-    panels_to_pairs(K, AF, reinterpret_cast<const float2*>(TV), ysc, tid, NTH);
+    panels_to_pairs(K, AF, reinterpret_cast<const float2*>(TV), tid, NTH);
     __syncthreads();
     const float2* __restrict__ L = reinterpret_cast<const float2*>(A);  // the unit factor
     double pT = 0.0;
@@ -352,7 +333,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
 // Shared memory of the CTA kernel for block size K.
 int big_smem_bytes(int K, bool sphere) {
   const int NTd = (K + 1) * (K + 2) / 2;
-  return 8 * (align_up(NTd, 2) + (sphere ? 7 : 6) * align_up(K + 1, 2) + 32 + 6 + 4 * kPanelCols + 4);
+  return 8 * (align_up(NTd, 2) + (sphere ? 7 : 6) * align_up(K + 1, 2) + 32 + 6 + 6 * kPanelCols);
 }
 
 // CTA size: the W warps with the largest c W / (W + 2), c the CTAs of that size resident on an SM

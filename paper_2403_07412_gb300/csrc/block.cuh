@@ -444,16 +444,10 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   // the border by the assembly (that order measured 1% faster there)
   const bool regather = regather_capable(GRAD, G) && W.regather;  // warp-uniform
   const bool sep_buffers = GRAD && !regather;
-  // Full-warp blocks: the panels' elimination on the tensor cores (mmapanel.cuh) holds the
-  // data row in units of 2^ky; in the rare case that one of its entries outgrows them, the
-  // block is built and eliminated again with larger units.
   static_assert(!FIXED || G == 32, "fixed point is for full-warp blocks");
   constexpr bool kPanels = FIXED;
-  PanelScale ysc;
-  long long corner[2] = {0, 0};
-  bool ok = true;
-  for (int attempt = 0;; ++attempt) {
-  unsigned ytop = 0u;  // largest exponent field of the data
+  const int f = kPanels ? panel_shift(tc.gamma1) : 0;
+  long long corner = 0;
 #pragma unroll
   for (int s = 0; s < NSG; ++s) {
     const int p = sub + G * s;
@@ -468,7 +462,6 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
         coord_offsets<SPHERE>(F, tc, ps, js, j, xv, yv, zv);
         fv = F.yf[j];
       }
-      if constexpr (kPanels) ytop = max(ytop, exponent_field(fv));
       if (sep_buffers) {
         W.TV1[p] = fv;
       } else {
@@ -483,7 +476,6 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     CX[m] = make_float2(0.0f, 0.0f);
     CY[m] = make_float2(0.0f, 0.0f);
     if constexpr (SPHERE) CZ[m] = make_float2(0.0f, 0.0f);
-    if constexpr (kPanels) ytop = max(ytop, exponent_field(F.yf[js]));
     if (sep_buffers) {
       W.TV1[m] = F.yf[js];
     } else {
@@ -496,20 +488,17 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     bad_idx = (__ballot_sync(0xffffffffu, bad_idx) & gmask) != 0u;
   }
   __syncwarp();
-  if constexpr (kPanels) ysc.init(ytop, tc.sigma2, tc.gamma1, attempt);
   // ---- assemble: diagonal (and, with separate column buffers, the data border), then
   // the correlation pairs
   for (int c = sub; c < K; c += G) {
     const int o = tri_off(K, c);
     const double dg = (c >= mi && c < m) ? 1.0 : tc.gamma1;
     if constexpr (kPanels) {  // in fixed point (mmapanel.cuh); a pad's diagonal is any positive number
-      const double yc = sep_buffers ? W.TV1[c] : A[o + K - c];
-      A[o] = __longlong_as_double(fixed_from_double(tc.gamma1, 60 - 2 * ysc.f));
-      A[o + K - c] = __longlong_as_double(ysc.nonfinite ? 0LL : fixed_from_double(yc, 60 - ysc.ky));
+      A[o] = __longlong_as_double(fixed_from_double(tc.gamma1, 60 - 2 * f));
     } else {
       A[o] = dg;
-      if (sep_buffers) A[o + K - c] = W.TV1[c];
     }
+    if (sep_buffers) A[o + K - c] = W.TV1[c];
   }
   if (sub == 0) A[0] = 0.0;
   // Two pairs per lane per iteration so one pair's loads overlap the other's FMAs.
@@ -547,7 +536,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   // j+1 updated by column j and scaled, then one pass over the remaining prefix applying
   // both (fma(-L1, T1, fma(-L0, T0, a)): the same roundings, in the same order, as two
   // single-column steps, with half the column transitions and shared-memory passes).
-  ok = true;
+  bool ok = true;
   double* __restrict__ TV1 = W.TV1;  // column j+1's unscaled entries
   // Column scaling by the pivot reciprocal: the integer round-to-nearest-even product
   // (mul_by_positive, bit-identical to the DMUL) in the 4-lane forward kernel, where it
@@ -555,10 +544,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   // 1.245 ms); the DMUL elsewhere (8- and 16-lane groups 2.5% faster with it at m = 30).
   constexpr bool kIntScale = G == 4 && !GRAD;
   if constexpr (kPanels) {
-    ok = panels_eliminate<GRAD>(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), ysc, corner, sub);
-    if (!ysc.grown || !ok || ysc.nonfinite || attempt == 7) break;
-    __syncwarp();
-    continue;
+    ok = panels_eliminate<GRAD>(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), f, corner, sub);
   } else {
   int j = 0;
   for (; j + 2 < K; j += 2) {
@@ -730,15 +716,8 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     __syncwarp();
   }
   }
-  break;
-  }
-  double st = A[1];  // s_i / sigma2
-  double rr = A[2];  // y_i - mu_i
-  if constexpr (kPanels) {
-    st = mul_pow2((double)corner[0], 2 * ysc.f - 60);
-    rr = mul_pow2((double)corner[1], ysc.ky - 60);
-    if (ysc.grown || ysc.nonfinite) rr = __longlong_as_double(0x7FF8000000000000LL);  // data not finite (or far out of any scale)
-  }
+  const double st = kPanels ? mul_pow2((double)corner, 2 * f - 60) : A[1];  // s_i / sigma2
+  const double rr = A[2];                                                    // y_i - mu_i
   // The pivots and s_i depend on the covariance only, the residual on the data: a
   // non-finite residual (with a positive definite block) means a non-finite y in B_i.
   const bool pd = ok && positive_finite(st);
@@ -798,7 +777,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   }
   constexpr int NS = (KCAP - 1 + G - 1) / G;  // slots of the K-1 <= KCAP-1 neighbour entries
   if constexpr (kPanels) {
-    panels_to_pairs(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), ysc, sub, 32);
+    panels_to_pairs(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), sub, 32);
     __syncwarp();
   }
   // The two unit backward solves run in double-float arithmetic on the FP32 pipe: each

@@ -100,9 +100,11 @@ struct SmemLayout {
 // Up to 13 warps per CTA for the forward pass (its two-vector blocks fit thirteen on an
 // SM at m = 60) and 12 for the gradient; the 8-lane gradient kernels are bounded for 16
 // warps per SM (two CTAs of 8, at most 128 registers a thread), which their second-gather
-// layout reaches at m = 25.  The fixed-point kernels (FIXED) take up to 168 registers a thread.
+// layout reaches at m = 25.  The fixed-point kernels (FIXED) with the gradient take 168 registers
+// a thread; without, they are bounded for 16 warps (128 registers), which the blocks up to m = 52 or
+// so leave room for (n = 100k, 12 and 16 warps an SM: m = 45 3.53 and 3.28 ms, m = 50 4.19 and 3.99).
 template <bool GRAD, int G, bool SPHERE, bool FIXED>
-__global__ void __launch_bounds__(GRAD && G == 8 ? 512 : GRAD || FIXED ? 384 : 32 * kMaxCtaWarps)
+__global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : (FIXED ? 512 : 32 * kMaxCtaWarps))
     vecchia_lik_kernel(const LikArgs a) {
   asm volatile("griddepcontrol.launch_dependents;");  // launch_finalize
   extern __shared__ __align__(16) unsigned char smem[];
@@ -349,7 +351,10 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return -2;
       int per_sm = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, bytes) != cudaSuccess) return -2;
-      const int warps = std::min(per_sm * W, 16);
+      int warps = std::min(per_sm * W, 16);
+      // Fixed point: an SM's four sub-partitions with the same number of warps each (n = 100k, 12 and 13
+      // warps: m = 54 4.56 and 4.96 ms, m = 60 5.68 and 6.09).
+      if (fixed_point_block(K, grad, G) && warps % 4) warps = std::max(1, (warps & ~3) - 1);
       if (per_sm > 0 && warps > best_warps) {
         best_warps = warps;
         out->G = G;

@@ -12,8 +12,13 @@
 //   - V = Lc 2^62.  Off-diagonal entries of Lc are at most 2^-f in magnitude: a Schur
 //     complement of R + gamma I is gamma I plus a positive semidefinite matrix with diagonal
 //     at most 1, hence Lc_rk^2 <= 1 / (1 + gamma);
-//   - the data row y and its factor entries z = Lc^-1 y in units of 2^(ky - 60) and
-//     2^(ky - 62) (PanelScale).
+//   - the data row y stays in FP64 (data have no common scale: one outlier, or a rough field under
+//     a smooth covariance, would cost a row of integers its digits): each column's
+//     z_c = y_c / sqrt(d_c) and y_r -= Lc_rc z_c, one conversion and one FMA a row and column on the
+//     pipe that the integers leave idle.  (A row of integers in units chosen from sigma and the largest
+//     datum, built again with larger ones where z outgrew them, took 3% less time with the gradient at m =
+//     60 and 7% less without where it fitted, and 60% and 85% more where it did not: n = 100k, white data
+//     under nu = 3/2, no nugget, 13.7 and 10.6 ms against 8.53 and 5.70.)
 // FP64's column-by-column update rounds entries of size 1 to 2^-54 at every step; here every
 // entry carries absolute errors of about 2^-58 and 2^-56.
 //
@@ -116,9 +121,9 @@ struct WordSlots {
 };
 
 // 1/sqrt(d) of a positive d < 2^62: with d 2^(2q) in [2^60, 2^62), 2^31 / sqrt(d 2^(2q)) =
-// (rh 2^31 + rl) 2^-60, in (1, 2].  FP32 seed y, then one third-order step y (1 + e/2 + 3
+// R 2^-60, in (1, 2].  FP32 seed y, then one third-order step y (1 + e/2 + 3
 // e^2/8), e = 1 - d y^2 in units of 2^-60 (|e| < 2^-20: the omitted 5 e^3/16 is below 2^-61).
-__device__ __forceinline__ void rsqrt_fixed(long long d, int& q, int& rh, int& rl) {
+__device__ __forceinline__ long long rsqrt_fixed(long long d, int& q) {
   q = (__clzll(d) - 2) >> 1;
   const long long dn = d << (2 * q);
   const float g = __int2float_rn((int)(dn >> 32)) * 0x1p-30f;  // d 2^(2q) / 2^62 in [1/4, 1]
@@ -134,19 +139,23 @@ __device__ __forceinline__ void rsqrt_fixed(long long d, int& q, int& rh, int& r
   const long long de = e + ((3LL * s) >> 14);         // (e/2 + 3 e^2/8) 2^61
   const long long R = ((long long)Y << 30) + (long long)Y * (int)(de >> 31) +
                       (((long long)Y * ((int)de & 0x7FFFFFFF)) >> 31);
-  rh = (int)(R >> 31);
-  rl = (int)R & 0x7FFFFFFF;
+  return R;
 }
 
-// A finite double times 2^sh as a 64-bit integer, rounded to nearest; the result must stay
-// below 2^62 in magnitude (sh chosen from the largest exponent).
+// A finite positive double times 2^sh as a 64-bit integer, rounded to nearest; the result must stay
+// below 2^62.
 __device__ __forceinline__ long long fixed_from_double(double x, int sh) {
   const long long b = __double_as_longlong(x);
   const int ef = (int)((b >> 52) & 0x7FF);
   const unsigned long long mant = (unsigned long long)((b & 0xFFFFFFFFFFFFFLL) | (ef ? 0x10000000000000LL : 0LL)) << 9;
   const int r = 9 - ((ef ? ef : 1) - 1075 + sh);  // x 2^sh = (mant << 9) >> r
-  const long long v = r <= 0 ? (long long)mant : r < 63 ? (long long)((mant + (1ull << (r - 1))) >> r) : 0LL;
-  return b < 0 ? -v : v;
+  return r <= 0 ? (long long)mant : r < 63 ? (long long)((mant + (1ull << (r - 1))) >> r) : 0LL;
+}
+
+// R 2^k for rsqrt_fixed's R in (2^60, 2^61], rounded to nearest; the pivot d 2^(2f - 60) has the
+// reciprocal square root R 2^(q - f - 61).
+__device__ __forceinline__ double pivot_scale(long long R, int k) {
+  return __longlong_as_double(((R + 128) >> 8) + ((long long)(1022 + 60 + k) << 52));
 }
 
 // x 2^k for any int k, by exact powers of two.
@@ -175,24 +184,8 @@ __device__ __forceinline__ long long scaled_entry(long long a, int q, int rh, in
   return f ? v >> min(f, 63) : v;
 }
 
-// Units of a block: f of the diagonal (see above) and ky of the data row, chosen so that z
-// stays below 2^(ky - 2) (every sum of products then fits in 64 bits): the entries are
-// standardised residuals times sigma, so there is room for 8 sigma (but no more than 2^12
-// above the largest datum).
-struct PanelScale {
-  int f = 0, ky = 0;
-  bool grown = false;      // an entry of z did not fit (warp-uniform)
-  bool nonfinite = false;  // a datum is not finite
-  __device__ __forceinline__ void init(unsigned ytop, const double sigma2, const double gamma1, int attempt) {
-    const int top = (int)__reduce_max_sync(0xffffffffu, ytop);
-    nonfinite = top == 0x7FF;
-    const int Ey = top - 1023;                                       // |y| < 2^(Ey + 1)
-    const int Es = (((int)exponent_field(sigma2) - 1023) >> 1) + 1;  // sigma < 2^Es
-    ky = max(Ey + 2, min(Es + 3, Ey + 12)) + 2 + 10 * attempt;
-    f = max(((int)exponent_field(gamma1) - 1023) >> 1, 0);
-    grown = false;
-  }
-};
+// f of the diagonal's units (see above).
+__device__ __forceinline__ int panel_shift(double gamma1) { return max(((int)exponent_field(gamma1) - 1023) >> 1, 0); }
 
 // A_rc -= sum_{k < c0} Lc_rk Lc_ck for the columns [c0, pe) of the panel and the sixteen rows
 // from rt on.  (Two row tiles at a time, which share the column operand's conversion, cost
@@ -200,8 +193,9 @@ struct PanelScale {
 __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, int rt, int c0, int pe, int f, int lane) {
   const int g = lane >> 2, t = lane & 3;
   const uint2* __restrict__ D = reinterpret_cast<const uint2*>(A);
-  const int rb = min(c0 + g, K);  // the panel's own rows: the MMA's columns
-  const int r0 = min(rt + g, K), r1 = min(rt + g + 8, K);
+  const int R = K - 1;            // the last row, the location's
+  const int rb = min(c0 + g, R);  // the panel's own rows: the MMA's columns
+  const int r0 = min(rt + g, R), r1 = min(rt + g + 8, R);
   float d[8][4];
 #pragma unroll
   for (int s = 0; s < 8; ++s)
@@ -249,7 +243,7 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
     const unsigned T = a[0] * 65536u + a[1] * 256u + a[2];
     long long sum = (long long)((unsigned long long)T << 32) + (long long)H * (1 << 16) + M;
     const int row = rt + g + 8 * (v >> 1), c = c0 + 2 * t + (v & 1);
-    if (row <= K && c < pe && row >= c) {
+    if (row <= R && c < pe && row >= c) {
       const int e = tri_off(K, c) + row - c;
       if (f && row == c) sum >>= min(2 * f, 63);
       A[e] -= sum;
@@ -258,28 +252,37 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
 }
 
 // The columns [c0, min(c0 + 8, K - 1)) of a panel, left-looking, a row per lane and slot (rows
-// c0 + lane and c0 + lane + 32): A becomes V there.  The corner {C_mm, C_Km} is returned in
-// corner when column m = K - 1 lies in the panel.  The high limbs' products are summed in 64
+// c0 + lane and c0 + lane + 32): A becomes V there.  C_mm is returned in corner when column
+// m = K - 1 lies in the panel.  The high limbs' products are summed in 64
 // bits, the mixed ones in units of 2^-56 (each rounded down, half a unit on average, which
-// the start values give back).  Returns whether the block can still be positive definite.
-// With CTA only the panel's own rows (of the last panel: all), and the pivots' reciprocals
-// are left in piv for panel_row.
+// the start values give back).  The data of the lane's rows (slots (K, r) of the triangle) take each
+// column's z_c times the row's entry off, and column c's own slot is left z_c / sqrt(d_c), the unit factor's
+// entry.  Returns whether the block can still be positive definite.
+// With CTA only the panel's own rows (of the last panel: all), and the pivots' reciprocals and the z_c 2^-62
+// are left in piv and zs for panel_row.
 template <bool GRAD, bool CTA>
 __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, float2* __restrict__ RJ,
-                                              int4* __restrict__ piv, int c0, int f, bool& grown,
-                                              long long (&corner)[2], int lane) {
-  const int rmax = CTA && c0 + kPanelCols < K ? c0 + kPanelCols - 1 : K;
+                                              int4* __restrict__ piv, double* __restrict__ zs, int c0, int f,
+                                              long long& corner, int lane) {
+  const int R = K - 1;
+  const int rmax = CTA && c0 + kPanelCols < K ? c0 + kPanelCols - 1 : R;
   const int last = K - 1 - c0;    // panel position of column m
   const int jn = min(last + 1, kPanelCols);
   const int r0 = c0 + lane, r1 = r0 + 32;
-  const bool two = !CTA && c0 + 32 <= K;  // warp-uniform
-  int over = 0, grow = 0;
+  const bool two = !CTA && c0 + 32 <= R;  // warp-uniform
+  int over = 0;
   bool ok = true;
   const int2* __restrict__ V = reinterpret_cast<const int2*>(A);
+  double* __restrict__ Y = reinterpret_cast<double*>(A);
+  const int y0s = tri_off(K, min(r0, R)) + K - min(r0, R), y1s = tri_off(K, min(r1, R)) + K - min(r1, R);
+  // The data: column j's z_j goes round (through the triangle's unused slot 0) after its V, and is taken off
+  // the rows in the next column, where the FP64 pipe's latency hides behind the integers.
+  double y0 = Y[y0s], y1 = two ? Y[y1s] : 0.0;
+  double v0 = 0.0, v1 = 0.0, z = 0.0, scale = 0.0;
 #pragma unroll 1
   for (int j = 0; j < jn; ++j) {
     const int oj = tri_off(K, c0 + j) - (c0 + j);
-    const int q0 = min(max(r0, c0 + j), rmax), q1 = min(r1, K);
+    const int q0 = min(max(r0, c0 + j), rmax), q1 = min(r1, R);
     long long s0 = 0, s1 = 0;
     int m0 = j, m1 = j;
     int ok_ = tri_off(K, c0) - c0, step = K - c0;  // slot of (row 0, column c0 + k)
@@ -299,12 +302,13 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       ok_ -= step + 1;
       --step;
     }
+    y0 = fma(-v0, z, y0);
+    if (two) y1 = fma(-v1, z, y1);
     s0 += (long long)m0 * 16;
     if (f && lane == j) s0 >>= min(2 * f, 63);
     const long long a0 = r0 >= c0 + j && r0 <= rmax ? A[oj + q0] - s0 : 0;
     if (j == last) {
-      corner[0] = __shfl_sync(0xffffffffu, a0, j);
-      corner[1] = __shfl_sync(0xffffffffu, a0, j + 1);
+      corner = __shfl_sync(0xffffffffu, a0, j);
       break;
     }
     long long d = __shfl_sync(0xffffffffu, a0, j);
@@ -312,62 +316,59 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       ok = false;
       d = 1LL << 60;
     }
-    int q, rh, rl;
-    rsqrt_fixed(d, q, rh, rl);
+    int q;
+    const long long pr = rsqrt_fixed(d, q);
+    const int rh = (int)(pr >> 31), rl = (int)pr & 0x7FFFFFFF;
     if (CTA && lane == 0) piv[j] = make_int4(q, rh, rl, 0);
-    if (GRAD && lane == 0) {  // 2^-62 / sqrt(d), the factor that makes V a unit-lower entry
-      const float h = __int2float_rz(rh);
-      const float lo = __int2float_rn(rh - (int)h) + __int2float_rn(rl) * 0x1p-31f;
-      const int se = 127 + q - 30 - 62 - f;  // below the floats' range past gamma = 2^70: 0
-      const float sc = se > 0 ? __uint_as_float((unsigned)se << 23) : 0.0f;
-      const float hs = h + lo;
-      RJ[c0 + j] = make_float2(hs * sc, (lo - (hs - h)) * sc);
-    }
-    // V of this lane's rows; |V| >= 2^62 2^-f: not a positive definite block, or, in the data
-    // row, |z| too large for its units
-    const int lim = max(29 - q, 0), ylim = max(27 - q, 0);
+    const double rs = pivot_scale(pr, q - f - 61 - 62);  // 2^-62 / sqrt(d)
+    const double zj = y0 * rs;  // lane j: z_j 2^-62
+    if (GRAD && lane == j) scale = rs;
+    // V of this lane's rows; |V| >= 2^62 2^-f: not a positive definite block
+    const int lim = max(29 - q, 0);
     __syncwarp();  // the pivot row's entries of this column are read
+    if (GRAD) v0 = 0.0;  // (without, the eliminated rows' data are not used again)
     if (lane > j && r0 <= rmax) {
-      if (r0 == K) grow |= top_magnitude(a0) >> ylim;
-      else over |= top_magnitude(a0) >> lim;
-      A[oj + r0] = scaled_entry(a0, q, rh, rl, f);
+      over |= top_magnitude(a0) >> lim;
+      const long long v = scaled_entry(a0, q, rh, rl, f);
+      A[oj + r0] = v;
+      v0 = (double)v;
     }
     if (two) {
       s1 += (long long)m1 * 16;
       const long long a1 = A[oj + q1] - s1;
-      if (r1 == K) grow |= top_magnitude(a1) >> ylim;
-      else if (r1 < K) over |= top_magnitude(a1) >> lim;
-      if (r1 <= K) A[oj + r1] = scaled_entry(a1, q, rh, rl, f);
-    }
-    if (!CTA && K == c0 + 64) {  // a 65-row panel (m = 63): its last row, the data row, on lane 0
-      long long s2 = 0;
-      int m2 = j;
-      int o2 = tri_off(K, c0) - c0;
-      for (int k = 0; k < j; ++k) {
-        const int2 p = V[o2 + c0 + j], x = V[o2 + K];
-        s2 += (long long)x.y * p.y;
-        m2 = mad_hi(x.y, (int)((unsigned)p.x >> 4), m2);
-        m2 = mad_hi((int)((unsigned)x.x >> 4), p.y, m2);
-        o2 -= K - c0 - k + 1;
-      }
-      const long long a2 = A[oj + K] - s2 - (long long)m2 * 16;
-      __syncwarp();
-      if (lane == 0) {
-        grow |= top_magnitude(a2) >> ylim;
-        A[oj + K] = scaled_entry(a2, q, rh, rl, f);
+      if (r1 <= R) {
+        over |= top_magnitude(a1) >> lim;
+        const long long v = scaled_entry(a1, q, rh, rl, f);
+        A[oj + r1] = v;
+        v1 = (double)v;
       }
     }
+    double* const at = CTA ? zs + j : Y;
+    if (lane == j) *at = zj;
     __syncwarp();
+    z = *at;
   }
-  grown = grown || __any_sync(0xffffffffu, grow != 0);
+  if (c0 + kPanelCols <= R) {  // (the last panel's last column takes nothing off)
+    y0 = fma(-v0, z, y0);
+    if (two) y1 = fma(-v1, z, y1);
+  }
+  if (r0 <= rmax) {
+    if (r0 >= c0 + kPanelCols || r0 == R) Y[y0s] = y0;
+    else if (GRAD) Y[y0s] = y0 * (scale * 0x1p62) * (scale * 0x1p62);
+    if (GRAD && r0 < min(c0 + kPanelCols, R)) RJ[r0] = d2f_trunc(scale);
+  }
+  if (two && r1 <= R) Y[y1s] = y1;
+  __syncwarp();
   return ok && !__any_sync(0xffffffffu, over != 0);
 }
 
 // Row r below the panel [c0, c0 + 8), by one thread: its eight entries of the factor, from the
-// panel's own rows and pivots, and then their digits, in place.
-__device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, const int4* __restrict__ piv, int c0, int f,
-                                          int r, int& over, int& grow) {
+// panel's own rows and pivots, and then their digits, in place; and its datum.
+__device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, const int4* __restrict__ piv,
+                                          const double* __restrict__ zs, int c0, int f, int r, int& over) {
   const int2* __restrict__ V = reinterpret_cast<const int2*>(A);
+  double* __restrict__ Y = reinterpret_cast<double*>(A) + tri_off(K, r) + K - r;
+  double y = *Y, v0 = 0.0, z = 0.0;
 #pragma unroll 1
   for (int j = 0; j < kPanelCols; ++j) {
     long long s0 = 0;
@@ -382,12 +383,16 @@ __device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, cons
       ok_ -= step + 1;
       --step;
     }
+    y = fma(-v0, z, y);
     const int4 pv = piv[j];
     const long long a = A[ok_ + r] - s0 - (long long)m0 * 16;
-    if (r == K) grow |= top_magnitude(a) >> max(27 - pv.x, 0);
-    else over |= top_magnitude(a) >> max(29 - pv.x, 0);
-    A[ok_ + r] = scaled_entry(a, pv.x, pv.y, pv.z, f);
+    over |= top_magnitude(a) >> max(29 - pv.x, 0);
+    const long long v = scaled_entry(a, pv.x, pv.y, pv.z, f);
+    A[ok_ + r] = v;
+    v0 = (double)v;
+    z = zs[j];
   }
+  *Y = fma(-v0, z, y);
 #pragma unroll 1
   for (int k0 = c0; k0 < c0 + kPanelCols; k0 += 4) {
     const WordSlots w(K, k0);
@@ -405,7 +410,7 @@ __device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, cons
 __device__ __forceinline__ void panel_to_digits(int K, long long* __restrict__ A, int c0, int lane) {
   const int r0 = c0 + kPanelCols;
 #pragma unroll 1
-  for (int u = lane; u < kPanelWords * (K + 1 - r0); u += 32) {  // (row, word)
+  for (int u = lane; u < kPanelWords * (K - r0); u += 32) {  // (row, word)
     const int r = r0 + u / kPanelWords, k0 = c0 + 4 * (u % kPanelWords);
     const WordSlots w(K, k0);
     long long v[4];
@@ -421,52 +426,56 @@ __device__ __forceinline__ void panel_to_digits(int K, long long* __restrict__ A
 
 // Cholesky over the neighbour columns.  Returns whether the block is positive definite.
 template <bool GRAD>
-__device__ __forceinline__ bool panels_eliminate(int K, long long* __restrict__ A, float2* __restrict__ RJ, PanelScale& ysc,
-                                                 long long (&corner)[2], int lane) {
+__device__ __forceinline__ bool panels_eliminate(int K, long long* __restrict__ A, float2* __restrict__ RJ, int f,
+                                                 long long& corner, int lane) {
   bool ok = true;
 #pragma unroll 1
   for (int c0 = 0; c0 < K; c0 += kPanelCols) {
     const int pe = min(c0 + kPanelCols, K);
     if (c0 > 0) {
 #pragma unroll 1
-      for (int rt = c0; rt <= K; rt += 16) update_tile(K, A, rt, c0, pe, ysc.f, lane);
+      for (int rt = c0; rt < K; rt += 16) update_tile(K, A, rt, c0, pe, f, lane);
       __syncwarp();
     }
-    const bool o = panel_columns<GRAD, false>(K, A, RJ, nullptr, c0, ysc.f, ysc.grown, corner, lane);
+    const bool o = panel_columns<GRAD, false>(K, A, RJ, nullptr, nullptr, c0, f, corner, lane);
     ok = ok && o;
     if (pe < K) panel_to_digits(K, A, c0, lane);
   }
   return ok;
 }
 
-// V 2^-62 / sqrt(d) 2^(unit's exponent) as a float pair, rj = 2^-62 / sqrt(d).
-__device__ __forceinline__ float2 unit_pair(long long v, float2 rj, float unit) {
+// V 2^-62 / sqrt(d) as a float pair, rj = 2^-62 / sqrt(d).
+__device__ __forceinline__ float2 unit_pair(long long v, float2 rj) {
   // v = a 2^39 + b 2^23 + c, each an exact float
   const float fa = __int2float_rn((int)(v >> 39)) * 0x1p39f;
   const float fb = __int2float_rn((int)(v >> 23) & 0xFFFF) * 0x1p23f;
   const float fc = __int2float_rn((int)((unsigned)v & 0x7FFFFFu));
-  float vh, vl, oh, ol;
+  float vh, vl;
+  float2 o;
   fast_two_sum(fa, fb, vh, vl);
-  df_mul(vh, __fadd_rn(vl, fc), rj.x, rj.y, oh, ol);
-  return make_float2(oh * unit, ol * unit);
+  df_mul(vh, __fadd_rn(vl, fc), rj.x, rj.y, o.x, o.y);
+  return o;
 }
 
 // After the elimination, for the adjoint: every entry of the factor below the diagonal
-// (neighbour columns) becomes a float pair of the unit factor in its place.  By nth threads.
-__device__ __forceinline__ void panels_to_pairs(int K, long long* __restrict__ A, const float2* __restrict__ RJ,
-                                                const PanelScale& ysc, int tid, int nth) {
+// (neighbour columns) becomes a float pair of the unit factor in its place, those of the data row too.
+// By nth threads.
+__device__ __forceinline__ void panels_to_pairs(int K, long long* __restrict__ A, const float2* __restrict__ RJ, int tid,
+                                                int nth) {
   float2* __restrict__ P = reinterpret_cast<float2*>(A);
-  const float yunit = __uint_as_float((unsigned)(min(max(ysc.ky, -126), 127) + 127) << 23);
+  for (int c = tid; c < K - 1; c += nth) {
+    const int e = tri_off(K, c) + K - c;
+    P[e] = d2f_trunc(reinterpret_cast<const double*>(A)[e]);
+  }
 #pragma unroll 1
   for (int c0 = 0; c0 < K - 1; c0 += kPanelCols) {
     // below the panel: digits, one (row, word) per lane; in it (and all of the last panel): V
     const bool lastp = c0 + kPanelCols >= K;
-    const int rb = lastp ? K + 1 : c0 + kPanelCols;
+    const int rb = lastp ? K : c0 + kPanelCols;
 #pragma unroll 1
-    for (int u = tid; u < kPanelWords * (K + 1 - c0); u += nth) {
+    for (int u = tid; u < kPanelWords * (K - c0); u += nth) {
       const int r = c0 + u / kPanelWords, k0 = c0 + 4 * (u % kPanelWords);
       const WordSlots ws(K, k0);
-      const float unit = r == K ? yunit : 1.0f;
       unsigned w[8];
       if (r >= rb) {
 #pragma unroll
@@ -481,7 +490,7 @@ __device__ __forceinline__ void panels_to_pairs(int K, long long* __restrict__ A
         const int c = k0 + x;
         if (r > c && c < K - 1) {
           const long long v = r >= rb ? planes_value(w, x) : A[ws.e[x] + r];
-          P[ws.e[x] + r] = unit_pair(v, RJ[c], unit);
+          P[ws.e[x] + r] = unit_pair(v, RJ[c]);
         }
       }
     }

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
     // ---- the term, on warp 0 (FP64)
     const double nan = __longlong_as_double(0x7FF8000000000000LL);
     if (wid == 0) {
-      const double st = mul_pow2((double)*corner, 2 * f - 60), rr = A[2];
+      const double st = *corner > kSmallestPivot ? mul_pow2((double)*corner, 2 * f - 60) : 0.0, rr = A[2];
       const bool pd = ok && positive_finite(st);  // a non-finite rr with pd: non-finite data
       const bool good = pd && finite_bits(rr) && !bad_idx;
       const double s = tc.sigma2 * st;

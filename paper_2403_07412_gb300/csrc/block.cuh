@@ -716,8 +716,9 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     __syncwarp();
   }
   }
-  const double st = kPanels ? mul_pow2((double)corner, 2 * f - 60) : A[1];  // s_i / sigma2
-  const double rr = A[2];                                                    // y_i - mu_i
+  // s_i / sigma2
+  const double st = !kPanels ? A[1] : corner > kSmallestPivot ? mul_pow2((double)corner, 2 * f - 60) : 0.0;
+  const double rr = A[2];  // y_i - mu_i
   // The pivots and s_i depend on the covariance only, the residual on the data: a
   // non-finite residual (with a positive definite block) means a non-finite y in B_i.
   const bool pd = ok && positive_finite(st);

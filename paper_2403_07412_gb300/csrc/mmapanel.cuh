@@ -20,7 +20,7 @@
 //     60 and 7% less without where it fitted, and 60% and 85% more where it did not: n = 100k, white data
 //     under nu = 3/2, no nugget, 13.7 and 10.6 ms against 8.53 and 5.70.)
 // FP64's column-by-column update rounds entries of size 1 to 2^-54 at every step; here every
-// entry carries absolute errors of about 2^-58 and 2^-56.
+// entry carries an absolute error of about 2^-58.
 //
 // Updates between panels: A_rc -= sum_{k < c0} Lc_rk Lc_ck, for the eight columns of the next
 // panel at once, as exact products of integers.  V is stored as its eight bytes, V +
@@ -30,7 +30,7 @@
 // accumulator's bits.  (A row's entries have squares that add up to at most 1, which bounds the
 // sums of the leading digits, and the digits below spread over their range: 8 pairs of 150
 // columns add up with a standard deviation below 2^18, or 2^20.7 in one pair where the two rows
-// are the same.)  Kept are i <= 7, j <= 6, i + j <= 7.
+// are the same.)  Kept are the pairs i + j <= 7; the dropped ones add up to a few units of 2^-60.
 //
 // The bytes take the factor entries' own places: the four entries (r, 4w .. 4w+3) of a row
 // become eight words, one per digit plane, each with the digit of the four columns; so the
@@ -53,6 +53,13 @@ namespace vecchia {
 constexpr int kPanelCols = 8;
 constexpr int kPanelWords = kPanelCols / 4;
 constexpr unsigned long long kByteBias = 0x8080808080808080ull;
+// A pivot, or s_i / sigma2, at or below 2^-53 of the variance (in units of 2^-60) counts as zero: the block is not
+// positive definite.  Two coincident points without a nugget leave a Schur complement that is exactly 0; the
+// rows are eliminated alike but for where a column's products are summed, on the tensor cores or in a
+// panel, so what is left of it is the rounding of one panel's fourteen mixed products (28 units at
+// most, 6 as a rule), of the dropped digits (some 3) and of V (2).  The smallest nugget that
+// FP64 tells from none leaves twice the threshold.
+constexpr long long kSmallestPivot = 128;
 constexpr float kAccZero = 12582912.0f;  // 1.5 2^23
 constexpr unsigned kAccZeroBits = 0x4B400000u;
 
@@ -217,9 +224,9 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
 #pragma unroll
       for (int i = 0; i < 4; ++i) x[i] = y[i] = z[i] = make_uint2(0x80808080u, 0x80808080u);
     }
-    unsigned bf[7][2];
+    unsigned bf[8][2];
 #pragma unroll
-    for (int j = 0; j < 7; ++j) {
+    for (int j = 0; j < 8; ++j) {
       const unsigned v = j & 1 ? z[j >> 1].y : z[j >> 1].x;
       bf[j][0] = digit_pair(v, 0x4140);
       bf[j][1] = digit_pair(v, 0x4342);
@@ -229,7 +236,7 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
       const unsigned u = i & 1 ? x[i >> 1].y : x[i >> 1].x, v = i & 1 ? y[i >> 1].y : y[i >> 1].x;
       const unsigned af[4] = {digit_pair(u, 0x4140), digit_pair(v, 0x4140), digit_pair(u, 0x4342), digit_pair(v, 0x4342)};
 #pragma unroll
-      for (int j = 0; j < 7; ++j)
+      for (int j = 0; j < 8; ++j)
         if (i + j < 8) mma_f16(d[i + j], af, bf[j]);
     }
   }
@@ -254,8 +261,9 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
 // The columns [c0, min(c0 + 8, K - 1)) of a panel, left-looking, a row per lane and slot (rows
 // c0 + lane and c0 + lane + 32): A becomes V there.  C_mm is returned in corner when column
 // m = K - 1 lies in the panel.  The high limbs' products are summed in 64
-// bits, the mixed ones in units of 2^-56 (each rounded down, half a unit on average, which
-// the start values give back).  The data of the lane's rows (slots (K, r) of the triangle) take each
+// bits, the mixed ones in units of 2^-58 (each rounded down, half a unit on average, which
+// the start values give back; a row's entries have squares that add up to at most 1, so that seven
+// columns' stay below 2^31).  The data of the lane's rows (slots (K, r) of the triangle) take each
 // column's z_c times the row's entry off, and column c's own slot is left z_c / sqrt(d_c), the unit factor's
 // entry.  Returns whether the block can still be positive definite.
 // With CTA only the panel's own rows (of the last panel: all), and the pivots' reciprocals and the z_c 2^-62
@@ -289,22 +297,22 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
 #pragma unroll 1
     for (int k = 0; k < j; ++k) {
       const int2 p = V[ok_ + c0 + j], x = V[ok_ + q0];
-      const int lp = (int)((unsigned)p.x >> 4);
+      const int lp = (int)((unsigned)p.x >> 2);
       s0 += (long long)x.y * p.y;
       m0 = mad_hi(x.y, lp, m0);
-      m0 = mad_hi((int)((unsigned)x.x >> 4), p.y, m0);
+      m0 = mad_hi((int)((unsigned)x.x >> 2), p.y, m0);
       if (two) {
         const int2 y = V[ok_ + q1];
         s1 += (long long)y.y * p.y;
         m1 = mad_hi(y.y, lp, m1);
-        m1 = mad_hi((int)((unsigned)y.x >> 4), p.y, m1);
+        m1 = mad_hi((int)((unsigned)y.x >> 2), p.y, m1);
       }
       ok_ -= step + 1;
       --step;
     }
     y0 = fma(-v0, z, y0);
     if (two) y1 = fma(-v1, z, y1);
-    s0 += (long long)m0 * 16;
+    s0 += (long long)m0 * 4;
     if (f && lane == j) s0 >>= min(2 * f, 63);
     const long long a0 = r0 >= c0 + j && r0 <= rmax ? A[oj + q0] - s0 : 0;
     if (j == last) {
@@ -312,7 +320,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       break;
     }
     long long d = __shfl_sync(0xffffffffu, a0, j);
-    if (d <= 0) {  // a failed block runs on (values unused)
+    if (d <= kSmallestPivot) {  // a failed block runs on (values unused)
       ok = false;
       d = 1LL << 60;
     }
@@ -334,7 +342,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       v0 = (double)v;
     }
     if (two) {
-      s1 += (long long)m1 * 16;
+      s1 += (long long)m1 * 4;
       const long long a1 = A[oj + q1] - s1;
       if (r1 <= R) {
         over |= top_magnitude(a1) >> lim;
@@ -378,14 +386,14 @@ __device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, cons
     for (int k = 0; k < j; ++k) {
       const int2 p = V[ok_ + c0 + j], x = V[ok_ + r];
       s0 += (long long)x.y * p.y;
-      m0 = mad_hi(x.y, (int)((unsigned)p.x >> 4), m0);
-      m0 = mad_hi((int)((unsigned)x.x >> 4), p.y, m0);
+      m0 = mad_hi(x.y, (int)((unsigned)p.x >> 2), m0);
+      m0 = mad_hi((int)((unsigned)x.x >> 2), p.y, m0);
       ok_ -= step + 1;
       --step;
     }
     y = fma(-v0, z, y);
     const int4 pv = piv[j];
-    const long long a = A[ok_ + r] - s0 - (long long)m0 * 16;
+    const long long a = A[ok_ + r] - s0 - (long long)m0 * 4;
     over |= top_magnitude(a) >> max(29 - pv.x, 0);
     const long long v = scaled_entry(a, pv.x, pv.y, pv.z, f);
     A[ok_ + r] = v;

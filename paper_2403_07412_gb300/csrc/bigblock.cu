@@ -87,7 +87,7 @@ __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, 
         __threadfence_block();
         asm volatile("bar.arrive 1, %0;" ::"r"(NTH) : "memory");
         __syncwarp();
-        update_tile(K, A, c1, c1, pe, f, lane);
+        update_tile<true>(K, A, c1, c1, pe, f, lane);
         __syncwarp();
       }
       long long cr = 0;
@@ -98,7 +98,7 @@ __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, 
       for (int r = c1 + 16 + tid - 32; r < K; r += NTH - 32) panel_row(K, A, pv, pz, c0, f, r, over);
       asm volatile("bar.sync 1, %0;" ::"r"(NTH) : "memory");
 #pragma unroll 1
-      for (int rt = c1 + 16 * wid; rt < K; rt += (NTH - 32) / 2) update_tile(K, A, rt, c1, pe, f, lane);
+      for (int rt = c1 + 16 * wid; rt < K; rt += (NTH - 32) / 2) update_tile<true>(K, A, rt, c1, pe, f, lane);
     }
     __syncthreads();
   }

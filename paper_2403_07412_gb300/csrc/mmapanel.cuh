@@ -25,12 +25,13 @@
 // Updates between panels: A_rc -= sum_{k < c0} Lc_rk Lc_ck, for the eight columns of the next
 // panel at once, as exact products of integers.  V is stored as its eight bytes, V +
 // 0x8080808080808080 = sum_i b_i 256^(7-i): digits d_i = b_i - 128, each a half exactly.  The
-// products d_i d'_j of one diagonal i + j = s add up to integers that an FP32 accumulator holds
-// exactly up to 2^22; it starts at 1.5 2^23, so that the integer is read off the
-// accumulator's bits.  (A row's entries have squares that add up to at most 1, which bounds the
-// sums of the leading digits, and the digits below spread over their range: 8 pairs of 150
-// columns add up with a standard deviation below 2^18, or 2^20.7 in one pair where the two rows
-// are the same.)  Kept are the pairs i + j <= 7; the dropped ones add up to a few units of 2^-60.
+// products d_i d'_j of one diagonal i + j = s add up to integers, which an FP32 accumulator holds
+// exactly below 2^24.  With c0 columns a pair of digits adds up to at most 2^14 c0, or, where one is d_0 =
+// 64 Lc rounded (a row's squares add up to at most 1), 2^13 sqrt(c0); of the eight pairs of s = 7, six of
+// the first kind.  Up to m = 150 (c0 <= 144) that is 2^23.8, so every sum is exact.  Up to 63 (c0 <=
+// 56) the sums to s = 5 stay below 2^22 too: they start at 1.5 2^23, so that the integer is read off the
+// accumulator's bits, without a conversion (all converted: n = 100k, m = 60 with the gradient 8.57 -> 8.69
+// ms).  Kept are the pairs i + j <= 7; the dropped ones add up to a few units of 2^-60.
 //
 // The bytes take the factor entries' own places: the four entries (r, 4w .. 4w+3) of a row
 // become eight words, one per digit plane, each with the digit of the four columns; so the
@@ -195,8 +196,9 @@ __device__ __forceinline__ long long scaled_entry(long long a, int q, int rh, in
 __device__ __forceinline__ int panel_shift(double gamma1) { return max(((int)exponent_field(gamma1) - 1023) >> 1, 0); }
 
 // A_rc -= sum_{k < c0} Lc_rk Lc_ck for the columns [c0, pe) of the panel and the sixteen rows
-// from rt on.  (Two row tiles at a time, which share the column operand's conversion, cost
+// from rt on; WIDE where c0 may exceed 56.  (Two row tiles at a time, which share the column operand's conversion, cost
 // more in registers and code than they save.)
+template <bool WIDE>
 __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, int rt, int c0, int pe, int f, int lane) {
   const int g = lane >> 2, t = lane & 3;
   const uint2* __restrict__ D = reinterpret_cast<const uint2*>(A);
@@ -207,7 +209,7 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
 #pragma unroll
   for (int s = 0; s < 8; ++s)
 #pragma unroll
-    for (int v = 0; v < 4; ++v) d[s][v] = kAccZero;
+    for (int v = 0; v < 4; ++v) d[s][v] = WIDE || s > 5 ? 0.0f : kAccZero;
 #pragma unroll 1
   for (int kb = 0; kb < c0; kb += 16) {
     const int k0 = kb + 4 * t;  // this lane's four columns; past the last panel: zeros
@@ -243,12 +245,14 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
   // sum_s acc_s 2^(48 - 8s), in units of 2^-60
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    unsigned a[8];
+    int a[8];
 #pragma unroll
-    for (int s = 0; s < 8; ++s) a[s] = __float_as_uint(d[s][v]) - kAccZeroBits;
-    const int H = (int)(a[3] * 256u + a[4]), M = (int)(a[5] * 256u + a[6]) + ((int)a[7] >> 8);
-    const unsigned T = a[0] * 65536u + a[1] * 256u + a[2];
-    long long sum = (long long)((unsigned long long)T << 32) + (long long)H * (1 << 16) + M;
+    for (int s = 0; s < 7; ++s)
+      a[s] = WIDE || s > 5 ? __float2int_rn(d[s][v]) : (int)(__float_as_uint(d[s][v]) - kAccZeroBits);
+    a[7] = (int)(__float_as_uint(__fadd_rn(d[7][v], 256.0f * kAccZero)) - kAccZeroBits - (8u << 23));  // to units of 2^8
+    const unsigned T = (unsigned)a[0] * 65536u + (unsigned)a[1] * 256u + (unsigned)a[2];
+    long long sum = (long long)((unsigned long long)T << 32) + (long long)a[3] * (1 << 24) + (long long)a[4] * (1 << 16) +
+                    (long long)a[5] * 256 + (a[6] + a[7]);
     const int row = rt + g + 8 * (v >> 1), c = c0 + 2 * t + (v & 1);
     if (row <= R && c < pe && row >= c) {
       const int e = tri_off(K, c) + row - c;
@@ -442,7 +446,7 @@ __device__ __forceinline__ bool panels_eliminate(int K, long long* __restrict__ 
     const int pe = min(c0 + kPanelCols, K);
     if (c0 > 0) {
 #pragma unroll 1
-      for (int rt = c0; rt < K; rt += 16) update_tile(K, A, rt, c0, pe, f, lane);
+      for (int rt = c0; rt < K; rt += 16) update_tile<false>(K, A, rt, c0, pe, f, lane);
       __syncwarp();
     }
     const bool o = panel_columns<GRAD, false>(K, A, RJ, nullptr, nullptr, c0, f, corner, lane);

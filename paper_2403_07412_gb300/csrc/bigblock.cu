@@ -105,6 +105,123 @@ __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, 
   return __syncthreads_or(over) == 0;
 }
 
+// B columns j..j+B-1 of the bordered L D L^T, CTA-wide.  Each column in turn is scaled by
+// its pivot's reciprocal (its unscaled entries kept in TVs[q]) and applied to the later
+// columns of the group; then one pass over the remaining prefix [1, o_{j+B-1}) applies
+// all B columns to each slot in column order, fma(-L_q T_q, .) for q = 0..B-1.  Every
+// slot sees the same roundings in the same order as with single-column steps, while the
+// trailing matrix is read and written once per B columns.  Returns false (uniformly over
+// the CTA) at a pivot outside rcp_fixed's domain or that counts as zero.
+template <int B>
+__device__ __forceinline__ bool cta_columns(double* A, double* const* TVs, int K, int j, int tid, int NTH) {
+  int o[B];
+#pragma unroll
+  for (int q = 0; q < B; ++q) o[q] = tri_off(K, j + q);
+#pragma unroll
+  for (int q = 0; q < B; ++q) {
+    const double d = A[o[q]];
+    if (!pivot_in_range(d) || zero_pivot(d)) return false;  // every thread reads the same pivot
+    const double inv = rcp_fixed(d);
+    double* T = TVs[q];
+    for (int r = j + q + 1 + tid; r <= K; r += NTH) {
+      const double tv = A[o[q] + r - j - q];
+      T[r] = tv;
+      A[o[q] + r - j - q] = tv * inv;
+    }
+    __syncthreads();
+    if (q + 1 < B) {
+      const double* Lq = A + o[q] - j - q;
+#pragma unroll
+      for (int p = q + 1; p < B; ++p) {
+        const double tp = T[j + p];
+        for (int r = j + p + tid; r <= K; r += NTH) {
+          const int e = o[p] + r - j - p;
+          A[e] = fma(-Lq[r], tp, A[e]);
+        }
+      }
+      __syncthreads();
+    }
+  }
+  const double* L[B];
+#pragma unroll
+  for (int q = 0; q < B; ++q) L[q] = A + o[q] - j - q;
+  constexpr int U = 8 / B;
+  const int end = o[B - 1];
+  const int nfull = (end - 1) / (NTH * U);
+  const int tail0 = 1 + NTH * U * nfull;
+  for (int bt = 0; bt < nfull; ++bt) {
+    const int base = 1 + tid + NTH * U * bt;
+    double av[U];
+    int rr[U], cc[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int e = base + NTH * k;
+      const int w = tri_root(e);
+      cc[k] = K - w;
+      rr[k] = cc[k] + (e - w * (w + 1) / 2);
+      av[k] = A[e];
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+#pragma unroll
+      for (int k = 0; k < U; ++k) av[k] = fma(-L[q][rr[k]], TVs[q][cc[k]], av[k]);
+#pragma unroll
+    for (int k = 0; k < U; ++k) A[base + NTH * k] = av[k];
+  }
+  for (int e = tail0 + tid; e < end; e += NTH) {
+    const int w = tri_root(e);
+    const int c = K - w, r = c + (e - w * (w + 1) / 2);
+    double a = A[e];
+#pragma unroll
+    for (int q = 0; q < B; ++q) a = fma(-L[q][r], TVs[q][c], a);
+    A[e] = a;
+  }
+  __syncthreads();
+  return true;
+}
+
+// The block in FP64 (mmapanel.cuh says which blocks): assembly, L D L^T four columns at a time, then two, then
+// one, and (GRAD) the factor as float pairs, as panels_to_pairs leaves it.  Returns whether the neighbours'
+// block is positive definite; s_i / sigma2 and y_i - mu_i are in A[1] and A[2].  The data are in the border
+// row; TV and the vectors before and after it are column buffers.  (A function of its own, for the registers
+// of its caller.)
+template <bool GRAD, bool SPHERE>
+static __device__ __noinline__ bool cta_fp64_block(int K, int mi, double* A, const float2* CX, const float2* CY,
+                                                   const float2* CZ, double* TV, int stride, double gamma1, float2 k2,
+                                                   double k2d, const double* __restrict__ tab) {
+  const int m = K - 1, NP = K * (K - 1) / 2, tid = threadIdx.x, NTH = blockDim.x;
+  const MaternConst mc = matern_const_at(fix_const(tab));
+  FieldView F;
+  F.k2 = k2;
+  F.k2d = k2d;
+  for (int c = tid; c < K; c += NTH) {
+    const int o = tri_off(K, c);
+    A[o] = (c >= mi && c < m) ? 1.0 : gamma1;
+  }
+#pragma unroll 1
+  for (int q = tid; q < NP; q += NTH) {
+    const int v = tri_root(q), c = K - 2 - v, r = c + 1 + (q - v * (v + 1) / 2);
+    float uh, ul;
+    pair_u<SPHERE>(F, CX, CY, CZ, r, c, uh, ul);
+    A[tri_off(K, c) + r - c] = c < mi && (r < mi || r == m) ? fixed_to_double(rho_fixed62(uh, ul, tab, mc)) : 0.0;
+  }
+  __syncthreads();
+  double* TVs[4] = {TV, TV - stride, TV + stride, TV + 2 * stride};
+  bool ok = true;
+  int j = 0;
+  for (; ok && j + 4 < K; j += 4) ok = cta_columns<4>(A, TVs, K, j, tid, NTH);
+  for (; ok && j + 2 < K; j += 2) ok = cta_columns<2>(A, TVs, K, j, tid, NTH);
+  if (ok && j + 1 < K) ok = cta_columns<1>(A, TVs, K, j, tid, NTH);
+  if (GRAD) {
+    for (int e = 3 + tid; e < (K + 1) * (K + 2) / 2; e += NTH) {
+      const int w = tri_root(e);
+      if (e > w * (w + 1) / 2) reinterpret_cast<float2*>(A)[e] = d2f_trunc(A[e]);
+    }
+    __syncthreads();
+  }
+  return ok;
+}
+
 template <bool GRAD, bool SPHERE>
 __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigArgs a) {
   asm volatile("griddepcontrol.launch_dependents;");  // the reduction of the records
@@ -188,6 +305,21 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
     }
     if (kChecked) bad_idx = __syncthreads_or(bad_idx) != 0;
     __syncthreads();
+    // whether few of the data are large (each warp for itself)
+    int top = lane == 0 ? (int)exponent_field(YV[m]) : 0, count = 0;  // twice the large ones, less all but the zeros
+    for (int p = lane; p < mi; p += 32) top = max(top, (int)exponent_field(YV[p]));
+    top = __reduce_max_sync(0xffffffffu, top);
+    for (int p = lane; p <= m; p += 32) {
+      const int e = p < mi || p == m ? (int)exponent_field(YV[p]) : 0;
+      if (e > 0) count += large_datum(e, top) ? 1 : -1;
+    }
+    bool exact = f > kMostShift || __reduce_add_sync(0xffffffffu, count) < 0;  // the block goes to cta_fp64_block
+    if (GRAD) {
+      unsigned near = __float_as_uint(INFINITY);  // u of the nearest neighbour
+      for (int p = lane; p < mi; p += 32) near = min(near, __float_as_uint(sq_offset<SPHERE>(CX, CY, CZ, p)));
+      near = __reduce_min_sync(0xffffffffu, near);
+      exact = exact || rho_below(scaled_offset<SPHERE>(F, __uint_as_float(near)), kWeakBits, a.tab, mc);
+    }
     // ---- assemble, in fixed point (mmapanel.cuh)
     for (int c = tid; c < K; c += NTH) {
       const int o = tri_off(K, c);
@@ -195,7 +327,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       A[o + K - c] = YV[c];
     }
     if (tid == 0) AF[0] = 0;
-    for (int q0 = tid; q0 < NP; q0 += 2 * NTH) {
+    for (int q0 = exact ? NP : tid; q0 < NP; q0 += 2 * NTH) {
       const int q1 = q0 + NTH;
       const bool has1 = q1 < NP;
       const int v0 = tri_root(q0), v1 = tri_root(has1 ? q1 : q0);
@@ -213,11 +345,14 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       if (has1) AF[tri_off(K, c1) + r1 - c1] = ok1 ? fixed60(val1) : 0LL;
     }
     __syncthreads();
-    const bool ok = cta_eliminate<GRAD>(K, AF, reinterpret_cast<float2*>(TV), piv, zs, f, corner, tid, NTH);
+    const bool ok = exact ? cta_fp64_block<GRAD, SPHERE>(K, mi, A, CX, CY, CZ, TV, align_up(K + 1, 2), tc.gamma1, F.k2, F.k2d, a.tab)
+                          : cta_eliminate<GRAD>(K, AF, reinterpret_cast<float2*>(TV), piv, zs, f, corner, tid, NTH);
     // ---- the term, on warp 0 (FP64)
     const double nan = __longlong_as_double(0x7FF8000000000000LL);
     if (wid == 0) {
-      const double st = *corner > kSmallestPivot ? mul_pow2((double)*corner, 2 * f - 60) : 0.0, rr = A[2];
+      double st = A[1];
+      st = exact ? (zero_pivot(st) ? 0.0 : st) : *corner > kSmallestPivot ? mul_pow2((double)*corner, 2 * f - 60) : 0.0;
+      const double rr = A[2];
       const bool pd = ok && positive_finite(st);  // a non-finite rr with pd: non-finite data
       const bool good = pd && finite_bits(rr) && !bad_idx;
       const double s = tc.sigma2 * st;
@@ -248,7 +383,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
     // the pair pass on all threads
     const double cb = coef[0], rsa = coef[1], sS = coef[2];
     const bool good = finite_bits(sS);
-    panels_to_pairs(K, AF, reinterpret_cast<const float2*>(TV), tid, NTH);
+    if (!exact) panels_to_pairs(K, AF, reinterpret_cast<const float2*>(TV), tid, NTH);
     __syncthreads();
     const float2* __restrict__ L = reinterpret_cast<const float2*>(A);  // the unit factor
     double pT = 0.0;

@@ -352,6 +352,25 @@ __device__ __forceinline__ void pair_u(const FieldView& F, const float2* __restr
   }
 }
 
+// The squared distance (plane: u itself) of row p from the block's own location, which is at 0, in FP32, and u
+// from it.
+template <bool SPHERE>
+__device__ __forceinline__ float sq_offset(const float2* __restrict__ CX, const float2* __restrict__ CY,
+                                           const float2* __restrict__ CZ, int p) {
+  const float z = SPHERE ? CZ[p].x : 0.0f;
+  return fmaf(CX[p].x, CX[p].x, fmaf(CY[p].x, CY[p].x, z * z));
+}
+template <bool SPHERE>
+__device__ __forceinline__ float scaled_offset(const FieldView& F, float d2) {
+  if constexpr (SPHERE) {
+    float uh, ul;
+    sphere_u_df(fminf(d2, 4.0f), 0.0f, F, uh, ul);
+    return uh;
+  } else {
+    return d2;
+  }
+}
+
 // (pbh, pbl) += h (w_r g_c + w_c g_r) in double-float arithmetic.
 __device__ __forceinline__ void beta_pair_add(float2 wr, float2 wc, float2 gr, float2 gc, float hh, float hl,
                                               float& pbh, float& pbl) {
@@ -410,142 +429,20 @@ __device__ __forceinline__ void coord_offsets(const FieldView& F, const ThetaCon
   }
 }
 
-// Returns whether the location's term is valid (positive definite block, finite data,
-// indices in range).
-template <bool GRAD, int G, bool SPHERE, bool FIXED>
-__device__ __forceinline__ bool process_location(int64_t i, bool active, const FieldView& F, const SchedSize& S,
-                                                 const uint16_t* __restrict__ sched,
-                                                 const uint32_t* __restrict__ pairs, const WarpArea& W,
-                                                 const double* __restrict__ tab, const MaternConst& mc,
-                                                 const ThetaConst& tc, Accum& acc, bool terms_mode,
-                                                 double* terms, unsigned long long* errloc, int sub) {
-  constexpr int KCAP = max_k_for_lanes(G);
-  constexpr int NSG = (KCAP - 1 + G - 1) / G;  // neighbour slots per lane (m <= KCAP - 1)
-  const int m = F.m;
-  const int K = m + 1;
-  double* __restrict__ A = W.A;
-  float2* __restrict__ CX = W.CX;
-  float2* __restrict__ CY = W.CY;
-  float2* __restrict__ CZ = W.CZ;
-  double* __restrict__ TV = W.TV;
-  const int mi = (i < m && !F.pmean) ? (int)i : m;
-  const int32_t* __restrict__ row = F.nbr + i * m;
-  const bool check = kChecked || F.check_idx;
-  bool bad_idx = false;
-  int js = F.self[i];
-  if (check && (unsigned long long)(int64_t)js >= (unsigned long long)F.nidx) {
-    bad_idx = true;
-    js = 0;
-  }
-  const double2 ps = F.xy[js];
-  // ---- gather: centred, 1/beta-scaled coordinates (as float pairs), and the data: with
-  // two vectors per block straight into the border row K of A (slot tri_off(K, c) + K - c;
-  // the location's own y lands in A[2]), with separate column buffers into TV1, copied to
-  // the border by the assembly (that order measured 1% faster there)
-  const bool regather = regather_capable(GRAD, G) && W.regather;  // warp-uniform
-  const bool sep_buffers = GRAD && !regather;
-  static_assert(!FIXED || G == 32, "fixed point is for full-warp blocks");
-  constexpr bool kPanels = FIXED;
-  const int f = kPanels ? panel_shift(tc.gamma1) : 0;
-  long long corner = 0;
-#pragma unroll
-  for (int s = 0; s < NSG; ++s) {
-    const int p = sub + G * s;
-    if (p < m) {
-      double xv = 0.0, yv = 0.0, zv = 0.0, fv = 0.0;
-      if (p < mi) {
-        int j = row[p];
-        if (check && (unsigned long long)(int64_t)j >= (unsigned long long)F.nidx) {
-          bad_idx = true;
-          j = 0;
-        }
-        coord_offsets<SPHERE>(F, tc, ps, js, j, xv, yv, zv);
-        fv = F.yf[j];
-      }
-      if (sep_buffers) {
-        W.TV1[p] = fv;
-      } else {
-        A[tri_off(K, p) + K - p] = fv;
-      }
-      CX[p] = d2f_pair(xv);
-      CY[p] = d2f_pair(yv);
-      if constexpr (SPHERE) CZ[p] = d2f_pair(zv);
-    }
-  }
-  if (sub == 0) {
-    CX[m] = make_float2(0.0f, 0.0f);
-    CY[m] = make_float2(0.0f, 0.0f);
-    if constexpr (SPHERE) CZ[m] = make_float2(0.0f, 0.0f);
-    if (sep_buffers) {
-      W.TV1[m] = F.yf[js];
-    } else {
-      A[tri_off(K, m) + K - m] = F.yf[js];
-    }
-  }
-  if (check) {  // a bad index anywhere in the group fails the group's block
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane & ~(unsigned)(G - 1));
-    bad_idx = (__ballot_sync(0xffffffffu, bad_idx) & gmask) != 0u;
-  }
-  __syncwarp();
-  // ---- assemble: diagonal (and, with separate column buffers, the data border), then
-  // the correlation pairs
-  for (int c = sub; c < K; c += G) {
-    const int o = tri_off(K, c);
-    const double dg = (c >= mi && c < m) ? 1.0 : tc.gamma1;
-    if constexpr (kPanels) {  // in fixed point (mmapanel.cuh); a pad's diagonal is any positive number
-      A[o] = __longlong_as_double(fixed_from_double(tc.gamma1, 60 - 2 * f));
-    } else {
-      A[o] = dg;
-    }
-    if (sep_buffers) A[o + K - c] = W.TV1[c];
-  }
-  if (sub == 0) A[0] = 0.0;
-  // Two pairs per lane per iteration so one pair's loads overlap the other's FMAs.
-  for (int q0 = sub; q0 < S.NP; q0 += 2 * G) {
-    const int q1 = q0 + G;
-    const bool has1 = q1 < S.NP;
-    const uint32_t w0 = pairs[q0];
-    const uint32_t w1 = has1 ? pairs[q1] : w0;
-    const int r0 = w0 & 0xFF, c0 = (w0 >> 8) & 0xFF;
-    const int r1 = w1 & 0xFF, c1 = (w1 >> 8) & 0xFF;
-    const bool v0 = c0 < mi && (r0 < mi || r0 == m);
-    const bool v1 = has1 && c1 < mi && (r1 < mi || r1 == m);
-    float u0h, u0l, u1h, u1l;
-    pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
-    pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
-    FixRho val0, val1;
-    if constexpr (GRAD && !FIXED) {
-      val0 = rho_fixed62(u0h, u0l, tab, mc);
-      val1 = rho_fixed62(u1h, u1l, tab, mc);
-    } else {
-      rho_fixed62(u0h, u0l, u1h, u1l, tab, mc, val0, val1);
-    }
-    if constexpr (kPanels) {  // units of 2^-60
-      A[w0 >> 16] = __longlong_as_double(v0 ? fixed60(val0) : 0LL);
-      if (has1) A[w1 >> 16] = __longlong_as_double(v1 ? fixed60(val1) : 0LL);
-    } else {
-      if (!v0) val0.v = 0;
-      if (!v1) val1.v = 0;
-      A[w0 >> 16] = fixed_to_double(val0);
-      if (has1) A[w1 >> 16] = fixed_to_double(val1);
-    }
-  }
-  __syncwarp();
-  // ---- L D L^T over the neighbour columns, two columns per step: column j, then column
-  // j+1 updated by column j and scaled, then one pass over the remaining prefix applying
-  // both (fma(-L1, T1, fma(-L0, T0, a)): the same roundings, in the same order, as two
-  // single-column steps, with half the column transitions and shared-memory passes).
-  bool ok = true;
-  double* __restrict__ TV1 = W.TV1;  // column j+1's unscaled entries
+// L D L^T over the neighbour columns by the G lanes of a group, two columns per step: column j, then column
+// j+1 updated by column j and scaled, then one pass over the remaining prefix applying
+// both (fma(-L1, T1, fma(-L0, T0, a)): the same roundings, in the same order, as two
+// single-column steps, with half the column transitions and shared-memory passes).  TV and TV1 take columns'
+// unscaled entries.  Returns whether every pivot is in range.
+template <bool GRAD, int G>
+__device__ __forceinline__ bool ldl_eliminate(int K, double* __restrict__ A, double* __restrict__ TV,
+                                              double* __restrict__ TV1, const uint16_t* __restrict__ sched, int sub) {
   // Column scaling by the pivot reciprocal: the integer round-to-nearest-even product
   // (mul_by_positive, bit-identical to the DMUL) in the 4-lane forward kernel, where it
   // keeps an FP64 instruction off the column step's serial path (m = 10, n = 1M: 1.266 ->
   // 1.245 ms); the DMUL elsewhere (8- and 16-lane groups 2.5% faster with it at m = 30).
   constexpr bool kIntScale = G == 4 && !GRAD;
-  if constexpr (kPanels) {
-    ok = panels_eliminate<GRAD>(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), f, corner, sub);
-  } else {
+  bool ok = true;
   int j = 0;
   for (; j + 2 < K; j += 2) {
     const int oj = tri_off(K, j), o1 = tri_off(K, j + 1);
@@ -715,9 +612,219 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     }
     __syncwarp();
   }
+  return ok;
+}
+
+// A full-warp block of the fixed-point kernels in FP64 (mmapanel.cuh says which): assembly and L D L^T, with the
+// roundings of the FP64 kernels, then (GRAD) the factor as float pairs, as panels_to_pairs leaves it.  Returns
+// whether the neighbours' block is positive definite; s_i / sigma2 and y_i - mu_i are in A[1] and A[2].  The data
+// are in the border row, or (sep) in TV1.  (A function of its own, for the registers of its caller.)
+template <bool GRAD, bool SPHERE>
+static __device__ __noinline__ bool fp64_block(int K, int mi, const uint16_t* __restrict__ sched,
+                                               const uint32_t* __restrict__ pairs, double* A, const float2* CX,
+                                               const float2* CY, const float2* CZ, double* TV, double* TV1, bool sep,
+                                               double gamma1, float2 k2, double k2d, const double* __restrict__ tab,
+                                               int lane) {
+  const int m = K - 1, NP = K * (K - 1) / 2;
+  const MaternConst mc = matern_const_at(fix_const(tab));
+  FieldView F;
+  F.k2 = k2;
+  F.k2d = k2d;
+  for (int c = lane; c < K; c += 32) {
+    const int o = tri_off(K, c);
+    A[o] = (c >= mi && c < m) ? 1.0 : gamma1;
+    if (sep) A[o + K - c] = TV1[c];
+  }
+  if (lane == 0) A[0] = 0.0;
+#pragma unroll 1
+  for (int q0 = lane; q0 < NP; q0 += 64) {
+    const uint32_t w0 = pairs[q0], w1 = pairs[min(q0 + 32, NP - 1)];
+    const int r0 = w0 & 0xFF, c0 = (w0 >> 8) & 0xFF, r1 = w1 & 0xFF, c1 = (w1 >> 8) & 0xFF;
+    float u0h, u0l, u1h, u1l;
+    pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
+    pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
+    FixRho v0, v1;
+    rho_fixed62(u0h, u0l, u1h, u1l, tab, mc, v0, v1);
+    A[w0 >> 16] = c0 < mi && (r0 < mi || r0 == m) ? fixed_to_double(v0) : 0.0;
+    if (q0 + 32 < NP) A[w1 >> 16] = c1 < mi && (r1 < mi || r1 == m) ? fixed_to_double(v1) : 0.0;
+  }
+  __syncwarp();
+  bool ok = ldl_eliminate<GRAD, 32>(K, A, TV, TV1, sched, lane);
+  for (int c = lane; c < K - 1; c += 32) ok = ok && !zero_pivot(A[tri_off(K, c)]);
+  ok = __all_sync(0xffffffffu, ok);
+  if (GRAD) {
+    for (int e = 3 + lane; e < (K + 1) * (K + 2) / 2; e += 32) {
+      const uint32_t rc = sched[e];
+      if ((rc & 0xFF) > (rc >> 8)) reinterpret_cast<float2*>(A)[e] = d2f_trunc(A[e]);
+    }
+    __syncwarp();
+  }
+  return ok;
+}
+
+// Returns whether the location's term is valid (positive definite block, finite data,
+// indices in range).
+template <bool GRAD, int G, bool SPHERE, bool FIXED>
+__device__ __forceinline__ bool process_location(int64_t i, bool active, const FieldView& F, const SchedSize& S,
+                                                 const uint16_t* __restrict__ sched,
+                                                 const uint32_t* __restrict__ pairs, const WarpArea& W,
+                                                 const double* __restrict__ tab, const MaternConst& mc,
+                                                 const ThetaConst& tc, Accum& acc, bool terms_mode,
+                                                 double* terms, unsigned long long* errloc, int sub) {
+  constexpr int KCAP = max_k_for_lanes(G);
+  constexpr int NSG = (KCAP - 1 + G - 1) / G;  // neighbour slots per lane (m <= KCAP - 1)
+  const int m = F.m;
+  const int K = m + 1;
+  double* __restrict__ A = W.A;
+  float2* __restrict__ CX = W.CX;
+  float2* __restrict__ CY = W.CY;
+  float2* __restrict__ CZ = W.CZ;
+  double* __restrict__ TV = W.TV;
+  const int mi = (i < m && !F.pmean) ? (int)i : m;
+  const int32_t* __restrict__ row = F.nbr + i * m;
+  const bool check = kChecked || F.check_idx;
+  bool bad_idx = false;
+  int js = F.self[i];
+  if (check && (unsigned long long)(int64_t)js >= (unsigned long long)F.nidx) {
+    bad_idx = true;
+    js = 0;
+  }
+  const double2 ps = F.xy[js];
+  // ---- gather: centred, 1/beta-scaled coordinates (as float pairs), and the data: with
+  // two vectors per block straight into the border row K of A (slot tri_off(K, c) + K - c;
+  // the location's own y lands in A[2]), with separate column buffers into TV1, copied to
+  // the border by the assembly (that order measured 1% faster there)
+  const bool regather = regather_capable(GRAD, G) && W.regather;  // warp-uniform
+  const bool sep_buffers = GRAD && !regather;
+  static_assert(!FIXED || G == 32, "fixed point is for full-warp blocks");
+  constexpr bool kPanels = FIXED;
+  const int f = kPanels ? panel_shift(tc.gamma1) : 0;
+  long long corner = 0;
+  bool exact = f > kMostShift;  // the block goes to fp64_block
+  int large[kPanels ? NSG + 1 : 1];  // exponent fields of this lane's data
+#pragma unroll
+  for (int s = 0; s < NSG; ++s) {
+    const int p = sub + G * s;
+    if (kPanels) large[s] = 0;
+    if (p < m) {
+      double xv = 0.0, yv = 0.0, zv = 0.0, fv = 0.0;
+      if (p < mi) {
+        int j = row[p];
+        if (check && (unsigned long long)(int64_t)j >= (unsigned long long)F.nidx) {
+          bad_idx = true;
+          j = 0;
+        }
+        coord_offsets<SPHERE>(F, tc, ps, js, j, xv, yv, zv);
+        fv = F.yf[j];
+        if (kPanels) large[s] = (int)exponent_field(fv);
+      }
+      if (sep_buffers) {
+        W.TV1[p] = fv;
+      } else {
+        A[tri_off(K, p) + K - p] = fv;
+      }
+      CX[p] = d2f_pair(xv);
+      CY[p] = d2f_pair(yv);
+      if constexpr (SPHERE) CZ[p] = d2f_pair(zv);
+    }
+  }
+  if (sub == 0) {
+    CX[m] = make_float2(0.0f, 0.0f);
+    CY[m] = make_float2(0.0f, 0.0f);
+    if constexpr (SPHERE) CZ[m] = make_float2(0.0f, 0.0f);
+    if (sep_buffers) {
+      W.TV1[m] = F.yf[js];
+    } else {
+      A[tri_off(K, m) + K - m] = F.yf[js];
+    }
+  }
+  if constexpr (kPanels) {
+    large[NSG] = sub == 0 && !F.pmean ? (int)exponent_field(F.yf[js]) : 0;
+    int top = large[0], count = 0;  // twice the large ones, less all but the zeros
+#pragma unroll
+    for (int s = 1; s <= NSG; ++s) top = max(top, large[s]);
+    top = __reduce_max_sync(0xffffffffu, top);
+#pragma unroll
+    for (int s = 0; s <= NSG; ++s)
+      count += 2 * __popc(__ballot_sync(0xffffffffu, large[s] > 0 && large_datum(large[s], top))) -
+               __popc(__ballot_sync(0xffffffffu, large[s] > 0));
+    exact = exact || count < 0;
+    if (GRAD || F.pmean) {
+      unsigned near = __float_as_uint(INFINITY);  // u of the nearest neighbour
+#pragma unroll
+      for (int s = 0; s < NSG; ++s) {
+        const int p = sub + 32 * s;
+        if (p < mi) near = min(near, __float_as_uint(sq_offset<SPHERE>(CX, CY, CZ, p)));
+      }
+      near = __reduce_min_sync(0xffffffffu, near);
+      exact = exact || rho_below(scaled_offset<SPHERE>(F, __uint_as_float(near)), kWeakBits, tab, mc);
+    }
+  }
+  if (check) {  // a bad index anywhere in the group fails the group's block
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane & ~(unsigned)(G - 1));
+    bad_idx = (__ballot_sync(0xffffffffu, bad_idx) & gmask) != 0u;
+  }
+  __syncwarp();
+  // ---- assemble: diagonal (and, with separate column buffers, the data border), then
+  // the correlation pairs
+  if (!exact) {
+  for (int c = sub; c < K; c += G) {
+    const int o = tri_off(K, c);
+    const double dg = (c >= mi && c < m) ? 1.0 : tc.gamma1;
+    if constexpr (kPanels) {  // in fixed point (mmapanel.cuh); a pad's diagonal is any positive number
+      A[o] = __longlong_as_double(fixed_from_double(tc.gamma1, 60 - 2 * f));
+    } else {
+      A[o] = dg;
+    }
+    if (sep_buffers) A[o + K - c] = W.TV1[c];
+  }
+  if (sub == 0) A[0] = 0.0;
+  // Two pairs per lane per iteration so one pair's loads overlap the other's FMAs.
+  for (int q0 = sub; q0 < S.NP; q0 += 2 * G) {
+    const int q1 = q0 + G;
+    const bool has1 = q1 < S.NP;
+    const uint32_t w0 = pairs[q0];
+    const uint32_t w1 = has1 ? pairs[q1] : w0;
+    const int r0 = w0 & 0xFF, c0 = (w0 >> 8) & 0xFF;
+    const int r1 = w1 & 0xFF, c1 = (w1 >> 8) & 0xFF;
+    const bool v0 = c0 < mi && (r0 < mi || r0 == m);
+    const bool v1 = has1 && c1 < mi && (r1 < mi || r1 == m);
+    float u0h, u0l, u1h, u1l;
+    pair_u<SPHERE>(F, CX, CY, CZ, r0, c0, u0h, u0l);
+    pair_u<SPHERE>(F, CX, CY, CZ, r1, c1, u1h, u1l);
+    FixRho val0, val1;
+    if constexpr (GRAD && !FIXED) {
+      val0 = rho_fixed62(u0h, u0l, tab, mc);
+      val1 = rho_fixed62(u1h, u1l, tab, mc);
+    } else {
+      rho_fixed62(u0h, u0l, u1h, u1l, tab, mc, val0, val1);
+    }
+    if constexpr (kPanels) {  // units of 2^-60
+      A[w0 >> 16] = __longlong_as_double(v0 ? fixed60(val0) : 0LL);
+      if (has1) A[w1 >> 16] = __longlong_as_double(v1 ? fixed60(val1) : 0LL);
+    } else {
+      if (!v0) val0.v = 0;
+      if (!v1) val1.v = 0;
+      A[w0 >> 16] = fixed_to_double(val0);
+      if (has1) A[w1 >> 16] = fixed_to_double(val1);
+    }
+  }
+  __syncwarp();
+  }
+  // ---- elimination (TV1: column j+1's unscaled entries)
+  bool ok;
+  if constexpr (kPanels) {
+    if (exact)
+      ok = fp64_block<GRAD, SPHERE>(K, mi, sched, pairs, A, CX, CY, CZ, TV, W.TV1, sep_buffers, tc.gamma1, F.k2, F.k2d, tab, sub);
+    else
+      ok = panels_eliminate<GRAD>(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), f, corner, sub);
+  } else {
+    ok = ldl_eliminate<GRAD, G>(K, A, TV, W.TV1, sched, sub);
   }
   // s_i / sigma2
-  const double st = !kPanels ? A[1] : corner > kSmallestPivot ? mul_pow2((double)corner, 2 * f - 60) : 0.0;
+  double st = A[1];
+  if (kPanels) st = exact ? (zero_pivot(st) ? 0.0 : st) : corner > kSmallestPivot ? mul_pow2((double)corner, 2 * f - 60) : 0.0;
   const double rr = A[2];  // y_i - mu_i
   // The pivots and s_i depend on the covariance only, the residual on the data: a
   // non-finite residual (with a positive definite block) means a non-finite y in B_i.
@@ -778,7 +885,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
   }
   constexpr int NS = (KCAP - 1 + G - 1) / G;  // slots of the K-1 <= KCAP-1 neighbour entries
   if constexpr (kPanels) {
-    panels_to_pairs(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), sub, 32);
+    if (!exact) panels_to_pairs(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), sub, 32);
     __syncwarp();
   }
   // The two unit backward solves run in double-float arithmetic on the FP32 pipe: each

@@ -130,6 +130,16 @@ __device__ __forceinline__ void rho_fixed62(float u0h, float u0l, float u1h, flo
   }
 }
 
+// Whether rho(u) is below 2^-bits, bits >= 7 (by the interval's E, so to within a factor of two).
+__device__ __forceinline__ bool rho_below(float u, int bits, const double* __restrict__ tab, const MaternConst& mc) {
+  if (fix_outside(u)) {
+    const FixRho r = rho_outside62_call(u, 0.0f, mc.kind, mc.nu, mc.a1, mc.G, mc.b0, mc.b1);
+    return r.v >> min((r.sh >> 20) - bits, 63) == 0;
+  }
+  const float4* __restrict__ w = reinterpret_cast<const float4*>(tab) + fix_arg(u, 0.0f).idx * kFixWords;
+  return (__float_as_int(__ldg(reinterpret_cast<const float*>(w + 2) + 3)) >> 20) - 62 >= bits - 6;
+}
+
 // In FP64: one conversion, and the power of two on the exponent field.  (A conversion holds the FP64 pipe
 // for 64 cycles; integer operations in its place, some 25, gave 2% at m = 30 and took 2% at m = 10.)
 __device__ __forceinline__ double fixed_to_double(FixRho r) {

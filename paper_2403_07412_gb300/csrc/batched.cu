@@ -32,13 +32,16 @@ bool theta_ok(const double* th);
 int lanes_for(int K, bool grad, int64_t count);
 
 // Locations an item gives each group of a warp: up to kMostSteps, fewer where the class has
-// not kItemsPerWarp such items for each resident warp.  A full-warp location of m = 60 takes
+// not kItemsPerWarp such items for each resident warp, more where it has kManyItems times as many, so
+// that a class's records (32 bytes an item) stay at some kManyItems kItemsPerWarp for each resident warp,
+// 4 MB or so, however large the batch.  A full-warp location of m = 60 takes
 // a warp some 75 us: eight make an item long enough to hide its hand-out (an atomic, the
 // field search, the constants: a few us).  Items of 256 locations took 19 ms each there, a
 // batch of two fields of n = 20,000, two thetas, 44 ms where its work takes 7; with eight for
-// every size, two fields of n = 700 took 1.40 ms.
+// every size, two fields of n = 700 took 1.40 ms, and 64 fields under 32 thetas kept 413 MB of records.
 constexpr int kMostSteps = 8;
 constexpr int kItemsPerWarp = 4;
+constexpr int kManyItems = 16;
 constexpr int kMaxNu = 8;        // prepared smoothness values
 constexpr int kMaxDistinctK = 4; // distinct block sizes per batch, and so most classes
 
@@ -371,7 +374,8 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
     const int64_t share = steps / ((int64_t)kItemsPerWarp * c.blocks * c.W);
     for (int k = a.first_field; k <= a.last_field; ++k) {
       FieldDesc& d = fd[k];
-      d.tile = (32 / L) * (int)std::max<int64_t>(1, std::min<int64_t>(kMostSteps, share));
+      const int64_t step = std::max<int64_t>({1, std::min<int64_t>(kMostSteps, share), share / kManyItems});
+      d.tile = (32 / L) * (int)std::min<int64_t>(step, (d.n + 32 / L - 1) / (32 / L));
       d.tiles = (int)((d.n + d.tile - 1) / d.tile);
       d.item_base = items;
       items += (int64_t)d.tiles * ntheta;

@@ -69,21 +69,24 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // columns, and warp 0 runs ahead with it: it takes the sixteen rows below a panel through the
 // panel's columns (panel_row, a row per lane), updates them for the next panel and factors
 // that panel's rows, while the other warps take the rows further down through the first
-// panel's columns and, once warp 0's sixteen rows are in (barrier 1), update them.
+// panel's columns and, once warp 0's sixteen rows are in (barrier 1), update them.  The data are the other
+// warps' work too, a panel behind: warp 1 solves for the first panel's z (barrier 2), each row's datum goes
+// with the row, and warp 1 takes the sixteen rows' from their digits.  (On warp 0, in the panels' columns:
+// n = 20k, m = 120 with the gradient 11.2 ms, m = 130 without 12.3; SOLVE_MS so.)
 template <bool GRAD>
 __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, float2* __restrict__ RJ, int4* __restrict__ piv,
                                               double* __restrict__ zs, int f, long long* corner, int tid, int NTH) {
   const int lane = tid & 31, wid = tid >> 5;
-  int over = 0;
-  // piv and zs hold those of this panel and the next
+  int over = 0, c1 = 0;
+  // piv holds those of this panel and the next
 #pragma unroll 1
   for (int c0 = -kPanelCols; c0 + kPanelCols < K; c0 += kPanelCols) {
-    const int c1 = c0 + kPanelCols, pe = min(c1 + kPanelCols, K);
+    c1 = c0 + kPanelCols;
+    const int pe = min(c1 + kPanelCols, K);
     const int4* __restrict__ pv = piv + (c0 & kPanelCols);
-    const double* __restrict__ pz = zs + (c0 & kPanelCols);
     if (wid == 0) {
       if (c0 >= 0) {
-        if (lane < 16 && c1 + lane < K) panel_row(K, A, pv, pz, c0, f, c1 + lane, over);
+        if (lane < 16 && c1 + lane < K) panel_row<false>(K, A, pv, zs, c0, f, c1 + lane, over);
         __threadfence_block();
         asm volatile("bar.arrive 1, %0;" ::"r"(NTH) : "memory");
         __syncwarp();
@@ -91,17 +94,21 @@ __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, 
         __syncwarp();
       }
       long long cr = 0;
-      if (!panel_columns<GRAD, true>(K, A, RJ, piv + (c1 & kPanelCols), zs + (c1 & kPanelCols), c1, f, cr, lane)) over = 1;
+      if (!panel_columns<GRAD, true>(K, A, RJ, piv + (c1 & kPanelCols), c1, f, cr, lane)) over = 1;
       if (pe == K && lane == 0) *corner = cr;
     } else if (c0 >= 0) {
+      if (wid == 1) panel_solve<GRAD>(K, A, RJ, pv, zs, c0, f, lane);
+      asm volatile("bar.sync 2, %0;" ::"r"(NTH - 32) : "memory");
 #pragma unroll 1
-      for (int r = c1 + 16 + tid - 32; r < K; r += NTH - 32) panel_row(K, A, pv, pz, c0, f, r, over);
+      for (int r = c1 + 16 + tid - 32; r < K; r += NTH - 32) panel_row<true>(K, A, pv, zs, c0, f, r, over);
       asm volatile("bar.sync 1, %0;" ::"r"(NTH) : "memory");
+      if (wid == 1 && lane < 16 && c1 + lane < K) panel_row_data(K, A, zs, c0, c1 + lane);
 #pragma unroll 1
       for (int rt = c1 + 16 * wid; rt < K; rt += (NTH - 32) / 2) update_tile<true>(K, A, rt, c1, pe, f, lane);
     }
     __syncthreads();
   }
+  if (wid == 1) panel_solve<GRAD>(K, A, RJ, piv + (c1 & kPanelCols), zs, c1, f, lane);
   return __syncthreads_or(over) == 0;
 }
 
@@ -468,7 +475,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
 // Shared memory of the CTA kernel for block size K.
 int big_smem_bytes(int K, bool sphere) {
   const int NTd = (K + 1) * (K + 2) / 2;
-  return 8 * (align_up(NTd, 2) + (sphere ? 7 : 6) * align_up(K + 1, 2) + 32 + 6 + 6 * kPanelCols);
+  return 8 * (align_up(NTd, 2) + (sphere ? 7 : 6) * align_up(K + 1, 2) + 32 + 6 + 5 * kPanelCols);
 }
 
 // CTA size: the W warps with the largest c W / (W + 2), c the CTAs of that size resident on an SM

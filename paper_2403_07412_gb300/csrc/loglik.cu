@@ -352,9 +352,9 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
       int per_sm = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, bytes) != cudaSuccess) return -2;
       int warps = std::min(per_sm * W, 16);
-      // Fixed point: an SM's four sub-partitions with the same number of warps each (n = 100k, 12 and 13
-      // warps: m = 54 4.56 and 4.96 ms, m = 60 5.68 and 6.09).
-      if (fixed_point_block(K, grad, G) && warps % 4) warps = std::max(1, (warps & ~3) - 1);
+      // Fixed point: not one warp more than the four sub-partitions share evenly (n = 100k, 12 and 13
+      // warps: m = 54 4.56 and 4.96 ms, m = 60 5.68 and 6.09; but 8 and 10 at m = 63 7.13 and 6.79).
+      if (fixed_point_block(K, grad, G) && warps > 1 && warps % 4 == 1) warps -= 2;
       if (per_sm > 0 && warps > best_warps) {
         best_warps = warps;
         out->G = G;

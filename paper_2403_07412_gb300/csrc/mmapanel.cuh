@@ -288,12 +288,11 @@ __device__ __forceinline__ void update_tile(int K, long long* __restrict__ A, in
 // columns' stay below 2^31).  The data of the lane's rows (slots (K, r) of the triangle) take each
 // column's z_c times the row's entry off, and column c's own slot is left z_c / sqrt(d_c), the unit factor's
 // entry.  Returns whether the block can still be positive definite.
-// With CTA only the panel's own rows (of the last panel: all), and the pivots' reciprocals and the z_c 2^-62
-// are left in piv and zs for panel_row.
+// With CTA only the panel's own rows (of the last panel: all) and not the data, and the pivots' reciprocals are
+// left in piv for panel_row and panel_solve.
 template <bool GRAD, bool CTA>
 __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, float2* __restrict__ RJ,
-                                              int4* __restrict__ piv, double* __restrict__ zs, int c0, int f,
-                                              long long& corner, int lane) {
+                                              int4* __restrict__ piv, int c0, int f, long long& corner, int lane) {
   const int R = K - 1;
   const int rmax = CTA && c0 + kPanelCols < K ? c0 + kPanelCols - 1 : R;
   const int last = K - 1 - c0;    // panel position of column m
@@ -307,7 +306,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
   const int y0s = tri_off(K, min(r0, R)) + K - min(r0, R), y1s = tri_off(K, min(r1, R)) + K - min(r1, R);
   // The data: column j's z_j goes round (through the triangle's unused slot 0) after its V, and is taken off
   // the rows in the next column, where the FP64 pipe's latency hides behind the integers.
-  double y0 = Y[y0s], y1 = two ? Y[y1s] : 0.0;
+  double y0 = CTA ? 0.0 : Y[y0s], y1 = two ? Y[y1s] : 0.0;
   double v0 = 0.0, v1 = 0.0, z = 0.0, scale = 0.0;
 #pragma unroll 1
   for (int j = 0; j < jn; ++j) {
@@ -332,7 +331,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       ok_ -= step + 1;
       --step;
     }
-    y0 = fma(-v0, z, y0);
+    if (!CTA) y0 = fma(-v0, z, y0);
     if (two) y1 = fma(-v1, z, y1);
     s0 += (long long)m0 * 4;
     if (f && lane == j) s0 >>= min(2 * f, 63);
@@ -361,7 +360,7 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
       over |= top_magnitude(a0) >> lim;
       const long long v = scaled_entry(a0, q, rh, rl, f);
       A[oj + r0] = v;
-      v0 = (double)v;
+      if (!CTA) v0 = (double)v;
     }
     if (two) {
       s1 += (long long)m1 * 4;
@@ -373,11 +372,11 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
         v1 = (double)v;
       }
     }
-    double* const at = CTA ? zs + j : Y;
-    if (lane == j) *at = zj;
+    if (!CTA && lane == j) Y[0] = zj;
     __syncwarp();
-    z = *at;
+    if (!CTA) z = Y[0];
   }
+  if (CTA) return ok && !__any_sync(0xffffffffu, over != 0);
   if (c0 + kPanelCols <= R) {  // (the last panel's last column takes nothing off)
     y0 = fma(-v0, z, y0);
     if (two) y1 = fma(-v1, z, y1);
@@ -393,12 +392,13 @@ __device__ __forceinline__ bool panel_columns(int K, long long* __restrict__ A, 
 }
 
 // Row r below the panel [c0, c0 + 8), by one thread: its eight entries of the factor, from the
-// panel's own rows and pivots, and then their digits, in place; and its datum.
+// panel's own rows and pivots, and then their digits, in place; and (DATA) its datum.
+template <bool DATA>
 __device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, const int4* __restrict__ piv,
                                           const double* __restrict__ zs, int c0, int f, int r, int& over) {
   const int2* __restrict__ V = reinterpret_cast<const int2*>(A);
   double* __restrict__ Y = reinterpret_cast<double*>(A) + tri_off(K, r) + K - r;
-  double y = *Y, v0 = 0.0, z = 0.0;
+  double y = DATA ? *Y : 0.0, v0 = 0.0, z = 0.0;  // a column's part is taken off in the next one
 #pragma unroll 1
   for (int j = 0; j < kPanelCols; ++j) {
     long long s0 = 0;
@@ -413,19 +413,21 @@ __device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, cons
       ok_ -= step + 1;
       --step;
     }
-    y = fma(-v0, z, y);
+    if (DATA) y = fma(-v0, z, y);
     const int4 pv = piv[j];
     const long long a = A[ok_ + r] - s0 - (long long)m0 * 4;
     over |= top_magnitude(a) >> max(29 - pv.x, 0);
     const long long v = scaled_entry(a, pv.x, pv.y, pv.z, f);
     A[ok_ + r] = v;
-    v0 = (double)v;
-    z = zs[j];
+    if (DATA) {
+      v0 = (double)v;
+      z = zs[j];
+    }
   }
-  *Y = fma(-v0, z, y);
+  if (DATA) *Y = fma(-v0, z, y);
 #pragma unroll 1
-  for (int k0 = c0; k0 < c0 + kPanelCols; k0 += 4) {
-    const WordSlots w(K, k0);
+  for (int k0 = 0; k0 < kPanelCols; k0 += 4) {
+    const WordSlots w(K, c0 + k0);
     long long v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = A[w.e[i] + r];
@@ -434,6 +436,56 @@ __device__ __forceinline__ void panel_row(int K, long long* __restrict__ A, cons
 #pragma unroll
     for (int i = 0; i < 4; ++i) reinterpret_cast<uint2*>(A)[w.e[i] + r] = make_uint2(pl[2 * i], pl[2 * i + 1]);
   }
+}
+
+// The data of panel [c0, c0 + 8)'s own rows, all earlier columns taken off, by one warp: z_c 2^-62 to zs, the unit
+// factor's entries z_c / sqrt(d_c) and (GRAD) 2^-62 / sqrt(d_c); row m's datum, in the last panel, becomes the
+// residual.
+template <bool GRAD>
+__device__ __forceinline__ void panel_solve(int K, long long* __restrict__ A, float2* __restrict__ RJ,
+                                            const int4* __restrict__ piv, double* __restrict__ zs, int c0, int f, int lane) {
+  const int R = K - 1, jn = min(kPanelCols, R - c0), r = min(c0 + lane, R);
+  double* __restrict__ Y = reinterpret_cast<double*>(A) + tri_off(K, r) + K - r;
+  const int4 pv = piv[min(lane, max(jn - 1, 0))];
+  const double rs = pivot_scale(((long long)pv.y << 31) + pv.z, pv.x - f - 61 - 62);
+  double y = *Y;
+#pragma unroll 1
+  for (int j = 0; j < jn; ++j) {
+    const double v = r > c0 + j ? (double)A[tri_off(K, c0 + j) + r - c0 - j] : 0.0;
+    const double z = __shfl_sync(0xffffffffu, y * rs, j);
+    if (lane == j) zs[j] = z;
+    if (r > c0 + j) y = fma(-v, z, y);
+  }
+  __syncwarp();
+  if (lane < jn) {
+    if (GRAD) {
+      *Y = y * (rs * 0x1p62) * (rs * 0x1p62);
+      RJ[r] = d2f_trunc(rs);
+    }
+  } else if (c0 + lane == R && lane < kPanelCols) {
+    *Y = y;
+  }
+  __syncwarp();
+}
+
+// Panel [c0, c0 + 8)'s columns taken off the datum of row r below it, from the digits.
+__device__ __forceinline__ void panel_row_data(int K, long long* __restrict__ A, const double* __restrict__ zs, int c0, int r) {
+  double* __restrict__ Y = reinterpret_cast<double*>(A) + tri_off(K, r) + K - r;
+  double y = *Y;
+#pragma unroll 1
+  for (int k0 = 0; k0 < kPanelCols; k0 += 4) {
+    const WordSlots ws(K, c0 + k0);
+    unsigned w[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint2 x = reinterpret_cast<const uint2*>(A)[ws.e[i] + r];
+      w[2 * i] = x.x;
+      w[2 * i + 1] = x.y;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) y = fma(-(double)planes_value(w, i), zs[k0 + i], y);
+  }
+  *Y = y;
 }
 
 // The panel's factor entries of the rows below it as digits, in place.
@@ -467,7 +519,7 @@ __device__ __forceinline__ bool panels_eliminate(int K, long long* __restrict__ 
       for (int rt = c0; rt < K; rt += 16) update_tile<false>(K, A, rt, c0, pe, f, lane);
       __syncwarp();
     }
-    const bool o = panel_columns<GRAD, false>(K, A, RJ, nullptr, nullptr, c0, f, corner, lane);
+    const bool o = panel_columns<GRAD, false>(K, A, RJ, nullptr, c0, f, corner, lane);
     ok = ok && o;
     if (pe < K) panel_to_digits(K, A, c0, lane);
   }

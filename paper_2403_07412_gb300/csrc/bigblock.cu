@@ -216,9 +216,9 @@ static __device__ __noinline__ bool cta_fp64_block(int K, int mi, double* A, con
   double* TVs[4] = {TV, TV - stride, TV + stride, TV + 2 * stride};
   bool ok = true;
   int j = 0;
-  for (; ok && j + 4 < K; j += 4) ok = cta_columns<4>(A, TVs, K, j, tid, NTH);
-  for (; ok && j + 2 < K; j += 2) ok = cta_columns<2>(A, TVs, K, j, tid, NTH);
-  if (ok && j + 1 < K) ok = cta_columns<1>(A, TVs, K, j, tid, NTH);
+  for (; ok && j + 4 <= mi; j += 4) ok = cta_columns<4>(A, TVs, K, j, tid, NTH);  // (pads' columns are the identity's)
+  for (; ok && j + 2 <= mi; j += 2) ok = cta_columns<2>(A, TVs, K, j, tid, NTH);
+  if (ok && j + 1 <= mi) ok = cta_columns<1>(A, TVs, K, j, tid, NTH);
   if (GRAD) {
     for (int e = 3 + tid; e < (K + 1) * (K + 2) / 2; e += NTH) {
       const int w = tri_root(e);

@@ -429,13 +429,14 @@ __device__ __forceinline__ void coord_offsets(const FieldView& F, const ThetaCon
   }
 }
 
-// L D L^T over the neighbour columns by the G lanes of a group, two columns per step: column j, then column
+// L D L^T over the first `cols` neighbour columns (the rest are pads' identity columns, or none) by the G lanes
+// of a group, two columns per step: column j, then column
 // j+1 updated by column j and scaled, then one pass over the remaining prefix applying
 // both (fma(-L1, T1, fma(-L0, T0, a)): the same roundings, in the same order, as two
 // single-column steps, with half the column transitions and shared-memory passes).  TV and TV1 take columns'
 // unscaled entries.  Returns whether every pivot is in range.
 template <bool GRAD, int G>
-__device__ __forceinline__ bool ldl_eliminate(int K, double* __restrict__ A, double* __restrict__ TV,
+__device__ __forceinline__ bool ldl_eliminate(int K, int cols, double* __restrict__ A, double* __restrict__ TV,
                                               double* __restrict__ TV1, const uint16_t* __restrict__ sched, int sub) {
   // Column scaling by the pivot reciprocal: the integer round-to-nearest-even product
   // (mul_by_positive, bit-identical to the DMUL) in the 4-lane forward kernel, where it
@@ -444,7 +445,7 @@ __device__ __forceinline__ bool ldl_eliminate(int K, double* __restrict__ A, dou
   constexpr bool kIntScale = G == 4 && !GRAD;
   bool ok = true;
   int j = 0;
-  for (; j + 2 < K; j += 2) {
+  for (; j + 2 <= cols; j += 2) {
     const int oj = tri_off(K, j), o1 = tri_off(K, j + 1);
     const double d0 = A[oj];
     ok = ok && pivot_in_range(d0);  // a failed block runs on (values unused) to stay in step
@@ -555,7 +556,7 @@ __device__ __forceinline__ bool ldl_eliminate(int K, double* __restrict__ A, dou
     }
     __syncwarp();
   }
-  if (j < K - 1) {  // an odd number of neighbour columns: the last one alone
+  if (j < cols) {  // an odd number of neighbour columns: the last one alone
     const int oj = tri_off(K, j);
     const double d = A[oj];
     ok = ok && pivot_in_range(d);  // a failed block runs on (values unused) to stay in step
@@ -649,7 +650,7 @@ static __device__ __noinline__ bool fp64_block(int K, int mi, const uint16_t* __
     if (q0 + 32 < NP) A[w1 >> 16] = c1 < mi && (r1 < mi || r1 == m) ? fixed_to_double(v1) : 0.0;
   }
   __syncwarp();
-  bool ok = ldl_eliminate<GRAD, 32>(K, A, TV, TV1, sched, lane);
+  bool ok = ldl_eliminate<GRAD, 32>(K, mi, A, TV, TV1, sched, lane);
   for (int c = lane; c < K - 1; c += 32) ok = ok && !zero_pivot(A[tri_off(K, c)]);
   ok = __all_sync(0xffffffffu, ok);
   if (GRAD) {
@@ -820,7 +821,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
     else
       ok = panels_eliminate<GRAD>(K, reinterpret_cast<long long*>(A), reinterpret_cast<float2*>(TV), f, corner, sub);
   } else {
-    ok = ldl_eliminate<GRAD, G>(K, A, TV, W.TV1, sched, sub);
+    ok = ldl_eliminate<GRAD, G>(K, K - 1, A, TV, W.TV1, sched, sub);
   }
   // s_i / sigma2
   double st = A[1];

@@ -224,6 +224,7 @@ namespace {
 struct LaunchCfg {
   int G = 32, W = 4, blocks = 0, smem = 0;
   bool regather = false;  // gradient, 8 lanes: coordinates gathered twice, two vectors per block
+  bool fixed = false;     // eliminated in fixed point
   int sms = 0;            // SMs of the device
 };
 
@@ -237,8 +238,7 @@ LikKernel kernel_ptr(int G, bool fixed) {
   return fixed ? vecchia_lik_kernel<GRAD, 32, SPHERE, true> : vecchia_lik_kernel<GRAD, 32, SPHERE, false>;
 }
 
-LikKernel lik_kernel(int K, bool grad, int G, bool sphere) {
-  const bool fixed = fixed_point_block(K, grad, G);
+LikKernel lik_kernel(bool grad, int G, bool sphere, bool fixed) {
   if (grad) return sphere ? kernel_ptr<true, true>(G, fixed) : kernel_ptr<true, false>(G, fixed);
   return sphere ? kernel_ptr<false, true>(G, fixed) : kernel_ptr<false, false>(G, fixed);
 }
@@ -322,14 +322,16 @@ int set_smem_limit(int dev, void* kern, int bytes) {
   return VECCHIA_OK;
 }
 
-int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere = false) {
+int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere = false, bool want_fixed = true) {
   if (K > max_k_for_lanes(G)) return VECCHIA_EINVAL;  // narrow groups hold small blocks only
+  const bool fixed = want_fixed && fixed_point_block(K, grad, G);
   int dev = 0, sms = 0, smem_optin = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_shape_mu);
-  void* kern = reinterpret_cast<void*>(lik_kernel(K, grad, G, sphere));
+  void* kern = reinterpret_cast<void*>(lik_kernel(grad, G, sphere, fixed));
   for (const ShapeEntry& e : g_shapes)
-    if (e.dev == dev && e.K == K && e.grad == (int)grad && e.G == G && e.W == forced_W && e.sphere == (int)sphere) {
+    if (e.dev == dev && e.K == K && e.grad == (int)grad && e.G == G && e.W == forced_W && e.sphere == (int)sphere &&
+        e.cfg.fixed == fixed) {
       const int rc = set_smem_limit(dev, kern, e.cfg.smem);
       if (rc) return rc;
       *cfg = e.cfg;
@@ -354,7 +356,7 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
       int warps = std::min(per_sm * W, 16);
       // Fixed point: not one warp more than the four sub-partitions share evenly (n = 100k, 12 and 13
       // warps: m = 54 4.56 and 4.96 ms, m = 60 5.68 and 6.09; but 8 and 10 at m = 63 7.13 and 6.79).
-      if (fixed_point_block(K, grad, G) && warps > 1 && warps % 4 == 1) warps -= 2;
+      if (fixed && warps > 1 && warps % 4 == 1) warps -= 2;
       if (per_sm > 0 && warps > best_warps) {
         best_warps = warps;
         out->G = G;
@@ -363,6 +365,7 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
         out->sms = sms;
         out->smem = bytes;
         out->regather = regather;
+        out->fixed = fixed;
       }
     }
     return best_warps;
@@ -435,11 +438,27 @@ int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t c
     }
   }
   while (K > max_k_for_lanes(G)) G *= 2;
-  return shape_for(K, grad, G, W, cfg, sphere);
+  int rc = shape_for(K, grad, G, W, cfg, sphere);
+  if (rc || chosen || count <= 0 || !cfg->fixed) return rc;
+  // A call of few turns of the resident warps takes as long as its last, nearly empty turn makes it.  Where
+  // fixed point takes twice the turns of FP64 of the same width (with the gradient: more registers, so fewer warps)
+  // or in 16 lanes (forward blocks of 39 to 42 rows, whose turn in 16 lanes takes some 1.8 times fixed point's in
+  // 32; at 38 rows it is two CTAs an SM and slower), FP64 is taken (us): n = 2,000, m = 50 with the gradient 209 for 265; m = 40, n = 3,000 128 for 142, 6,000
+  // 275 and 239 (3 turns and 2), 7,500 275 for 310.
+  if (!grad && (K < 39 || K > 42)) return VECCHIA_OK;
+  LaunchCfg fp64;
+  rc = shape_for(K, grad, grad ? G : 16, W, &fp64, sphere, false);
+  if (rc) return rc;
+  auto turns = [&](const LaunchCfg& c) {
+    const int64_t at_once = (int64_t)c.blocks * c.W * (32 / c.G);
+    return (count + at_once - 1) / at_once;
+  };
+  if (turns(*cfg) >= 2 * turns(fp64)) *cfg = fp64;
+  return VECCHIA_OK;
 }
 
 void launch_lik(const LaunchCfg& cfg, bool grad, const LikArgs& a, cudaStream_t stream) {
-  lik_kernel(a.m + 1, grad, cfg.G, a.metric == 1)<<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
+  lik_kernel(grad, cfg.G, a.metric == 1, cfg.fixed)<<<cfg.blocks, cfg.W * 32, cfg.smem, stream>>>(a);
 }
 }  // namespace
 
@@ -463,11 +482,19 @@ namespace {
 LaunchCfg fit_to_work(LaunchCfg c, int K, bool grad, bool sphere, int64_t count) {
   const int NL = 32 / c.G;
   const int64_t groups = (count + NL - 1) / NL;
-  if (c.sms <= 0 || groups >= (int64_t)c.blocks * c.W) return c;
-  const int W = (int)std::max<int64_t>(1, std::min<int64_t>(c.W, (groups + c.sms - 1) / c.sms));
-  c.W = W;
-  c.blocks = (int)((groups + W - 1) / W);
-  c.smem = SmemLayout(K, grad, c.G, sphere, c.regather).bytes(W);
+  if (c.sms <= 0) return c;
+  if (c.fixed && c.blocks > c.sms) {
+    // Two or more CTAs an SM: as many warps as the turns they take anyway need, the same on each SM.
+    const int64_t turns = (groups + (int64_t)c.blocks * c.W - 1) / ((int64_t)c.blocks * c.W), per = c.blocks / c.sms;
+    const int64_t each = (groups + turns * c.sms - 1) / (turns * c.sms), ctas = std::min(per, (each + c.W - 1) / c.W);
+    c.W = (int)std::max<int64_t>(1, (each + ctas - 1) / ctas);
+    c.blocks = (int)std::min<int64_t>(ctas * c.sms, (groups + c.W - 1) / c.W);
+  } else {
+    if (groups >= (int64_t)c.blocks * c.W) return c;
+    c.W = (int)std::max<int64_t>(1, std::min<int64_t>(c.W, (groups + c.sms - 1) / c.sms));
+    c.blocks = (int)((groups + c.W - 1) / c.W);
+  }
+  c.smem = SmemLayout(K, grad, c.G, sphere, c.regather).bytes(c.W);
   return c;
 }
 

@@ -113,8 +113,8 @@ __device__ __forceinline__ void run_item(const FieldDesc& fd, int64_t tile, cons
   write_partial<G>(acc, out, lane);
 }
 
-template <bool GRAD, int G, bool FIXED>
-__global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : (FIXED ? 512 : 32 * kMaxCtaWarps))
+template <bool GRAD, int G, int FIXED>
+__global__ void __launch_bounds__(lik_threads(GRAD, G, FIXED))
     vecchia_batched_kernel(const BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   for (int k = 0; k < a.nk; ++k)
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : (FIXED ? 512 : 3
     const MaternConst mc = matern_const_at(fix_const(tab));
     ThetaConst tc;
     tc.set(s2, beta, t2, kFamilyMatern, nu);
-    run_item<GRAD, G, FIXED>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
+    run_item<GRAD, G, FIXED != 0>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
     __syncwarp();
   }
 }
@@ -228,17 +228,20 @@ struct PreparedNu {
 using BatchKernel = void (*)(const BatchArgs);
 
 template <bool GRAD>
-BatchKernel batch_kernel(int lanes, bool fixed) {
-  if (lanes == 4) return vecchia_batched_kernel<GRAD, 4, false>;
-  if (lanes == 8) return vecchia_batched_kernel<GRAD, 8, false>;
-  if (lanes == 16) return vecchia_batched_kernel<GRAD, 16, false>;
-  return fixed ? vecchia_batched_kernel<GRAD, 32, true> : vecchia_batched_kernel<GRAD, 32, false>;
+BatchKernel batch_kernel(int lanes, int fixed) {
+  if (lanes == 4) return vecchia_batched_kernel<GRAD, 4, 0>;
+  if (lanes == 8) return vecchia_batched_kernel<GRAD, 8, 0>;
+  if (lanes == 16) return vecchia_batched_kernel<GRAD, 16, 0>;
+  if (fixed == 0) return vecchia_batched_kernel<GRAD, 32, 0>;
+  if constexpr (!GRAD)
+    if (fixed == 2) return vecchia_batched_kernel<GRAD, 32, 2>;
+  return vecchia_batched_kernel<GRAD, 32, 1>;
 }
 
 struct BatchClass {
   BatchArgs args{};
   BatchKernel kern = nullptr;
-  int W = 0, blocks = 0, smem = 0;
+  int W = 0, per_sm = 0, blocks = 0, smem = 0;
 };
 
 struct BatchState {
@@ -273,7 +276,7 @@ PreparedNu* prepared_for(int dev) {
 // The class's warps per CTA with the most resident warps per SM (at most 16) and a grid of
 // one wave, with the coordinates gathered twice where that gives a fifth more warps (as in
 // the single-field launch).
-int class_shape(BatchClass* c, const int* areas, int fixed_bytes) {
+int class_shape(BatchClass* c, const int* areas, int fixed_bytes, bool fixed) {
   int dev = 0, sms = 0, optin = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
   VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -289,7 +292,8 @@ int class_shape(BatchClass* c, const int* areas, int fixed_bytes) {
       if (areas[r] == 0 || bytes > optin - (int)fa.sharedSizeBytes || 32 * w > fa.maxThreadsPerBlock) continue;
       int per_sm = 0;
       VECCHIA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, c->kern, w * 32, bytes));
-      const int warps = std::min(per_sm * w, 16);
+      int warps = std::min(per_sm * w, 16);
+      if (fixed && warps > 1 && warps % 4 == 1) warps -= 2;  // as in the single-field launch
       if (per_sm > 0 && warps > best[r]) {
         best[r] = warps;
         W[r] = w;
@@ -299,6 +303,7 @@ int class_shape(BatchClass* c, const int* areas, int fixed_bytes) {
   const int r = best[1] > 0 && 5 * best[1] >= 6 * best[0] ? 1 : 0;
   if (best[r] <= 0) return VECCHIA_EINVAL;
   c->W = W[r];
+  c->per_sm = per[r];
   c->blocks = per[r] * sms;
   c->smem = fixed_bytes + W[r] * areas[r] * 8;
   c->args.regather = r == 1;
@@ -333,7 +338,7 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
     BatchClass c;
     BatchArgs& a = c.args;
     const int k0 = key(order[s]), L = lanes(order[s]);
-    c.kern = grad ? batch_kernel<true>(L, k0 & 1) : batch_kernel<false>(L, k0 & 1);
+    c.kern = grad ? batch_kernel<true>(L, k0 & 1) : batch_kernel<false>(L, 2 * (k0 & 1));
     a.ntheta = ntheta;
     a.first_field = s;
     a.first_item = items;
@@ -369,7 +374,11 @@ int build_batch(const Plan* const* plans, const double* const* ys, int nfields, 
       off += S.pairs_bytes;
     }
     a.area_off = off;
-    const int rc = class_shape(&c, areas, off);
+    int rc = class_shape(&c, areas, off, k0 & 1);
+    if (!rc && !grad && (k0 & 1) && c.W * c.per_sm < 16) {  // not room for 16 warps: the other form
+      c.kern = batch_kernel<false>(L, 1);
+      rc = class_shape(&c, areas, off, true);
+    }
     if (rc) { delete b; return rc; }
     const int64_t share = steps / ((int64_t)kItemsPerWarp * c.blocks * c.W);
     for (int k = a.first_field; k <= a.last_field; ++k) {

@@ -71,6 +71,11 @@ __host__ __device__ constexpr bool fixed_point_block(int K, bool grad, int G) {
   return G == 32 && K >= (grad ? kFixedMinGrad : kFixedMinFwd);
 }
 
+// Most threads of a CTA of the warp kernels (loglik.cu), which bounds their registers.
+__host__ __device__ constexpr int lik_threads(bool grad, int G, int fixed) {
+  return grad ? (G == 8 ? 512 : 384) : fixed == 2 ? 512 : fixed == 1 ? 384 : 32 * kMaxCtaWarps;
+}
+
 // Per-warp shared-memory area for blocks up to size K: the packed triangle A and the
 // block rows' coordinates CX, CY (float pairs; on the sphere a third array CZ follows CY).
 // The elimination's two column buffers TV and TV1 hold the unscaled entries of columns j

@@ -100,11 +100,12 @@ struct SmemLayout {
 // Up to 13 warps per CTA for the forward pass (its two-vector blocks fit thirteen on an
 // SM at m = 60) and 12 for the gradient; the 8-lane gradient kernels are bounded for 16
 // warps per SM (two CTAs of 8, at most 128 registers a thread), which their second-gather
-// layout reaches at m = 25.  The fixed-point kernels (FIXED) with the gradient take 168 registers
-// a thread; without, they are bounded for 16 warps (128 registers), which the blocks up to m = 52 or
-// so leave room for (n = 100k, 12 and 16 warps an SM: m = 45 3.53 and 3.28 ms, m = 50 4.19 and 3.99).
-template <bool GRAD, int G, bool SPHERE, bool FIXED>
-__global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : (FIXED ? 512 : 32 * kMaxCtaWarps))
+// layout reaches at m = 25.  The fixed-point kernels (FIXED = 1) are bounded for 12 warps (168
+// registers a thread); without the gradient there is a form for 16 (FIXED = 2: 128 registers), for the blocks
+// that leave room for them, up to m = 52 or so (n = 100k, 12 and 16 warps an SM: m = 45 3.53 and 3.28 ms, m = 50
+// 4.19 and 3.99; and 12 warps of either form: m = 60 5.65 and 5.70).
+template <bool GRAD, int G, bool SPHERE, int FIXED>
+__global__ void __launch_bounds__(lik_threads(GRAD, G, FIXED))
     vecchia_lik_kernel(const LikArgs a) {
   asm volatile("griddepcontrol.launch_dependents;");  // launch_finalize
   extern __shared__ __align__(16) unsigned char smem[];
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(GRAD ? (G == 8 ? 512 : 384) : (FIXED ? 512 : 3
     const bool active = i < a.i1;
     const int64_t ii = active ? i : base;
     double* trow = terms_mode ? a.terms + ii * (GRAD ? 4 : 1) : nullptr;
-    process_location<GRAD, G, SPHERE, FIXED>(ii, active, F, L.S, sched, pairs, area, a.tab, mc, tc, acc, terms_mode, trow,
+    process_location<GRAD, G, SPHERE, FIXED != 0>(ii, active, F, L.S, sched, pairs, area, a.tab, mc, tc, acc, terms_mode, trow,
                               a.errloc, sub);
   }
   // The CTA's warps' sums are combined in warp order (compensated), one record per CTA.
@@ -224,21 +225,24 @@ namespace {
 struct LaunchCfg {
   int G = 32, W = 4, blocks = 0, smem = 0;
   bool regather = false;  // gradient, 8 lanes: coordinates gathered twice, two vectors per block
-  bool fixed = false;     // eliminated in fixed point
+  int fixed = 0;          // eliminated in fixed point: the kernel's FIXED
   int sms = 0;            // SMs of the device
 };
 
 using LikKernel = void (*)(const LikArgs);
 
 template <bool GRAD, bool SPHERE>
-LikKernel kernel_ptr(int G, bool fixed) {
-  if (G == 4) return vecchia_lik_kernel<GRAD, 4, SPHERE, false>;
-  if (G == 8) return vecchia_lik_kernel<GRAD, 8, SPHERE, false>;
-  if (G == 16) return vecchia_lik_kernel<GRAD, 16, SPHERE, false>;
-  return fixed ? vecchia_lik_kernel<GRAD, 32, SPHERE, true> : vecchia_lik_kernel<GRAD, 32, SPHERE, false>;
+LikKernel kernel_ptr(int G, int fixed) {
+  if (G == 4) return vecchia_lik_kernel<GRAD, 4, SPHERE, 0>;
+  if (G == 8) return vecchia_lik_kernel<GRAD, 8, SPHERE, 0>;
+  if (G == 16) return vecchia_lik_kernel<GRAD, 16, SPHERE, 0>;
+  if (fixed == 0) return vecchia_lik_kernel<GRAD, 32, SPHERE, 0>;
+  if constexpr (!GRAD)
+    if (fixed == 2) return vecchia_lik_kernel<GRAD, 32, SPHERE, 2>;
+  return vecchia_lik_kernel<GRAD, 32, SPHERE, 1>;
 }
 
-LikKernel lik_kernel(bool grad, int G, bool sphere, bool fixed) {
+LikKernel lik_kernel(bool grad, int G, bool sphere, int fixed) {
   if (grad) return sphere ? kernel_ptr<true, true>(G, fixed) : kernel_ptr<true, false>(G, fixed);
   return sphere ? kernel_ptr<false, true>(G, fixed) : kernel_ptr<false, false>(G, fixed);
 }
@@ -324,14 +328,14 @@ int set_smem_limit(int dev, void* kern, int bytes) {
 
 int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere = false, bool want_fixed = true) {
   if (K > max_k_for_lanes(G)) return VECCHIA_EINVAL;  // narrow groups hold small blocks only
-  const bool fixed = want_fixed && fixed_point_block(K, grad, G);
+  int fixed = want_fixed && fixed_point_block(K, grad, G) ? (grad ? 1 : 2) : 0;
   int dev = 0, sms = 0, smem_optin = 0;
   VECCHIA_CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(g_shape_mu);
-  void* kern = reinterpret_cast<void*>(lik_kernel(grad, G, sphere, fixed));
   for (const ShapeEntry& e : g_shapes)
     if (e.dev == dev && e.K == K && e.grad == (int)grad && e.G == G && e.W == forced_W && e.sphere == (int)sphere &&
-        e.cfg.fixed == fixed) {
+        (e.cfg.fixed != 0) == (fixed != 0)) {
+      void* kern = reinterpret_cast<void*>(lik_kernel(grad, G, sphere, e.cfg.fixed));
       const int rc = set_smem_limit(dev, kern, e.cfg.smem);
       if (rc) return rc;
       *cfg = e.cfg;
@@ -339,6 +343,7 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
     }
   VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   VECCHIA_CUDA_TRY(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  void* kern = reinterpret_cast<void*>(lik_kernel(grad, G, sphere, fixed));
   cudaFuncAttributes fa;
   VECCHIA_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));  // the forward kernel takes up to 13 warps
   // most resident warps per SM (capped at 16 by the registers) for one layout, or -1
@@ -371,7 +376,13 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
     return best_warps;
   };
   LaunchCfg sep, rg;
-  const int ws = best_for(false, &sep);
+  int ws = best_for(false, &sep);
+  if (fixed == 2 && ws < 16 && ws != -2) {  // not room for 16 warps: the other form
+    fixed = 1;
+    kern = reinterpret_cast<void*>(lik_kernel(grad, G, sphere, fixed));
+    VECCHIA_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
+    ws = best_for(false, &sep);
+  }
   const int wr = regather_capable(grad, G) ? best_for(true, &rg) : -1;
   if (ws == -2 || wr == -2) return VECCHIA_ECUDA;
   if (ws <= 0 && wr <= 0) return VECCHIA_EINVAL;

@@ -72,7 +72,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // panel's columns and, once warp 0's sixteen rows are in (barrier 1), update them.  The data are the other
 // warps' work too, a panel behind: warp 1 solves for the first panel's z (barrier 2), each row's datum goes
 // with the row, and warp 1 takes the sixteen rows' from their digits.  (On warp 0, in the panels' columns:
-// n = 20k, m = 120 with the gradient 11.2 ms, m = 130 without 12.3; SOLVE_MS so.)
+// n = 20k, m = 130 16.0 ms with the gradient and 12.3 without; so 15.0 and 11.6.)
 template <bool GRAD>
 __device__ __forceinline__ bool cta_eliminate(int K, long long* __restrict__ A, float2* __restrict__ RJ, int4* __restrict__ piv,
                                               double* __restrict__ zs, int f, long long* corner, int tid, int NTH) {
@@ -323,9 +323,9 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
     bool exact = f > kMostShift || __reduce_add_sync(0xffffffffu, count) < 0;  // the block goes to cta_fp64_block
     if (GRAD) {
       unsigned near = __float_as_uint(INFINITY);  // u of the nearest neighbour
-      for (int p = lane; p < mi; p += 32) near = min(near, __float_as_uint(sq_offset<SPHERE>(CX, CY, CZ, p)));
+      for (int p = lane; p < mi; p += 32) near = min(near, __float_as_uint(near_u<SPHERE>(F, CX, CY, CZ, p)));
       near = __reduce_min_sync(0xffffffffu, near);
-      exact = exact || rho_below(scaled_offset<SPHERE>(F, __uint_as_float(near)), kWeakBits, a.tab, mc);
+      exact = exact || rho_below(__uint_as_float(near), kWeakBits, a.tab, mc);
     }
     // ---- assemble, in fixed point (mmapanel.cuh)
     for (int c = tid; c < K; c += NTH) {

@@ -357,23 +357,14 @@ __device__ __forceinline__ void pair_u(const FieldView& F, const float2* __restr
   }
 }
 
-// The squared distance (plane: u itself) of row p from the block's own location, which is at 0, in FP32, and u
-// from it.
+// u of row p and the block's own location, which is at 0, in FP32 (on the sphere by the chord, which is the
+// arc's 2/pi at least).
 template <bool SPHERE>
-__device__ __forceinline__ float sq_offset(const float2* __restrict__ CX, const float2* __restrict__ CY,
-                                           const float2* __restrict__ CZ, int p) {
-  const float z = SPHERE ? CZ[p].x : 0.0f;
-  return fmaf(CX[p].x, CX[p].x, fmaf(CY[p].x, CY[p].x, z * z));
-}
-template <bool SPHERE>
-__device__ __forceinline__ float scaled_offset(const FieldView& F, float d2) {
-  if constexpr (SPHERE) {
-    float uh, ul;
-    sphere_u_df(fminf(d2, 4.0f), 0.0f, F, uh, ul);
-    return uh;
-  } else {
-    return d2;
-  }
+__device__ __forceinline__ float near_u(const FieldView& F, const float2* __restrict__ CX, const float2* __restrict__ CY,
+                                        const float2* __restrict__ CZ, int p) {
+  const float d2 = fmaf(CX[p].x, CX[p].x, CY[p].x * CY[p].x);
+  if constexpr (SPHERE) return 0.25f * F.k2.x * fmaf(CZ[p].x, CZ[p].x, d2);
+  else return d2;
 }
 
 // (pbh, pbl) += h (w_r g_c + w_c g_r) in double-float arithmetic.
@@ -760,10 +751,10 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
 #pragma unroll
       for (int s = 0; s < NSG; ++s) {
         const int p = sub + 32 * s;
-        if (p < mi) near = min(near, __float_as_uint(sq_offset<SPHERE>(CX, CY, CZ, p)));
+        if (p < mi) near = min(near, __float_as_uint(near_u<SPHERE>(F, CX, CY, CZ, p)));
       }
       near = __reduce_min_sync(0xffffffffu, near);
-      exact = exact || rho_below(scaled_offset<SPHERE>(F, __uint_as_float(near)), kWeakBits, tab, mc);
+      exact = exact || rho_below(__uint_as_float(near), kWeakBits, tab, mc);
     }
   }
   if (check) {  // a bad index anywhere in the group fails the group's block

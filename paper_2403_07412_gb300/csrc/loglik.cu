@@ -378,6 +378,8 @@ int shape_for(int K, bool grad, int G, int forced_W, LaunchCfg* cfg, bool sphere
   LaunchCfg sep, rg;
   int ws = best_for(false, &sep);
   if (fixed == 2 && ws < 16 && ws != -2) {  // not room for 16 warps: the other form
+    for (SmemLimit& l : g_smem_limits)
+      if (l.dev == dev && l.kern == kern) l.bytes = -1;  // the search left another limit on this one
     fixed = 1;
     kern = reinterpret_cast<void*>(lik_kernel(grad, G, sphere, fixed));
     VECCHIA_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
       unsigned near = __float_as_uint(INFINITY);  // u of the nearest neighbour
       for (int p = lane; p < mi; p += 32) near = min(near, __float_as_uint(near_u<SPHERE>(F, CX, CY, CZ, p)));
       near = __reduce_min_sync(0xffffffffu, near);
-      exact = exact || rho_below(__uint_as_float(near), kWeakBits, a.tab, mc);
+      exact = exact || rho_below(__uint_as_float(near), kWeakGradient, a.tab, mc);
     }
     // ---- assemble, in fixed point (mmapanel.cuh)
     for (int c = tid; c < K; c += NTH) {

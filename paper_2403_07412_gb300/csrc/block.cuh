@@ -754,7 +754,7 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
         if (p < mi) near = min(near, __float_as_uint(near_u<SPHERE>(F, CX, CY, CZ, p)));
       }
       near = __reduce_min_sync(0xffffffffu, near);
-      exact = exact || rho_below(__uint_as_float(near), kWeakBits, tab, mc);
+      exact = exact || rho_below(__uint_as_float(near), GRAD ? kWeakGradient : kWeakPrediction, tab, mc);
     }
   }
   if (check) {  // a bad index anywhere in the group fails the group's block

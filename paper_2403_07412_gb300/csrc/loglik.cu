@@ -460,8 +460,7 @@ int pick_config(int K, bool grad, LaunchCfg* cfg, bool sphere = false, int64_t c
   // 275 and 239 (3 turns and 2), 7,500 275 for 310.
   if (!grad && (K < 39 || K > 42)) return VECCHIA_OK;
   LaunchCfg fp64;
-  rc = shape_for(K, grad, grad ? G : 16, W, &fp64, sphere, false);
-  if (rc) return rc;
+  if (shape_for(K, grad, grad ? G : 16, W, &fp64, sphere, false)) return VECCHIA_OK;  // (a forced W it cannot take)
   auto turns = [&](const LaunchCfg& c) {
     const int64_t at_once = (int64_t)c.blocks * c.W * (32 / c.G);
     return (count + at_once - 1) / at_once;

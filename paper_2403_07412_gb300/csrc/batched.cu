@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(lik_threads(GRAD, G, FIXED))
     const MaternConst mc = matern_const_at(fix_const(tab));
     ThetaConst tc;
     tc.set(s2, beta, t2, kFamilyMatern, nu);
+    if (FIXED) tc.weak_u = (float)fix_const(tab)[GRAD ? kConstWeakGradient : kConstWeakPrediction];
     run_item<GRAD, G, FIXED != 0>(fd, tile, smem, a, base, tab, mc, tc, out, lane);
     __syncwarp();
   }

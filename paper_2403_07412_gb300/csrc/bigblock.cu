@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
   const MaternConst mc = matern_const_at(fix_const(a.tab));
   ThetaConst tc;
   tc.set(a.sigma2, a.beta, a.tau2, a.family, a.nu);
+  tc.weak_u = (float)fix_const(a.tab)[kConstWeakGradient];
   const int f = panel_shift(tc.gamma1);
   const double2* __restrict__ xy2 = reinterpret_cast<const double2*>(a.xy);
   FieldView F;  // the distance fields pair_u reads
@@ -322,10 +323,10 @@ __global__ void __launch_bounds__(kCtaThreadsMax) vecchia_big_kernel(const BigAr
     }
     bool exact = f > kMostShift || __reduce_add_sync(0xffffffffu, count) < 0;  // the block goes to cta_fp64_block
     if (GRAD) {
-      unsigned near = __float_as_uint(INFINITY);  // u of the nearest neighbour
+      unsigned near = 0x7F800000u;  // u of the nearest neighbour
       for (int p = lane; p < mi; p += 32) near = min(near, __float_as_uint(near_u<SPHERE>(F, CX, CY, CZ, p)));
       near = __reduce_min_sync(0xffffffffu, near);
-      exact = exact || rho_below(__uint_as_float(near), kWeakGradient, a.tab, mc);
+      exact = exact || (__uint_as_float(near) >= tc.weak_u && mi > 0);
     }
     // ---- assemble, in fixed point (mmapanel.cuh)
     for (int c = tid; c < K; c += NTH) {

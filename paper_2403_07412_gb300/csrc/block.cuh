@@ -157,6 +157,7 @@ __device__ __forceinline__ void build_schedules(int K, uint16_t* sched, uint32_t
 // -2 sigma2 / beta (Matérn) or -2 sigma2 / (alpha beta) (power exponential).
 struct ThetaConst {
   double sigma2, inv_len, gamma1, inv_sigma2, tau2, dbeta_coef;
+  float weak_u = INFINITY;  // fixed-point sizes: from this u of the nearest neighbour on, FP64
   __device__ void set(double s2, double beta, double t2, int family, double nu) {
     sigma2 = s2;
     const bool pe = family == kFamilyPowExp;
@@ -747,14 +748,14 @@ __device__ __forceinline__ bool process_location(int64_t i, bool active, const F
                __popc(__ballot_sync(0xffffffffu, large[s] > 0));
     exact = exact || count < 0;
     if (GRAD || F.pmean) {
-      unsigned near = __float_as_uint(INFINITY);  // u of the nearest neighbour
+      unsigned near = 0x7F800000u;  // u of the nearest neighbour
 #pragma unroll
       for (int s = 0; s < NSG; ++s) {
         const int p = sub + 32 * s;
         if (p < mi) near = min(near, __float_as_uint(near_u<SPHERE>(F, CX, CY, CZ, p)));
       }
       near = __reduce_min_sync(0xffffffffu, near);
-      exact = exact || rho_below(__uint_as_float(near), GRAD ? kWeakGradient : kWeakPrediction, tab, mc);
+      exact = exact || (__uint_as_float(near) >= tc.weak_u && mi > 0);
     }
   }
   if (check) {  // a bad index anywhere in the group fails the group's block

@@ -28,6 +28,11 @@ namespace vecchia {
 __host__ __device__ __forceinline__ double* fix_const(double* tab) { return tab + 2 * kFixWords * kFixInt; }
 __device__ __forceinline__ const double* fix_const(const double* tab) { return tab + 2 * kFixWords * kFixInt; }
 
+// After the small-u constants: the least u, by intervals, from which on rho is below 2^-kWeakPrediction and
+// 2^-kWeakGradient (E two and six; to within a factor of two).
+constexpr int kWeakPrediction = 8, kWeakGradient = 12;
+constexpr int kConstWeakPrediction = 6, kConstWeakGradient = 7;
+
 // s + e = a + b exactly for |a| >= |b| (or a = 0).
 __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
@@ -128,16 +133,6 @@ __device__ __forceinline__ void rho_fixed62(float u0h, float u0l, float u1h, flo
     if (fix_outside(u0h)) r0 = rho_outside62_call(u0h, u0l, mc.kind, mc.nu, mc.a1, mc.G, mc.b0, mc.b1);
     if (fix_outside(u1h)) r1 = rho_outside62_call(u1h, u1l, mc.kind, mc.nu, mc.a1, mc.G, mc.b0, mc.b1);
   }
-}
-
-// Whether rho(u) is below 2^-bits, bits >= 7 (by the interval's E, so to within a factor of two).
-__device__ __forceinline__ bool rho_below(float u, int bits, const double* __restrict__ tab, const MaternConst& mc) {
-  if (fix_outside(u)) {
-    const FixRho r = rho_outside62_call(u, 0.0f, mc.kind, mc.nu, mc.a1, mc.G, mc.b0, mc.b1);
-    return r.v >> min((r.sh >> 20) - bits, 63) == 0;
-  }
-  const float4* __restrict__ w = reinterpret_cast<const float4*>(tab) + fix_arg(u, 0.0f).idx * kFixWords;
-  return (__float_as_int(__ldg(reinterpret_cast<const float*>(w + 2) + 3)) >> 20) - 62 >= bits - 6;
 }
 
 // In FP64: one conversion, and the power of two on the exponent field.  (A conversion holds the FP64 pipe

@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(lik_threads(GRAD, G, FIXED))
   const MaternConst mc = matern_const_at(fix_const(a.tab));
   ThetaConst tc;
   tc.set(a.sigma2, a.beta, a.tau2, a.family, a.nu);
+  if (FIXED) tc.weak_u = (float)fix_const(a.tab)[GRAD ? kConstWeakGradient : kConstWeakPrediction];
   FieldView F;
   F.xy = reinterpret_cast<const double2*>(a.xy);
   F.yf = a.yf;

@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <mutex>
 #include <vector>
 
@@ -202,6 +203,7 @@ struct FixSetup {
     stirling = 0.0f;
     for (double& v : c) v = 0.0;
     c[1] = nu;
+    c[kConstWeakPrediction] = c[kConstWeakGradient] = std::numeric_limits<double>::infinity();
     const bool integer = nu == std::floor(nu);
     const long long kind = family == kFamilyPowExp ? 3 : integer ? (nu == 1.0 ? 1 : 2) : 0;
     std::memcpy(&c[0], &kind, sizeof(kind));
@@ -351,13 +353,14 @@ constexpr int kFixMostE = 960;  // (62 + E) 2^20 is subtracted from an exponent 
 
 __global__ void __launch_bounds__(kFixThreads) fix_table_kernel(const FixSetup s, double* tab) {
   __shared__ unsigned long long ea[kFixChunk][kFixGroup], eb[kFixChunk][8], part[4][64];
-  __shared__ int scale[kFixGroup];  // E
+  __shared__ int scale[kFixGroup + 1];  // E; the last one the interval's before the group
   const int tid = threadIdx.x;
   const int e = kELo + (blockIdx.x * kFixGroup >> kFixSub);
   const int j0 = blockIdx.x * kFixGroup & ((1 << kFixSub) - 1);
   const float nu = (float)s.nu;
-  if (tid < kFixGroup) {
-    const float u = ldexpf((float)(32 + j0 + tid), e - kFixSub);
+  if (tid <= kFixGroup) {
+    const float u = tid < kFixGroup ? ldexpf((float)(32 + j0 + tid), e - kFixSub)
+                                    : j0 > 0 ? ldexpf((float)(31 + j0), e - kFixSub) : ldexpf(63.0f, e - 1 - kFixSub);
     float bits;  // -log2 rho
     if (s.family == kFamilyPowExp) {
       bits = 1.442695041f * expf(0.5f * nu * logf(u));
@@ -368,6 +371,12 @@ __global__ void __launch_bounds__(kFixThreads) fix_table_kernel(const FixSetup s
     scale[tid] = (int)fminf(fmaxf(floorf(bits) - 6.0f, 0.0f), (float)kFixMostE);
   }
   __syncthreads();
+  if (tid < kFixGroup) {
+    const int E = scale[tid], before = tid ? scale[tid - 1] : scale[kFixGroup];
+    const double u = ldexp((double)(32 + j0 + tid), e - kFixSub);
+    if (E >= kWeakPrediction - 6 && before < kWeakPrediction - 6) fix_const(tab)[kConstWeakPrediction] = u;
+    if (E >= kWeakGradient - 6 && before < kWeakGradient - 6) fix_const(tab)[kConstWeakGradient] = u;
+  }
   if (s.family == kFamilyPowExp) {
     if (tid < 64) {
       const double t = (double)kFixInterp.t[tid & 7] * 0x1p-64;

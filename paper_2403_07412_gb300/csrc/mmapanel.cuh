@@ -66,12 +66,12 @@ constexpr long long kSmallestPivot = 128;
 //  - where a few data tower over the others, whose small weights' errors they multiply: fewer than half
 //    of the block's data (zeros left aside) within 2^6 (by exponent) of the largest.  Of 61 normal variates 58 are;
 //  - where the location is barely correlated with any neighbour and what is wanted is as small: a prediction
-//    (rho < 2^-8), or derivatives (rho < 2^-12: they are double-float, to 2^-46);
+//    (rho < 2^-8), or derivatives (rho < 2^-12: they are double-float, to 2^-46).  The nearest neighbour's u
+//    says so (looked up in the table at every location: n = 50k on the sphere, m = 60 5.26 -> 5.52 ms);
 //  - where the nugget is 2^16 times the variance or more (f >= 8).
 // They cost what FP64 costs (n = 100k, m = 60, value and with the gradient, ms: every block 8.97 and 11.1; one
 // datum in 60 a million times larger 7.81 and 11.3; none 5.83 and 8.54).
 constexpr int kEvenBits = 6;
-constexpr int kWeakPrediction = 8, kWeakGradient = 12;
 constexpr int kMostShift = 7;
 constexpr float kAccZero = 12582912.0f;  // 1.5 2^23
 constexpr unsigned kAccZeroBits = 0x4B400000u;

@@ -306,6 +306,13 @@ __device__ __forceinline__ void sq_chord_df(float2 xr, float2 xc, float2 yr, flo
   cl = __fsub_rn(e, __fsub_rn(ch, s2));
 }
 
+// u = K2 asin^2(c / 2) at chords above 1/16 of the radius, w = c^2 / 4.  (A function: in line at every use it lengthened the gradient kernels; n = 50k, m = 60 5.50 -> 5.25
+// ms.)
+static __device__ __noinline__ float2 sphere_far_u(float wh, float wl, double k2d) {
+  const double a = asin(sqrt(f2d_scaled(wh, 0) + f2d_scaled(wl, 0)));
+  return d2f_pair(k2d * a * a);
+}
+
 // u = K2 asin^2(c / 2) from the squared chord c^2 = ch + cl of two unit vectors: the
 // great-circle distance d = 2 r asin(c / 2) (Sec. VI-C), over the length scale, squared.
 // With w = c^2 / 4, asin^2(sqrt(w)) = w + w^2 T(w), T(w) = 1/3 + 8w/45 + 4w^2/35 +
@@ -315,8 +322,7 @@ __device__ __forceinline__ void sq_chord_df(float2 xr, float2 xc, float2 yr, flo
 __device__ __forceinline__ void sphere_u_df(float ch, float cl, const FieldView& F, float& uh, float& ul) {
   const float wh = ch * 0.25f, wl = cl * 0.25f;
   if (wh > 0x1p-10f) {
-    const double a = asin(sqrt(f2d_scaled(wh, 0) + f2d_scaled(wl, 0)));
-    const float2 u = d2f_pair(F.k2d * a * a);
+    const float2 u = sphere_far_u(wh, wl, F.k2d);
     uh = u.x;
     ul = u.y;
     return;

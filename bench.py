@@ -743,7 +743,10 @@ def main():
                      "flops_count": "F(k) = k^3/3 + k^2/2 + k/6 + k^2 per location, k = m_i + 1 "
                                     "(Cholesky and two triangular solves)",
                      "frac_with_adjoint_solves": (flops_adj / (kern_ms * 1e-3) / 1e12) / peak,
-                     "peak_source": "FP64 DFMA-chain kernel measured in this run (vecchia_fp64_peak)"},
+                     "peak_source": "FP64 DFMA-chain kernel measured in this run (vecchia_fp64_peak)",
+                     "note": "frac compares the algorithm's FP64 operation count with the FP64 pipe's peak; blocks of 38 "
+                             "rows and more (51 with the gradient) do most of it in fixed point on the integer and tensor "
+                             "pipes (FP64 pipe 24 to 31% busy at m = 60), so frac is not that pipe's use and can exceed 1"},
         "covariance": {"entries_per_call": cov_evals, "entries_per_s": cov_evals / (kern_ms * 1e-3),
                        "note": "off-diagonal covariance entries k(k-1)/2 per location, k = m_i + 1"},
         "hbm": {"gbs": hbm_gbs, "source": "ncu dram bytes per launch (profiles/traffic.json) / CUDA-event time"},

@@ -196,8 +196,8 @@ int vecchia_loglik_range(vecchia_plan_t plan, const double* y_dev, const double 
                          int want_grad, double* out_dev, void* stream);
 
 /*
- * vecchia_matern — the covariance of Eq. (2) and its beta-derivative, evaluated by the
- * same device code the likelihood kernels use.
+ * vecchia_matern — the covariance of Eq. (2) and its beta-derivative, from a piecewise polynomial
+ * table of its own (the likelihood kernels read another one, which is at least as close).
  *   d_dev        : count distances (>= 0) on the device.
  *   c_dev        : count doubles on the device: C(d) (sigma2 at d = 0, without nugget).
  *   dcdbeta_dev  : count doubles on the device (may be NULL): dC/dbeta(d).
@@ -208,7 +208,7 @@ int vecchia_matern(const double* d_dev, int64_t count, const double theta[4], do
 
 /*
  * vecchia_covariance — vecchia_matern for either covariance family (VECCHIA_KERNEL_*):
- * C(d) of Eq. (2) or Eq. (3) and dC/dbeta, through the kernels' device code.  Same
+ * C(d) of Eq. (2) or Eq. (3) and dC/dbeta.  Same
  * arguments and errors as vecchia_matern, plus EINVAL for an unknown kernel or, for the
  * power exponential, an exponent outside (0, 2].
  */
@@ -256,7 +256,8 @@ int vecchia_mul_by_positive(const double* a_dev, const double* b_dev, int64_t co
 int vecchia_batched_prepare(const double* nus, int32_t nnu, void* stream);
 
 /*
- * vecchia_loglik_batched — many (field, theta) evaluations in one persistent launch (not
+ * vecchia_loglik_batched — many (field, theta) evaluations in one call, one persistent launch for
+ * each class of fields whose blocks run the same way, at most four (not
  * in the paper, which batches only over the locations of one field).
  *   plans      : nfields plan handles (host array); fields may differ in n and m (at most
  *                four distinct m per call, each m <= VECCHIA_MAX_M_WARP).
@@ -270,7 +271,8 @@ int vecchia_batched_prepare(const double* nus, int32_t nnu, void* stream);
  *   out_dev    : nfields x ntheta x (1|4) doubles on the device.
  * Asynchronous on `stream`.  The first call for a given (plans, y_devs, ntheta, want_grad)
  * lays out the work and allocates for it (it must not be made during stream capture:
- * EINVAL); later calls with the same arguments reuse that layout, allocate nothing and
+ * EINVAL): 80 bytes a field, and a 32-byte record for each item of work, some 64 items for each warp
+ * resident at once (5 MB a class at most) and one at least for each (field, theta); later calls with the same arguments reuse that layout, allocate nothing and
  * may be captured in a CUDA graph and replayed with new values in thetas_dev.  A theta
  * whose nu was not prepared, an invalid theta or a block that is not positive definite
  * makes that (field, theta)'s outputs NaN.  Destroying a plan drops the layouts that use
@@ -330,10 +332,14 @@ int vecchia_loglik_noalloc(const double* xy_dev, const double* y_dev, const int3
  * including the batched call's layouts created afterwards.  Without tuning, blocks of
  * up to 16 rows use 4 lanes, up to 29 rows 8 and up to 37 rows 16 (gradient: up to 26 and
  * 35 rows), larger ones a full warp; a call over fewer locations than would give
- * one group of them per SM sub-partition widens those defaults (up to 16 lanes), and
+ * one group of them per SM sub-partition widens those defaults (up to 16 lanes for blocks
+ * of up to 16 rows, else to a full warp) or, where they then fit in one turn of the resident
+ * warps, narrows them again, and
  * a call with fewer groups than the shape's resident warps spreads them over every SM
  * with fewer warps per CTA.  Results are deterministic for a given plan, range and
- * shape; a different shape changes only the order of the final additions.
+ * shape.  A different shape changes the order of the final additions and, for blocks of 38
+ * rows and more (gradient: 51), with the lanes per location also whether a block is eliminated in
+ * fixed point (a full warp) or in FP64: terms then agree to rounding, not bit for bit.
  * Not in the paper (its batched kernels are library routines).
  *   y_dev, theta : as for vecchia_loglik (theta on the host).
  *   lanes_out, warps_out : host int32 (may be NULL): the chosen shape.  For m >

@@ -47,10 +47,9 @@ constexpr int kMaxCtaWarps = 13;
 __host__ __device__ constexpr int max_k_for_lanes(int G) { return G == 4 ? 16 : (G == 8 ? 32 : kMaxMWarp + 1); }
 
 // Smallest full-warp blocks (rows) eliminated in fixed point (mmapanel.cuh) instead of FP64.
-// n = 100k, FP64 / fixed point, ms: forward m = 34 2.19 / 2.33, m = 38 2.79 / 2.55, m = 60 8.75 /
-// 5.39; with the gradient m = 42 4.16 / 4.69, m = 46 5.04 / 5.11, m = 50 6.20 / 6.03, m = 60 11.1 /
-// 8.32 (its adjoint reads the factor from digits; at m = 48 the two are even, and FP64 ahead by 3%
-// in the smallest calls).
+// n = 100k, FP64 / fixed point, ms: forward m = 34 2.19 / 2.33, m = 38 2.79 / 2.60, m = 60 8.70 /
+// 5.71; with the gradient m = 42 4.16 / 4.69, m = 46 5.04 / 5.11, m = 50 6.27 / 6.16, m = 60 11.0 /
+// 8.55 (its adjoint reads the factor from digits; at m = 48 the two are even).
 constexpr int kFixedMinFwd = 38;
 constexpr int kFixedMinGrad = 51;
 

@@ -795,7 +795,7 @@ __global__ void pivot_reciprocal_kernel(const double* __restrict__ d, int64_t co
   }
 }
 
-// The column-scaling product of the full-warp kernels on its own.
+// The column-scaling product of the 4-lane forward kernel on its own.
 __global__ void mul_by_positive_kernel(const double* __restrict__ a, const double* __restrict__ b, int64_t count,
                                        double* __restrict__ out) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;

@@ -598,7 +598,7 @@ int launch_matern_table(double nu, double* tab, cudaStream_t stream) {
 }
 
 // ------------------------------------------------------------------ vecchia_matern
-// C(d) and dC/dbeta through the kernels' device code.  u = (d * inv_len)^2 with the
+// C(d) and dC/dbeta from the evaluators' table.  u = (d * inv_len)^2 with the
 // family's length scale (beta for the Matérn, beta^(1/alpha) for the power
 // exponential), and dC/dbeta = dcoef h(u), dcoef = -2 sigma2 / (beta a), a = 1 or alpha.
 __global__ void matern_eval_kernel(const double* __restrict__ d, int64_t count, double sigma2,

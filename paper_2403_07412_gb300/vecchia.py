@@ -351,7 +351,7 @@ def vecchia_predict(plan: Plan, xy_new, y, theta, with_var: bool = True, return_
 
 
 def vecchia_covariance(kernel: int, d: torch.Tensor, theta, with_dbeta: bool = True, stream=None):
-    """C(d) (and dC/dbeta) of either covariance family through the kernels' device code."""
+    """C(d) (and dC/dbeta) of either covariance family."""
     d = _dev_f64(d, d.numel(), "d")
     c = torch.empty_like(d)
     dc = torch.empty_like(d) if with_dbeta else None
